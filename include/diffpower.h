@@ -97,13 +97,14 @@ typedef struct {
                                forward and the reverse pass each run in one thread block, with
                                block barriers between levels and the pairs and edge adjoints
                                in shared memory; for a mid-size one (dp_info.cluster_threads >
-                               0) in one cluster of 16 blocks, with the cluster barrier between
-                               levels and the pairs and edge adjoints spread over the blocks'
-                               shared memory; otherwise, and for the simulation, as 2;
+                               0) in one cluster of 16 blocks, with the pairs and edge adjoints
+                               spread over the blocks' shared memory; otherwise over the whole
+                               grid.  The last two have no barrier between levels: each cell
+                               waits for its own inputs.  The simulation as 2;
                             2: one cooperative launch per pass with grid-wide level barriers;
                             1: one launch per level;
-                            3: dataflow forward pass - warps take cells in topological order and
-                               wait only for their own fanins (other passes as 2).
+                            3: the whole grid without barriers for the forward and the reverse
+                               pass of every design, and for the simulation.
                             Where a cooperative grid cannot be co-resident the library uses 1.
                             All give bitwise identical results. */
     uint64_t seed;       /* Philox4x32-10 key for the startpoint Markov chains (Sec. III-C) */

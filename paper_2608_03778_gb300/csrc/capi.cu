@@ -46,6 +46,7 @@ dp_status check_device_error(dp_ctx *c) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_err(c, e, "device error word");
     if (v != 0) {
+        c->timeouts++;
         cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
         cudaStreamSynchronize(c->stream);
         return set_err(c, DP_ETIMEOUT, "a bounded device wait gave up (grid barrier timeout)");
@@ -218,8 +219,20 @@ bool persistent(const dp_design *D, const dp_config &c, int which) {
 bool small_pass(const dp_design *D, const dp_config &c) { return c.schedule == 0 && D->block_threads > 0; }
 // ... and of a mid-size design in one thread-block cluster (schedule 0)
 bool cluster_pass(const dp_design *D, const dp_config &c) { return c.schedule == 0 && D->cl.threads > 0; }
+// the dataflow passes: the forward and the reverse pass of the designs that do not fit the two
+// above (schedule 0), and on request (schedule 3, which has a dataflow simulation too)
 bool dataflow(const dp_design *D, const dp_config &c, int which) {
-    return c.schedule == 3 && D->flow_grid[which] > 0 && D->d.n_levels > 0;
+    return (c.schedule == 3 || (c.schedule == 0 && which != 1)) && D->flow_grid[which] > 0 && D->d.n_levels > 0;
+}
+
+// A pass that timed out may have left nets of two parities behind, which a later dataflow pass
+// could take for its own: back to the state after the upload.
+void repair_tags(dp_design *D, cudaStream_t s) {
+    if (D->timeouts_seen == D->ctx->timeouts) return;
+    D->timeouts_seen = D->ctx->timeouts;
+    cudaMemsetAsync(D->d.pq, 0, sizeof(float4) * (size_t)D->d.n_nets, s);
+    cudaMemsetAsync(D->d.epoch, 0, sizeof(uint32_t), s);
+    cudaMemsetAsync(D->d.epoch + 4, 0, 2 * sizeof(uint32_t), s);
 }
 
 // each q_* returns the first launch error (a cooperative launch reports it directly)
@@ -233,16 +246,16 @@ cudaError_t q_forward(dp_design *D, const dp_config &c, cudaStream_t s, cudaEven
         dp::launch_power(D->d, false, power_K(c), 0, s);
         return cudaGetLastError();
     }
+    if (cluster_pass(D, c) || dataflow(D, c, 0)) {   // these advance it too
+        if (ready) cudaEventRecord(ready, s);
+        cudaError_t e = cluster_pass(D, c) ? dp::launch_fwd_cluster(D->d, D->ops, D->cl, c.tr_mode, s)
+                                           : dp::launch_fwd_flow(D->d, D->ops, c.tr_mode, D->flow_grid[0], s);
+        if (e != cudaSuccess) return e;
+        dp::launch_power(D->d, false, power_K(c), 0, s);
+        return cudaGetLastError();
+    }
     dp::launch_bump(D->d.epoch, s);   // new parity for the stored (P, Q) pairs
-    if (cluster_pass(D, c)) {
-        if (ready) cudaEventRecord(ready, s);
-        cudaError_t e = dp::launch_fwd_cluster(D->d, D->ops, D->cl, c.tr_mode, s);
-        if (e != cudaSuccess) return e;
-    } else if (dataflow(D, c, 0)) {
-        if (ready) cudaEventRecord(ready, s);
-        cudaError_t e = dp::launch_fwd_flow(D->d, D->ops, c.tr_mode, D->flow_grid[0], D->flow_sleep, s);
-        if (e != cudaSuccess) return e;
-    } else if (persistent(D, c, 0)) {
+    if (persistent(D, c, 0)) {
         cudaError_t e = dp::launch_fwd_persist(D->d, D->ops, c.tr_mode, D->grid[0], s, ready);
         if (e != cudaSuccess) return e;
     } else {
@@ -285,14 +298,20 @@ cudaError_t q_hybrid(dp_design *D, const dp_config &c, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// what the cluster's and the dataflow reverse pass need of the forward pass alone
+void q_coef(dp_design *D, const dp_config &c, cudaStream_t s) {
+    if (small_pass(D, c) || !(cluster_pass(D, c) || dataflow(D, c, 2))) return;
+    dp::launch_bwd_coef(D->d, D->ops, c.tr_mode, (float)power_K(c), cluster_pass(D, c) ? D->cl.coef : nullptr, s);
+}
+
 // beside: other kernels run beside this pass (the step's gradient outputs), so its grid-wide
 // form leaves them room on the SMs
 cudaError_t q_backward(dp_design *D, const dp_config &c, float *gsp, cudaStream_t s, bool beside = false) {
     const float K = (float)power_K(c);
     if (small_pass(D, c))
         return dp::launch_bwd_block(D->d, D->ops, c.grad_mode, c.tr_mode, K, gsp, D->n_edges, D->block_threads, s);
-    if (cluster_pass(D, c))
-        return dp::launch_bwd_cluster(D->d, D->ops, D->cl, c.grad_mode, c.tr_mode, K, gsp, s);
+    if (cluster_pass(D, c)) return dp::launch_bwd_cluster(D->d, D->cl, c.grad_mode, gsp, s);   // after q_coef
+    if (dataflow(D, c, 2)) return dp::launch_bwd_flow(D->d, c.grad_mode, gsp, D->flow_grid[2], s);
     if (persistent(D, c, 2))
         return dp::launch_bwd_persist(D->d, D->ops, c.grad_mode, c.tr_mode, K, gsp, D->grid[2], !beside, s);
     for (int l = D->d.n_levels; l >= 1; l--)
@@ -566,12 +585,6 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
     dp_status s = DP_OK;
     uint4 *fanin = nullptr;
     int32_t *fptr = nullptr, *fedge = nullptr, *nou = nullptr, *cou = nullptr, *efpos = nullptr, *lvl = nullptr;
-    int32_t *chunks = nullptr;
-    // level-aligned chunks of 32: level 0 = startpoints, then each level of cells
-    std::vector<int32_t> chunk_ptr((size_t)cp->n_levels + 2, 0);
-    chunk_ptr[1] = (int32_t)((cp->n_start + 31) / 32);
-    for (int l = 1; l <= cp->n_levels; l++)
-        chunk_ptr[l + 1] = chunk_ptr[l] + (cp->lvl_ptr[l] - cp->lvl_ptr[l - 1] + 31) / 32;
     // nets by death level: the highest level of a cell reading the net, else the net's own level
     std::vector<int32_t> dead_ptr((size_t)cp->n_levels + 2, 0), dead_net((size_t)cp->n_nets);
     {
@@ -620,8 +633,9 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
     TRY(dalloc(D, &efpos, 4 * nc));
     TRY(dalloc(D, &lvl, (size_t)cp->n_levels + 1));
     TRY(dalloc(D, &d.bar, dp::persist_bar_words(cp->n_levels)));
-    TRY(dalloc(D, &d.epoch, 4));
-    TRY(dalloc(D, &chunks, chunk_ptr.size()));
+    TRY(dalloc(D, &d.gcell, nc));
+    TRY(dalloc(D, &d.edges, (size_t)cp->n_edges));
+    TRY(dalloc(D, &d.epoch, 8));
     TRY(dalloc(D, &pairs, pair_ptr.size()));
     TRY(dalloc(D, &dptr, dead_ptr.size()));
     TRY(dalloc(D, &dnet, dead_net.size()));
@@ -632,7 +646,6 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
     d.fout_edge = fedge;
     d.edge_fpos = efpos;
     d.lvl = lvl;
-    d.chunk_ptr = chunks;
     d.pair_ptr = pairs;
     d.dead_ptr = dptr;
     d.dead_net = dnet;
@@ -650,7 +663,6 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
     up(fedge, cp->fout_edge.data(), sizeof(int32_t) * cp->fout_edge.size());
     up(efpos, cp->edge_fpos.data(), sizeof(int32_t) * cp->edge_fpos.size());
     up(lvl, cp->lvl_ptr.data(), sizeof(int32_t) * cp->lvl_ptr.size());
-    up(chunks, chunk_ptr.data(), sizeof(int32_t) * chunk_ptr.size());
     up(pairs, pair_ptr.data(), sizeof(int32_t) * pair_ptr.size());
     up(dptr, dead_ptr.data(), sizeof(int32_t) * dead_ptr.size());
     up(dnet, dead_net.data(), sizeof(int32_t) * dead_net.size());
@@ -659,7 +671,8 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
     up(base, cp->base_cap.data(), sizeof(float) * nn);
     up(d.pincap, cp->pincap.data(), sizeof(float) * nc);
     if (e == cudaSuccess) e = cudaMemsetAsync(d.power, 0, 4 * sizeof(double), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.epoch, 0, 4 * sizeof(uint32_t), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d.epoch, 0, 8 * sizeof(uint32_t), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d.gcell, 0, sizeof(unsigned long long) * nc, st);
     // tag 0 everywhere: the first forward pass writes tag 1
     if (e == cudaSuccess) e = cudaMemsetAsync(d.pq, 0, sizeof(float4) * nn, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(d.bar, 0, sizeof(unsigned) * dp::persist_bar_words(cp->n_levels), st);
@@ -709,38 +722,43 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
                 fill[b] += cp->fout_ptr[(size_t)n + 1] - cp->fout_ptr[(size_t)n];
             }
             const int64_t edges = *std::max_element(fill.begin(), fill.end());
-            const size_t sf = dp::cluster_smem(0, slots, 0, L), sb = dp::cluster_smem(1, slots, edges, L);
-            if (sb <= (size_t)dp::kBlockSmemMax && dp::cluster_fits(threads, sf, sb)) {
-                std::vector<int32_t> floc(4 * (size_t)nc, 0), lefpos(4 * (size_t)nc, -1);
+            const size_t sf = dp::cluster_smem(0, slots, 0, L), sb = dp::cluster_smem(1, 0, edges, L);
+            if (dp::cluster_smem(2, slots, edges, L) <= (size_t)dp::kBlockSmemMax && dp::cluster_fits(threads, sf, sb)) {
+                std::vector<int32_t> floc(4 * (size_t)nc, 0), push(4 * (size_t)nc, -1), range(2 * (size_t)nn);
+                for (int64_t n = 0; n < nn; n++) {
+                    range[2 * (size_t)n] = lfptr[(size_t)n];
+                    range[2 * (size_t)n + 1] = cp->fout_ptr[(size_t)n + 1] - cp->fout_ptr[(size_t)n];
+                }
                 for (int64_t c = 0; c < nc; c++) {
                     const uint32_t *r = &cp->fanin[4 * (size_t)c];
                     const int k = cp->op_arity[r[0] >> 24];
                     for (int j = 0; j < k; j++) {
                         const uint32_t m = j == 0 ? (r[0] & dp::kNetMask) : r[j];
                         floc[4 * (size_t)c + j] = loc[m];
-                        lefpos[4 * (size_t)c + j] = lfptr[m] + (cp->edge_fpos[4 * (size_t)c + j] - cp->fout_ptr[m]);
+                        push[4 * (size_t)c + j] = (loc[m] & ~0xFFFFFF) |
+                                                  (lfptr[m] + (cp->edge_fpos[4 * (size_t)c + j] - cp->fout_ptr[m]));
                     }
                 }
-                int32_t *dchunk = nullptr, *dbase = nullptr, *dfloc = nullptr, *dlfptr = nullptr, *dlefpos = nullptr;
+                int32_t *dchunk = nullptr, *dbase = nullptr, *dfloc = nullptr, *drange = nullptr, *dpush = nullptr;
+                float *dcoef = nullptr;
                 TRY(dalloc(D, &dchunk, chunk.size()));
                 TRY(dalloc(D, &dbase, base.size()));
                 TRY(dalloc(D, &dfloc, floc.size()));
-                TRY(dalloc(D, &dlfptr, lfptr.size()));
-                TRY(dalloc(D, &dlefpos, lefpos.size()));
+                TRY(dalloc(D, &drange, range.size()));
+                TRY(dalloc(D, &dpush, push.size()));
+                TRY(dalloc(D, &dcoef, 4 * (size_t)nc));
                 up(dchunk, chunk.data(), sizeof(int32_t) * chunk.size());
                 up(dbase, base.data(), sizeof(int32_t) * base.size());
                 up(dfloc, floc.data(), sizeof(int32_t) * floc.size());
-                up(dlfptr, lfptr.data(), sizeof(int32_t) * lfptr.size());
-                up(dlefpos, lefpos.data(), sizeof(int32_t) * lefpos.size());
+                up(drange, range.data(), sizeof(int32_t) * range.size());
+                up(dpush, push.data(), sizeof(int32_t) * push.size());
                 if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // before the host vectors go
-                D->cl = dp::ClusterMap{threads, slots, edges, dchunk, dbase, dfloc, dlfptr, dlefpos};
+                D->cl = dp::ClusterMap{threads, slots, edges, dchunk, dbase, dfloc, drange, dpush, dcoef};
             }
         }
     }
-    if (const char *v = std::getenv("DP_FLOW_BLOCKS")) D->flow_blocks_per_sm = std::atoi(v);
-    if (const char *v = std::getenv("DP_FLOW_SLEEP")) D->flow_sleep = (unsigned)std::atoi(v);
-    D->flow_grid[0] = dp::flow_grid(0, ctx->sm_count, D->flow_blocks_per_sm);
-    D->flow_grid[1] = dp::flow_grid(1, ctx->sm_count, 2);
+    for (int w = 0; w < 3; w++) D->flow_grid[w] = dp::flow_grid(w, ctx->sm_count);
+    D->timeouts_seen = ctx->timeouts;
     if (e != cudaSuccess) { s = cuda_err(ctx, e, "upload"); free_design(D); return s; }
     dp::launch_cload(d, st);
     for (auto &ev : D->ev)
@@ -879,6 +897,7 @@ dp_status dp_propagate(dp_design *D, const dp_config *cfg) {
     if (cfg->tr_mode == 2) return set_err(D->ctx, DP_EUNSUPPORTED, "the lag-one mode runs on batched inputs");
     DeviceGuard g(D->ctx->device);
     cudaStream_t st = D->ctx->stream;
+    repair_tags(D, st);
     rec(D, 0, st);
     cudaError_t le = q_forward(D, *cfg, st);
     rec(D, 1, st);
@@ -942,6 +961,7 @@ dp_status dp_backward(dp_design *D, const dp_config *cfg, float *gsp, float *gtr
     DeviceGuard g(D->ctx->device);
     cudaStream_t st = D->ctx->stream;
     rec(D, 3, st);
+    q_coef(D, *cfg, st);
     cudaError_t le = q_backward(D, *cfg, on_device ? gsp : nullptr, st);
     rec(D, 4, st);
     if ((s = cuda_err(D->ctx, le, "dp_backward")) != DP_OK) return s;
@@ -1025,6 +1045,7 @@ dp_status dp_step(dp_design *D, const dp_config *cfg, float *gsp, float *gtr, fl
         cudaEventRecordWithFlags(D->ev[0], cs, cudaEventRecordExternal);
         cudaError_t le = q_forward(D, *cfg, cs, D->fork);
         cudaEventRecordWithFlags(D->ev[1], cs, cudaEventRecordExternal);
+        q_coef(D, *cfg, cs);   // beside the rest of the generator
         cudaStreamWaitEvent(D->cap_stream2, D->fork, 0);
         q_sim_start(D, *cfg, D->cap_stream2);
         cudaEventRecord(D->join, D->cap_stream2);
@@ -1063,6 +1084,7 @@ dp_status dp_step(dp_design *D, const dp_config *cfg, float *gsp, float *gtr, fl
         if (e != cudaSuccess) { D->graph = nullptr; return cuda_err(D->ctx, e, "graph instantiate"); }
         D->graph_cfg = *cfg;
     }
+    repair_tags(D, st);
     cudaError_t e = cudaGraphLaunch(D->graph, st);
     if (e != cudaSuccess) return cuda_err(D->ctx, e, "graph launch");
     for (int i = 0; i < 5; i++) D->ev_valid[i] = true;

@@ -16,6 +16,7 @@ struct dp_ctx {
     int sm_count = 0;
     int clock_khz = 0;
     int *d_err = nullptr;   // device error word: a bounded wait gave up
+    unsigned timeouts = 0;  // times a synchronising call found it set
     std::string err;
 };
 
@@ -86,12 +87,10 @@ struct dp_design {
     cudaStream_t out_stream = nullptr;
     cudaEvent_t ev_grads = nullptr, ev_copies = nullptr;
     int grid[4] = {0, 0, 0, 0};   // persistent grids: forward, simulation, backward, wide simulation
-    int flow_grid[2] = {0, 0};     // dataflow grids: forward, simulation
+    int flow_grid[3] = {0, 0, 0};  // dataflow grids: forward, simulation, reverse
     int block_threads = 0;         // > 0: the design fits the single-block passes, with this many threads
     dp::ClusterMap cl;             // the single-cluster passes (cl.threads > 0: the design uses them)
-    // launch-shape tuning (defaults, overridable by DP_FLOW_BLOCKS / DP_FLOW_SLEEP for sweeps)
-    int flow_blocks_per_sm = 2;
-    unsigned flow_sleep = 0;
+    unsigned timeouts_seen = 0;    // the context's count of timed-out waits when the pair tags were last sound
     int64_t graph_kernels = 0;
     int64_t step_kernels = 0;
     // phase boundaries: start, forward, simulation levels, hybrid + power, backward, outputs

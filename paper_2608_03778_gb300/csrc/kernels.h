@@ -49,12 +49,15 @@ struct DevDesign {
     uint32_t *toggles, *ones;  // [n_nets]
     float *gnet;               // [n_nets] SP adjoint per net
     float *gfo;                // [n_edges] adjoint contribution of each edge, in fanout-CSR order
+    unsigned long long *edges; // [n_edges] the dataflow reverse pass's edges, in fanout-CSR order: partial
+                               // derivative, sink cell << 32
     uint64_t *words;           // [n_nets * T]
     double *partials;          // [2 * power_blocks]
     double *power;             // [4]: model, hybrid
     unsigned *bar;             // level-barrier arrival counters of the persistent passes (128-byte lines)
-    uint32_t *epoch;           // [4] pass counters: [0] forward (its parity tags the stored pairs)
-    const int32_t *chunk_ptr;  // [n_levels+2] level-aligned chunks of 32 (level 0 = startpoints)
+    unsigned long long *gcell; // [n_cells] the dataflow reverse pass's cell adjoints: value, pass number << 32
+    uint32_t *epoch;           // [8] pass counters: [0] forward (its parity tags the stored pairs), [1] dataflow
+                               // simulation, [2] dataflow reverse; [4], [5] blocks done of [0], [2] (0 at rest)
     const int32_t *pair_ptr;   // [n_levels+1] level-aligned cell pairs: pairs of level l are [pair_ptr[l-1], pair_ptr[l])
     unsigned *simdone;         // [n_cells] pass number of the simulation pass that last wrote the cell's words
     const int32_t *dead_ptr;   // [n_levels+2] nets by death level d (the highest level reading the net, else
@@ -85,11 +88,15 @@ void launch_bwd_level(const DevDesign &d, const OpTable &ops, int32_t c0, int32_
                       cudaStream_t s);
 void launch_bwd_start(const DevDesign &d, int grad_mode, int tr_mode, float K, float *grad_sp_in, cudaStream_t s);
 
-// pass counters and the dataflow schedule (kern_flow.cu)
+// pass counters and the dataflow schedule (kern_flow.cu); the passes advance their own counters
 void launch_bump(uint32_t *counter, cudaStream_t s);
-int flow_grid(int which, int sm_count, int blocks_per_sm);   // which: 0 forward, 1 simulation; 0 = unavailable
-cudaError_t launch_fwd_flow(const DevDesign &d, const OpTable &ops, int tr_mode, int grid, unsigned sleep_max,
-                            cudaStream_t s);
+int flow_grid(int which, int sm_count);   // which: 0 forward, 1 simulation, 2 reverse; 0 = unavailable
+cudaError_t launch_fwd_flow(const DevDesign &d, const OpTable &ops, int tr_mode, int grid, cudaStream_t s);
+// the reverse pass in two kernels: the partial derivatives and local terms, which need the forward pass
+// only (so they can run beside the simulation), then the levels.  cells: the partial derivatives by cell
+// (the cluster's pass); NULL: by fanout edge, with the sink cell, into d.edges
+void launch_bwd_coef(const DevDesign &d, const OpTable &ops, int tr_mode, float K, float *cells, cudaStream_t s);
+cudaError_t launch_bwd_flow(const DevDesign &d, int grad_mode, float *out_gsp, int grid, cudaStream_t s);
 // simulation levels without barriers (T % 4 == 0), bumps epoch[1] first
 cudaError_t launch_sim_flow(const DevDesign &d, const OpTable &ops, int T, int grid, cudaStream_t s);
 
@@ -112,18 +119,20 @@ struct ClusterMap {
     const int32_t *chunk = nullptr;     // [L+1] cells of level l per block (level 0: the startpoints)
     const int32_t *base = nullptr;      // [C][L+1] first slot of block b's chunk of level l
     const int32_t *floc = nullptr;      // [4 nc] location of each input net: owner block << 24 | slot
-    const int32_t *lfptr = nullptr;     // [nn] start of net n's fanout range in its owner's copy
-    const int32_t *lefpos = nullptr;    // [4 nc] position of each input edge in its owner's copy
+    const int32_t *range = nullptr;     // [2 nn] net n's fanout range in its owner's copy: first, count
+    const int32_t *push = nullptr;      // [4 nc] each input edge's place: owner block << 24 | position, -1 unused
+    float *coef = nullptr;              // [4 nc] the reverse pass's partial derivatives
 };
-// cluster_smem(0 forward, 1 reverse, ...): dynamic shared memory per block; cluster_fits:
+// cluster_smem: dynamic shared memory per block (0 forward, 1 reverse, 2 the state of both passes,
+// which decides whether a design takes the cluster); cluster_fits:
 // whether one such cluster can run on this device (also sets the kernels' shared-memory and
 // cluster-size attributes)
 size_t cluster_smem(int which, int64_t slots, int64_t n_edges_local, int n_levels);
 bool cluster_fits(int threads, size_t smem_fwd, size_t smem_bwd);
 cudaError_t launch_fwd_cluster(const DevDesign &d, const OpTable &ops, const ClusterMap &m, int tr_mode,
                                cudaStream_t s);
-cudaError_t launch_bwd_cluster(const DevDesign &d, const OpTable &ops, const ClusterMap &m, int grad_mode,
-                               int tr_mode, float K, float *out_gsp, cudaStream_t s);
+cudaError_t launch_bwd_cluster(const DevDesign &d, const ClusterMap &m, int grad_mode, float *out_gsp,
+                               cudaStream_t s);   // after launch_bwd_coef with m.coef
 
 // the forward and the reverse pass of a small design in one block (kern_persist.cu);
 // block_smem(0 forward, 1 reverse, ...): the dynamic shared memory each needs;

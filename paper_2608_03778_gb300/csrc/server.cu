@@ -732,9 +732,9 @@ dp_status dp_server_add_design(dp_server *srv, const char *netlist, size_t netli
     const int64_t ns = cp->n_start, nc = cp->n_cells, nn = cp->n_nets, ne = cp->n_edges;
     const int64_t S = srv->cfg.max_batch;
     const int nslots = srv->cfg.slots_per_design;
-    // device bytes per slot: resident netlist (about 24 B per net, 40 per cell, 8 per edge) and
+    // device bytes per slot: resident netlist (about 24 B per net, 48 per cell, 16 per edge) and
     // batch buffers
-    const double need = 24.0 * nn + 40.0 * nc + 8.0 * ne + 72.0 * nn +
+    const double need = 24.0 * nn + 48.0 * nc + 16.0 * ne + 72.0 * nn +
                         (double)S * (8.0 * nn + 4.0 * ne + 16.0 * ns + 4.0 * nn + 4.0 * std::max(nn, nc) +
                                      4.0 * (2 * ns + nc) + 8.0 * ns + 8.0 * dp::kBatchPowerChunks + 8.0 * nc +
                                      4.0 * nn) +

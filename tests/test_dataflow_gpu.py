@@ -1,0 +1,55 @@
+"""The dataflow forward and reverse passes (no barrier between levels) against the grid-wide
+passes and the per-level launches: the same bits, at the sizes where their work splits change."""
+import numpy as np
+import pytest
+
+from paper_2608_03778_gb300 import netgen
+from tests.test_parity_gpu import ctx, dp, gpu_run  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+KEYS = ["sp", "tr", "beta", "tr_hyb", "toggles", "grad_sp_in", "grad_tr_in", "grad_pincap", "grad_cload"]
+
+# levels wider than the 38,912 cells the grid holds at once, with fanouts far above the eight edges a
+# thread preloads; a narrow deep netlist; one level; more startpoints than the grid holds
+SPECS = [netgen.NetlistSpec(130_000, 300, 200, 3, 64, 5), netgen.NetlistSpec(1_500, 9, 8, 200, 32, 6),
+         netgen.NetlistSpec(2_500, 2_000, 500, 1, 16, 7), netgen.NetlistSpec(4_000, 45_000, 5_000, 9, 8, 8)]
+
+
+@pytest.mark.parametrize("spec", SPECS, ids=lambda s: f"{s.n_cells}x{s.depth}")
+def test_dataflow_matches_barriers_and_launches(dp, ctx, library_text, spec):  # noqa: F811
+    text = netgen.netlist_text(spec)
+    sp, tr = netgen.scenario_inputs(spec.n_start, 50)
+    for grad_mode, tr_mode, use_step in [(0, 0, False), (1, 1, True)]:
+        runs = [gpu_run(dp, ctx, text, library_text, sp[:, 0], tr[:, 0],
+                        dp.config(grad_mode=grad_mode, tr_mode=tr_mode, schedule=s, sim_words=16), use_step, True)
+                for s in (0, 3, 2, 1)]
+        for other in runs[1:]:
+            for k in KEYS:
+                np.testing.assert_array_equal(runs[0][k], other[k], err_msg=k)
+
+
+def test_dataflow_after_a_wait_that_gave_up(dp, ctx, library_text):  # noqa: F811
+    """A timed-out wait may leave pairs of two passes behind; the next pass must not take one for its own."""
+    spec = netgen.NetlistSpec(20_000, 300, 700, 12, 16, 9)
+    text = netgen.netlist_text(spec)
+    sp, tr = netgen.scenario_inputs(spec.n_start, 51, 2)
+    d = dp.dp_design_load(ctx, text, library_text)
+    try:
+        nn = dp.dp_design_info(d).n_nets
+        got = []
+        for schedule in (3, 2):
+            cfg = dp.config(schedule=schedule)
+            for s in (0, 1):
+                dp.dp_set_inputs(ctx, d, sp[:, s].copy(), tr[:, s].copy())
+                with pytest.raises(dp.DPError):
+                    dp.dp_selftest_wait(ctx, 0.01)
+                dp.dp_propagate(ctx, d, cfg)
+                out = np.zeros(nn, np.float32)
+                dp.dp_get_nets(ctx, d, out)
+                got.append(out)
+        np.testing.assert_array_equal(got[0], got[2])
+        np.testing.assert_array_equal(got[1], got[3])
+        assert not np.array_equal(got[0], got[1])
+    finally:
+        dp.dp_design_free(d)
