@@ -7,6 +7,8 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "capi_internal.h"
@@ -219,6 +221,12 @@ bool persistent(const dp_design *D, const dp_config &c, int which) {
 bool small_pass(const dp_design *D, const dp_config &c) { return c.schedule == 0 && D->block_threads > 0; }
 // ... and of a mid-size design in one thread-block cluster (schedule 0)
 bool cluster_pass(const dp_design *D, const dp_config &c) { return c.schedule == 0 && D->cl.threads > 0; }
+// the sliced simulation, where a design's live nets fit in shared memory and it is the faster one
+// (nv > 0; schedule 0)
+dp::SliceShape sliced(const dp_design *D, const dp_config &c) {
+    if (c.schedule != 0 || D->sl.slots == 0) return dp::SliceShape{0, 0};
+    return dp::slice_shape(D->sl, D->d.n_cells, D->d.n_levels, c.sim_words, D->ctx->sm_count);
+}
 // the dataflow passes: the forward and the reverse pass of the designs that do not fit the two
 // above (schedule 0), and on request (schedule 3, which has a dataflow simulation too)
 bool dataflow(const dp_design *D, const dp_config &c, int which) {
@@ -275,7 +283,10 @@ void q_sim_start(dp_design *D, const dp_config &c, cudaStream_t s) {
 
 // the simulation levels, beta and the hybrid power (after the generator and the forward pass)
 cudaError_t q_sim_levels(dp_design *D, const dp_config &c, cudaStream_t s) {
-    if (dataflow(D, c, 1) && dp::wide_ok(c.sim_words) && D->d.simdone) {
+    if (const dp::SliceShape sh = sliced(D, c); sh.nv > 0) {
+        cudaError_t e = dp::launch_sim_slice(D->d, D->sl, c.sim_words, sh, s);
+        if (e != cudaSuccess) return e;
+    } else if (dataflow(D, c, 1) && dp::wide_ok(c.sim_words) && D->d.simdone) {
         cudaError_t e = dp::launch_sim_flow(D->d, D->ops, c.sim_words, D->flow_grid[1], s);
         if (e != cudaSuccess) return e;
     } else if (persistent(D, c, 3) && dp::wide_ok(c.sim_words)) {
@@ -559,6 +570,106 @@ dp_status dp_selftest_pending_error(int action, int32_t *pending) {
     return DP_OK;
 }
 
+namespace {
+// The tables of the sliced simulation (kern_slice.cu), built on a thread of their own beside the
+// rest of an upload.  slots = 0: the design does not use it.
+struct SliceTables {
+    std::vector<int32_t> start_slot, round_ptr;
+    std::vector<uint32_t> rec;
+    std::vector<uint16_t> fourth;
+    int64_t slots = 0;
+    int threads = 0;
+    struct Worker {
+        std::thread t;
+        void join() {
+            if (t.joinable()) t.join();
+        }
+        ~Worker() { join(); }
+    } worker;   // the last member: it ends before the tables go
+
+    void build(const dp_compiled *cp, const dp::OpTable &ops, const std::vector<int32_t> &dead_ptr,
+               const std::vector<int32_t> &dead_net) {
+        const int L = cp->n_levels;
+        const int64_t ns = cp->n_start, nc = cp->n_cells, nn = cp->n_nets;
+        const int32_t *lvl = cp->lvl_ptr.data(), *fout = cp->fout_ptr.data();
+        // slots by lifetime: a net holds one from its level to the last level that reads it; level l
+        // takes slots that were free before it (its cells still read the others) and, cell i of a level,
+        // one congruent to i mod 32 if there is one: neighbouring lanes then store to different banks
+        std::vector<int32_t> slot((size_t)nn, -1);
+        std::vector<std::vector<int32_t>> open(32);
+        int64_t high = 0, n_open = 0;
+        for (int l = 0; l <= L; l++) {
+            const int64_t lo = l ? ns + lvl[l - 1] : 0, hi = l ? ns + lvl[l] : ns;
+            for (int64_t n = lo; n < hi; n++) {
+                if (fout[n + 1] == fout[n]) continue;
+                size_t b = (size_t)((n - lo) & 31);
+                if (n_open == 0) {
+                    slot[(size_t)n] = (int32_t)high++;
+                    continue;
+                }
+                while (open[b].empty()) b = (b + 1) & 31;
+                slot[(size_t)n] = open[b].back();
+                open[b].pop_back();
+                n_open--;
+            }
+            if (high > dp::kSliceMaxSlots) return;
+            for (int32_t k = dead_ptr[(size_t)l]; k < dead_ptr[(size_t)l + 1]; k++) {
+                const int32_t v = slot[(size_t)dead_net[(size_t)k]];
+                if (v >= 0) open[(size_t)(v & 31)].push_back(v), n_open++;
+            }
+        }
+        // threads per block: a round costs about 14 cycles per warp, or its latency, and a level a barrier
+        double best = 0;
+        for (int p = 128; p <= 1024; p += 32) {
+            double cost = 0;
+            for (int l = 1; l <= L; l++)
+                cost += 60.0 + (double)((lvl[l] - lvl[l - 1] + p - 1) / p) * std::max(200.0, 14.0 * p / 32);
+            if (threads == 0 || cost < best) threads = p, best = cost;
+        }
+        round_ptr.assign((size_t)L + 1, 0);
+        for (int l = 1; l <= L; l++)
+            round_ptr[(size_t)l] = round_ptr[(size_t)l - 1] + (lvl[l] - lvl[l - 1] + threads - 1) / threads;
+        rec.resize(4 * (size_t)threads * (size_t)round_ptr[(size_t)L]);
+        fourth.assign((size_t)nc, 0);
+        start_slot.assign(slot.begin(), slot.begin() + ns);
+        for (int l = 1; l <= L; l++) {
+            uint32_t *o = &rec[4 * (size_t)threads * (size_t)round_ptr[(size_t)l - 1]];
+            uint32_t *const end = &rec[0] + 4 * (size_t)threads * (size_t)round_ptr[(size_t)l];
+            for (int64_t c = lvl[l - 1]; c < lvl[l]; c++, o += 4) {
+                const uint32_t *r = &cp->fanin[4 * (size_t)c];
+                const uint32_t op = r[0] >> 24, k = cp->op_arity[op], tt = cp->op_tt[op];
+                uint32_t in[4] = {0, 0, 0, 0};
+                for (uint32_t j = 0; j < k; j++) in[j] = (uint32_t)slot[j == 0 ? (r[0] & dp::kNetMask) : r[j]];
+                o[0] = in[0] | in[1] << 16;
+                o[1] = in[2] | ((uint32_t)slot[(size_t)(ns + c)] & 0xFFFFu) << 16;
+                o[2] = k <= 3 ? ops.e[op] >> 24 : (tt & 0xFFu) | 0x100u | (tt >> 8) << 16;
+                o[3] = (uint32_t)c;
+                if (k > 3) fourth[(size_t)c] = (uint16_t)in[3];
+            }
+            for (; o < end; o += 4) o[0] = 0u, o[1] = 0xFFFF0000u, o[2] = 0u, o[3] = 0xFFFFFFFFu;   // padding
+        }
+        slots = std::max<int64_t>(high, 1);
+    }
+    void start(const dp_compiled *cp, const dp::OpTable &ops, const std::vector<int32_t> &dead_ptr,
+               const std::vector<int32_t> &dead_net) {
+        if (cp->n_levels < 1) return;
+        auto run = [this, cp, ops, &dead_ptr, &dead_net] {   // (the design may be freed first)
+            try {
+                build(cp, ops, dead_ptr, dead_net);
+            } catch (const std::bad_alloc &) {
+                slots = 0;   // without memory for them the other simulations run
+            }
+        };
+        try {
+            worker.t = std::thread(run);
+        } catch (const std::system_error &) {
+            run();   // no thread to be had
+        }
+    }
+};
+
+}  // namespace
+
 dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) {
     if (!ctx || !cp || !out) return set_err(ctx, DP_EINVAL, "NULL argument");
     *out = nullptr;
@@ -604,6 +715,8 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
         std::vector<int32_t> at(dead_ptr.begin(), dead_ptr.end() - 1);
         for (size_t n = 0; n < death.size(); n++) dead_net[(size_t)at[(size_t)death[n]]++] = (int32_t)n;
     }
+    SliceTables slice;
+    slice.start(cp, D->ops, dead_ptr, dead_net);
     int32_t *dptr = nullptr, *dnet = nullptr;
     // level-aligned cell pairs (the dataflow simulation's unit of work)
     std::vector<int32_t> pair_ptr((size_t)cp->n_levels + 1, 0);
@@ -709,12 +822,14 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
         const int64_t slots = *std::max_element(held.begin(), held.end());
         if (threads <= dp::kClusterMaxThreads && dp::cluster_smem(0, slots, 0, L) <= (size_t)dp::kBlockSmemMax) {
             std::vector<int32_t> loc((size_t)nn), lfptr((size_t)nn);
-            for (int l = 0; l <= L; l++)
-                for (int64_t i = 0; i < hi_of(l) - lo_of(l); i++) {
-                    const int64_t b = i / chunk[(size_t)l];
-                    loc[(size_t)(lo_of(l) + i)] =
-                        (int32_t)((b << 24) | (base[(size_t)b * (L + 1) + l] + i % chunk[(size_t)l]));
+            for (int l = 0; l <= L; l++) {
+                int64_t n = lo_of(l);
+                const int64_t hi = hi_of(l);
+                for (int64_t b = 0; n < hi; b++) {
+                    const int32_t first = (int32_t)(b << 24) | base[(size_t)b * (L + 1) + l];
+                    for (int32_t i = 0; i < chunk[(size_t)l] && n < hi; i++) loc[(size_t)n++] = first + i;
                 }
+            }
             std::vector<int64_t> fill((size_t)C, 0);
             for (int64_t n = 0; n < nn; n++) {
                 const size_t b = (size_t)((uint32_t)loc[(size_t)n] >> 24);
@@ -756,6 +871,21 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
                 D->cl = dp::ClusterMap{threads, slots, edges, dchunk, dbase, dfloc, drange, dpush, dcoef};
             }
         }
+    }
+    slice.worker.join();
+    if (slice.slots > 0 && e == cudaSuccess && dp::slice_fits(slice.slots)) {
+        uint32_t *drec = nullptr;
+        uint16_t *dfourth = nullptr;
+        int32_t *dround = nullptr, *dstart = nullptr;
+        TRY(dalloc(D, &drec, slice.rec.size()));
+        TRY(dalloc(D, &dround, slice.round_ptr.size()));
+        TRY(dalloc(D, &dfourth, slice.fourth.size()));
+        TRY(dalloc(D, &dstart, slice.start_slot.size()));
+        up(drec, slice.rec.data(), sizeof(uint32_t) * slice.rec.size());
+        up(dround, slice.round_ptr.data(), sizeof(int32_t) * slice.round_ptr.size());
+        up(dfourth, slice.fourth.data(), sizeof(uint16_t) * slice.fourth.size());
+        up(dstart, slice.start_slot.data(), sizeof(int32_t) * slice.start_slot.size());
+        D->sl = dp::SlicePlan{slice.slots, slice.threads, drec, dround, dfourth, dstart};
     }
     for (int w = 0; w < 3; w++) D->flow_grid[w] = dp::flow_grid(w, ctx->sm_count);
     D->timeouts_seen = ctx->timeouts;

@@ -89,6 +89,7 @@ struct dp_design {
     int grid[4] = {0, 0, 0, 0};   // persistent grids: forward, simulation, backward, wide simulation
     int flow_grid[3] = {0, 0, 0};  // dataflow grids: forward, simulation, reverse
     int block_threads = 0;         // > 0: the design fits the single-block passes, with this many threads
+    dp::SlicePlan sl;              // the sliced simulation (sl.slots > 0: the design uses it)
     dp::ClusterMap cl;             // the single-cluster passes (cl.threads > 0: the design uses them)
     unsigned timeouts_seen = 0;    // the context's count of timed-out waits when the pair tags were last sound
     int64_t graph_kernels = 0;

@@ -24,79 +24,18 @@ __device__ __forceinline__ uint32_t threshold16(double p) {
 // and its high 16 bits at odd cycles.  t = 0 draws the initial state with
 // P(1) = SP; t >= 1 flips a 1 with p10 = TR / 2SP and a 0 with
 // p01 = TR / 2(1 - SP), which keeps SP stationary and makes TR the expected
-// toggle rate.  The four lanes' states live in a 4-bit mask; the 64-bit word
-// of each cycle is assembled from four warp ballots.
-__global__ void __launch_bounds__(256) k_sim_start(const float *__restrict__ sp_in, const float *__restrict__ tr_in,
-                                                   uint64_t *words, uint32_t *toggles, uint32_t *ones, int64_t ns,
-                                                   int T, uint32_t key0, uint32_t key1) {
-    const int q = threadIdx.x & 15;
-    const int half = (threadIdx.x >> 4) & 1;
-    const int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 4) + (threadIdx.x >> 4);
-    const bool valid = k < ns;
-    // the three thresholds of startpoint k, computed by one thread of its half-warp (the
-    // divisions run on the FP64 pipe, slow on this part) and shared with the other fifteen
-    uint32_t t_init = 0, t10 = 0, t01 = 0;
-    if (valid && q == 0) {
-        const double sp = (double)sp_in[k], tr = (double)tr_in[k];
-        const double p10 = sp > 0.0 ? tr / (2.0 * sp) : 0.0;
-        const double p01 = sp < 1.0 ? tr / (2.0 * (1.0 - sp)) : 0.0;
-        t_init = threshold16(sp);
-        t10 = threshold16(p10);
-        t01 = threshold16(p01);
-    }
-    t_init = __shfl_sync(0xFFFFFFFFu, t_init, 0, 16);
-    t10 = __shfl_sync(0xFFFFFFFFu, t10, 0, 16);
-    t01 = __shfl_sync(0xFFFFFFFFu, t01, 0, 16);
-    const uint32_t sel = half ? 0x7632u : 0x5410u;  // this half-warp's 16 ballot bits of two ballots
-    uint32_t st = 0;                                // bit r = current value of lane 16 r + q
-    uint32_t n_flip = 0, n_one = 0;
-    uint64_t mine = 0;                              // word t with t % 16 == q of the current 16 cycles
-    uint4 u = make_uint4(0, 0, 0, 0);
-    for (int t = 0; t < T; t++) {
-        if ((t & 1) == 0) u = philox4x32_10(make_uint4((uint32_t)k, (uint32_t)(t >> 1), (uint32_t)q, 0u), key0, key1);
-        const int sh = (t & 1) << 4;
-        const uint32_t d0 = (u.x >> sh) & 0xFFFFu, d1 = (u.y >> sh) & 0xFFFFu;
-        const uint32_t d2 = (u.z >> sh) & 0xFFFFu, d3 = (u.w >> sh) & 0xFFFFu;
-        if (t == 0) {
-            st = (uint32_t)(d0 < t_init) | ((uint32_t)(d1 < t_init) << 1) | ((uint32_t)(d2 < t_init) << 2) |
-                 ((uint32_t)(d3 < t_init) << 3);
-        } else {
-            const uint32_t f = (uint32_t)(d0 < ((st & 1u) ? t10 : t01)) |
-                               ((uint32_t)(d1 < ((st & 2u) ? t10 : t01)) << 1) |
-                               ((uint32_t)(d2 < ((st & 4u) ? t10 : t01)) << 2) |
-                               ((uint32_t)(d3 < ((st & 8u) ? t10 : t01)) << 3);
-            n_flip += __popc(f);
-            st ^= f;
-        }
-        n_one += __popc(st);
-        const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, st & 1u), b1 = __ballot_sync(0xFFFFFFFFu, st & 2u);
-        const uint32_t b2 = __ballot_sync(0xFFFFFFFFu, st & 4u), b3 = __ballot_sync(0xFFFFFFFFu, st & 8u);
-        const uint64_t w = (uint64_t)__byte_perm(b0, b1, sel) | ((uint64_t)__byte_perm(b2, b3, sel) << 32);
-        if ((t & 15) == q) mine = w;
-        if ((t & 15) == 15 || t == T - 1) {
-            const int t_q = (t & ~15) + q;
-            if (valid && t_q < T) words[k * T + t_q] = mine;
-        }
-    }
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
-        n_flip += __shfl_xor_sync(0xFFFFFFFFu, n_flip, o);
-        n_one += __shfl_xor_sync(0xFFFFFFFFu, n_one, o);
-    }
-    if (valid && q == 0) {
-        toggles[k] = n_flip;
-        ones[k] = n_one;
-    }
-}
-
-// The same chains for T a multiple of 16, arranged for fewer instructions: one
-// Philox call per two cycles with its low and high halves at fixed positions,
-// sixteen cycles unrolled per block (so the word a thread keeps and the store
-// are fixed at compile time), and the first cycle - the initial draw -
-// peeled off.  Each flip is formed from both threshold tests and the state by
-// one bitwise select.  Identical bits to k_sim_start.
+// toggle rate.  The 64-bit word of each cycle is assembled from four warp ballots.
+//
+// One Philox call per two cycles with its low and high halves at fixed positions, sixteen cycles
+// unrolled per block (so the word a thread keeps and the store are fixed at compile time), the
+// first cycle - the initial draw - peeled off.  When the word count is no multiple of sixteen the
+// last block's chains run on past it; those words are neither stored nor counted (13,000-cell step
+// with 250 words: 48 us with a loop over single cycles, one Philox call in two of them).
+//
+// General form: the four lanes' states live in a 4-bit mask; each flip is formed from both
+// threshold tests and the state by one bitwise select.
 struct ChainState {
-    uint32_t st, n_flip, n_one;
+    uint32_t st;
 };
 
 // one cycle: the four lanes' 16-bit draws d[r]; FIRST draws the initial state
@@ -112,10 +51,8 @@ __device__ __forceinline__ uint64_t chain_cycle(ChainState &c, const uint32_t (&
         const uint32_t c01 = (uint32_t)(d[0] < t01) | ((uint32_t)(d[1] < t01) << 1) | ((uint32_t)(d[2] < t01) << 2) |
                              ((uint32_t)(d[3] < t01) << 3);
         const uint32_t f = (c.st & c10) | (~c.st & c01 & 15u);   // a 1 flips on p10, a 0 on p01
-        c.n_flip += __popc(f);
         c.st ^= f;
     }
-    c.n_one += __popc(c.st);
     const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, c.st & 1u), b1 = __ballot_sync(0xFFFFFFFFu, c.st & 2u);
     const uint32_t b2 = __ballot_sync(0xFFFFFFFFu, c.st & 4u), b3 = __ballot_sync(0xFFFFFFFFu, c.st & 8u);
     return (uint64_t)__byte_perm(b0, b1, sel) | ((uint64_t)__byte_perm(b2, b3, sel) << 32);
@@ -197,7 +134,7 @@ __device__ __forceinline__ uint64_t fast_block16(FastChain &c, uint32_t k, int t
     return mine;
 }
 
-__global__ void __launch_bounds__(256) k_sim_start16(const float *__restrict__ sp_in, const float *__restrict__ tr_in,
+__global__ void __launch_bounds__(256) k_sim_start(const float *__restrict__ sp_in, const float *__restrict__ tr_in,
                                                      uint64_t *words, uint32_t *toggles, uint32_t *ones, int64_t ns,
                                                      int T, uint32_t key0, uint32_t key1) {
     const int q = threadIdx.x & 15;
@@ -218,47 +155,38 @@ __global__ void __launch_bounds__(256) k_sim_start16(const float *__restrict__ s
     t01 = __shfl_sync(0xFFFFFFFFu, t01, 0, 16);
     const uint32_t sel = half ? 0x7632u : 0x5410u;
     uint64_t *out = words + (valid ? k : 0) * T;
+    uint32_t n_one = 0, n_flip = 0;
+    uint64_t carry = 0;
+    auto take = [&](uint64_t w, int t) {   // word t = t0 + q: stored and counted if it exists
+        const uint64_t prev = __shfl_up_sync(0xFFFFFFFFu, w, 1, 16);
+        if (t < T) {
+            if (valid) out[t] = w;
+            n_one += __popcll(w);
+            if (t > 0) n_flip += __popcll(w ^ (q > 0 ? prev : carry));
+        }
+        carry = __shfl_sync(0xFFFFFFFFu, w, 15, 16);
+    };
     if (!__any_sync(0xFFFFFFFFu, (t_init | t10 | t01) >= 65536u)) {   // warp-uniform
         FastChain c{};
-        uint32_t n_one = 0, n_flip = 0;
-        uint64_t carry = 0;
-        for (int t0 = 0; t0 < T; t0 += 16) {
-            const uint64_t w = t0 == 0 ? fast_block16<true>(c, (uint32_t)k, 0, q, key0, key1, t_init << 16,
-                                                            t10 << 16, t01 << 16, sel)
-                                       : fast_block16<false>(c, (uint32_t)k, t0, q, key0, key1, t_init << 16,
-                                                             t10 << 16, t01 << 16, sel);
-            if (valid) out[t0 + q] = w;
-            const uint64_t prev = __shfl_up_sync(0xFFFFFFFFu, w, 1, 16);
-            n_one += __popcll(w);
-            if (t0 + q > 0) n_flip += __popcll(w ^ (q > 0 ? prev : carry));
-            carry = __shfl_sync(0xFFFFFFFFu, w, 15, 16);
-        }
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) {
-            n_flip += __shfl_xor_sync(0xFFFFFFFFu, n_flip, o);
-            n_one += __shfl_xor_sync(0xFFFFFFFFu, n_one, o);
-        }
-        if (valid && q == 0) {
-            toggles[k] = n_flip;
-            ones[k] = n_one;
-        }
-        return;
-    }
-    ChainState c{0u, 0u, 0u};
-    uint64_t w = chain_block16<true>(c, (uint32_t)k, 0, q, key0, key1, t_init, t10, t01, sel);
-    if (valid) out[q] = w;
-    for (int t0 = 16; t0 < T; t0 += 16) {
-        w = chain_block16<false>(c, (uint32_t)k, t0, q, key0, key1, t_init, t10, t01, sel);
-        if (valid) out[t0 + q] = w;
+        for (int t0 = 0; t0 < T; t0 += 16)
+            take(t0 == 0 ? fast_block16<true>(c, (uint32_t)k, 0, q, key0, key1, t_init << 16, t10 << 16, t01 << 16, sel)
+                         : fast_block16<false>(c, (uint32_t)k, t0, q, key0, key1, t_init << 16, t10 << 16, t01 << 16,
+                                               sel),
+                 t0 + q);
+    } else {
+        ChainState c{0u};
+        take(chain_block16<true>(c, (uint32_t)k, 0, q, key0, key1, t_init, t10, t01, sel), q);
+        for (int t0 = 16; t0 < T; t0 += 16)
+            take(chain_block16<false>(c, (uint32_t)k, t0, q, key0, key1, t_init, t10, t01, sel), t0 + q);
     }
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) {
-        c.n_flip += __shfl_xor_sync(0xFFFFFFFFu, c.n_flip, o);
-        c.n_one += __shfl_xor_sync(0xFFFFFFFFu, c.n_one, o);
+        n_flip += __shfl_xor_sync(0xFFFFFFFFu, n_flip, o);
+        n_one += __shfl_xor_sync(0xFFFFFFFFu, n_one, o);
     }
     if (valid && q == 0) {
-        toggles[k] = c.n_flip;
-        ones[k] = c.n_one;
+        toggles[k] = n_flip;
+        ones[k] = n_one;
     }
 }
 
@@ -347,14 +275,8 @@ __global__ void k_hybrid(const uint32_t *__restrict__ toggles, const float *__re
 
 void launch_sim_start(const DevDesign &d, int T, uint64_t seed, cudaStream_t s) {
     if (d.n_start == 0) return;
-    if (T % 16 == 0) {
-        k_sim_start16<<<(unsigned)cdiv(d.n_start, 16), 256, 0, s>>>(d.sp_in, d.tr_in, d.words, d.toggles, d.ones,
-                                                                    d.n_start, T, (uint32_t)seed,
-                                                                    (uint32_t)(seed >> 32));
-        return;
-    }
     k_sim_start<<<(unsigned)cdiv(d.n_start, 16), 256, 0, s>>>(d.sp_in, d.tr_in, d.words, d.toggles, d.ones,
-                                                              d.n_start, T, (uint32_t)seed, (uint32_t)(seed >> 32));
+                                                                d.n_start, T, (uint32_t)seed, (uint32_t)(seed >> 32));
 }
 
 void launch_sim_level(const DevDesign &d, const OpTable &ops, int32_t c0, int32_t c1, int T, cudaStream_t s) {

@@ -235,6 +235,24 @@ void launch_radix_hist(const float *scores, int64_t n, uint32_t prefix, uint32_t
 void launch_radix_collect(const float *scores, int64_t n, uint32_t thr, int32_t *idx, unsigned *count, int64_t cap,
                           cudaStream_t s);
 
+// simulation by slices of lanes and cycles, the live nets in shared memory (kern_slice.cu)
+struct SlicePlan {
+    int64_t slots = 0;                    // live nets at most (0: the design does not use it)
+    int threads = 0;                      // threads per block: cells per round
+    const uint32_t *rec = nullptr;        // [4 x threads x rounds] the cells' records, levels padded to whole rounds
+    const int32_t *round_ptr = nullptr;   // [L+1] first round of level l + 1
+    const uint16_t *fourth = nullptr;     // [nc] 4-input cells: fourth input slot
+    const int32_t *start_slot = nullptr;  // [ns] slot of each startpoint, -1 if nothing reads it
+};
+struct SliceShape {
+    int nv, lanes;   // 32-bit words per net and block; lanes per block (8, 16 or 32)
+};
+constexpr int64_t kSliceMaxSlots = 224 * 1024 / 4;   // one 32-bit word per net
+bool slice_fits(int64_t slots);   // also raises the kernels' shared-memory limit
+// the fastest shape for T words; nv = 0 where the wide simulation is faster
+SliceShape slice_shape(const SlicePlan &p, int64_t n_cells, int n_levels, int T, int sm_count);
+cudaError_t launch_sim_slice(const DevDesign &d, const SlicePlan &p, int T, SliceShape sh, cudaStream_t s);
+
 // simulation (kern_sim.cu)
 void launch_sim_start(const DevDesign &d, int T, uint64_t seed, cudaStream_t s);
 void launch_sim_level(const DevDesign &d, const OpTable &ops, int32_t c0, int32_t c1, int T, cudaStream_t s);

@@ -53,3 +53,36 @@ def test_dataflow_after_a_wait_that_gave_up(dp, ctx, library_text):  # noqa: F81
         assert not np.array_equal(got[0], got[1])
     finally:
         dp.dp_design_free(d)
+
+
+# word counts around the sliced simulation's runs (a run of N cycles adds N - 1), one wave of blocks and
+# several, startpoint words around the generator's blocks of sixteen
+@pytest.mark.parametrize("T", [2, 3, 4, 5, 15, 16, 17, 31, 32, 64, 65, 127, 250, 400])
+def test_sliced_simulation_matches_the_others(dp, ctx, library_text, T):  # noqa: F811
+    from tests._netlists import custom_case
+    rng = np.random.default_rng(T)
+    cases = [(netgen.netlist_text(netgen.NetlistSpec(3_000, 40, 60, 11, 16, 12)), library_text),
+             (netgen.netlist_text(netgen.NetlistSpec(9_000, 400, 100, 3, 16, 13)), library_text)]   # 3 rounds a level
+    if T in (5, 64, 65):
+        cases.append(custom_case(rng, n_in=30, n_cells=2_500))   # 0- to 4-input cells, constants
+    for text, lib in cases:
+        d = dp.dp_design_load(ctx, text, lib)
+        try:
+            i = dp.dp_design_info(d)
+            sp = rng.uniform(0, 1, i.n_start).astype(np.float32)
+            sp[0] = 1.0                                          # a threshold of 2^16: the general chains
+            tr = (rng.uniform(0, 1, i.n_start) * 2 * np.minimum(sp, 1 - sp)).astype(np.float32)
+            dp.dp_set_inputs(ctx, d, sp, tr)
+            got = []
+            for schedule in (0, 2, 1):
+                cfg = dp.config(schedule=schedule, sim_words=T, seed=T)
+                dp.dp_propagate(ctx, d, cfg)
+                dp.dp_simulate(ctx, d, cfg)
+                tg, on = np.zeros(i.n_nets, np.uint32), np.zeros(i.n_nets, np.uint32)
+                dp.dp_get_nets(ctx, d, None, None, None, None, tg, on)
+                got.append((tg, on))
+            for other in got[1:]:
+                np.testing.assert_array_equal(got[0][0], other[0])
+                np.testing.assert_array_equal(got[0][1], other[1])
+        finally:
+            dp.dp_design_free(d)
