@@ -333,11 +333,13 @@ dp_status dp_phase_times(dp_design *d, float *ms5);
  * with a new n_scen outside capture also runs the launch-shape autotuner
  * (times every candidate shape of the forward and reverse kernels on the
  * staged inputs and keeps the fastest; synchronises).  The environment
- * variable DP_BATCH_SHAPE="bx,by[,bx2,by2]" fixes the shapes instead.
+ * variable DP_BATCH_SHAPE="bx,by[,bx2,by2]" fixes the shapes instead.  Where a
+ * level's work is small both passes may run by scenario groups, one launch each
+ * (DP_BATCH_GROUP="lanes,v,blocks,threads" fixes that).
  * Every shape gives bitwise identical results. */
 dp_status dp_set_inputs_batch(dp_design *d, const float *sp, const float *tr, int32_t n_scen, int on_device);
 
-/* Shapes in use (bx threads over scenarios x by cells per block x v scenarios
+/* Shapes of the level launches (bx threads over scenarios x by cells per block x v scenarios
  * per thread, v = 1 or 2; v = 2 applies to even n_scen) for the forward
  * (shape6[0..2]) and the reverse pass (shape6[3..5]), and the tuner's best
  * times in ms (ms2, may be NULL; 0 when fixed by the environment).  Every

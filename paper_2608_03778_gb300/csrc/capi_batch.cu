@@ -115,14 +115,55 @@ bool parse_shape_env(dp::BatchShape *f, dp::BatchShape *b) {
     return true;
 }
 
+// DP_BATCH_GROUP = "lanes,v,blocks,threads": that group shape for both passes wherever v divides S
+bool parse_group_env(dp::GroupShape *g) {
+    const char *v = std::getenv("DP_BATCH_GROUP");
+    if (!v || std::sscanf(v, "%d,%d,%d,%d", &g->lanes, &g->v, &g->blocks, &g->threads) != 4) return false;
+    return (g->v == 1 || g->v == 2 || g->v == 4) && g->blocks >= 1 && g->blocks <= 16 &&
+           (g->blocks & (g->blocks - 1)) == 0 && g->threads >= 32 && g->threads <= 512 && (g->threads & 31) == 0 &&
+           g->lanes >= 1 && g->lanes <= 32 && g->threads % g->lanes == 0;
+}
+
+// The group shape of a batch that was not tuned, v = 0 for the level launches.  Groups win where a level's
+// work is small (W cells of a level times S scenarios) and a launch per level costs more than it: level
+// launches against groups, forward with power + reverse, 5,000 cells / 30 levels S = 1 85 + 146 / 55 + 74 us, S = 64
+// 82 + 101 / 60 + 74; 20,000 / 38 S = 32 104 + 127 / 85 + 104; 50,000 / 44 S = 16 137 + 157 / 116 + 111, S = 96
+// 145 + 186 / 156 + 192; 120,000 / 48 S = 1 132 + 190 / 106 + 133, S = 16 174 + 174 / 176 + 162; 300,000 / 54
+// S = 8 247 + 212 / 258 + 227.  The cluster of 16 blocks takes a level in one round (512 rows / lanes each) where it
+// can, and six such clusters are resident at a time.
+dp::GroupShape group_rule(const dp_design *D, int64_t S) {
+    const int64_t W = D->d.n_cells / (D->d.n_levels > 0 ? D->d.n_levels : 1);
+    if (D->d.n_levels < 1 || W * S > 40000 || W > 6000) return dp::GroupShape{};
+    dp::GroupShape g{8, 1, 16, 512};
+    while (g.lanes > 1 && W * g.lanes > 8192) g.lanes /= 2;
+    while (cdiv(S, (int64_t)g.lanes * g.v) > 6) {
+        if (S % (2 * g.v) == 0 && g.v < 2) g.v *= 2;
+        else if (g.lanes < 32) g.lanes *= 2;
+        else break;
+    }
+    return g;
+}
+
+// the group shape of the staged batch's pass (0 forward, 1 reverse); v = 0: level launches
+dp::GroupShape group_in_use(const dp_design *D, int tr_mode, int pass) {
+    const dp_batch &B = D->batch;
+    dp::GroupShape g;
+    if (parse_group_env(&g) && B.S % g.v == 0) return g;
+    if (B.shape_from_env) return dp::GroupShape{};
+    if (B.tuned_S == B.S && !B.shapes_locked && tr_mode != 2) return pass == 0 ? B.fwd_group : B.bwd_group;
+    return group_rule(D, B.S);
+}
+
 // Autotuner: times the forward and the reverse pass of this design at this S
 // for every candidate shape (CUDA events, best of two after a warm-up) and
-// keeps the fastest of each.  Runs on the staged inputs; the results it
+// keeps the fastest of each; where the rule above takes groups, or nearly, a few group shapes too.  Runs on the staged inputs; the results it
 // leaves are overwritten by the next dp_propagate.
 dp_status tune(dp_design *D) {
     dp_batch &B = D->batch;
     dp_ctx *c = D->ctx;
-    if (parse_shape_env(&B.fwd_shape, &B.bwd_shape)) {
+    B.fwd_group = B.bwd_group = dp::GroupShape{};
+    B.shape_from_env = parse_shape_env(&B.fwd_shape, &B.bwd_shape);
+    if (B.shape_from_env) {
         B.tuned_S = B.S;
         return DP_OK;
     }
@@ -159,6 +200,36 @@ dp_status tune(dp_design *D) {
             }
         }
     }
+    const int64_t W = D->d.n_cells / (D->d.n_levels > 0 ? D->d.n_levels : 1);
+    if (D->d.n_levels > 0 && W * S <= 150000 && W <= 6000) {
+        dp::GroupShape cand[8];
+        int n = 0;
+        for (int lanes : {2, 4, 8, 16})
+            if (W * lanes <= 16384 && cdiv(S, lanes) <= 8) cand[n++] = dp::GroupShape{lanes, 1, 16, 512};
+        if (S % 2 == 0 && cdiv(S, 8) <= 8) cand[n++] = dp::GroupShape{4, 2, 16, 512};
+        if (cdiv(S, 8) <= 18) cand[n++] = dp::GroupShape{8, 1, 8, 512};
+        if (S % 2 == 0 && cdiv(S, 16) <= 18) cand[n++] = dp::GroupShape{8, 2, 8, 512};
+        for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
+            float least = best[pass];
+            for (int i = 0; i < n && e == cudaSuccess; i++) {
+                float t = 1e30f;
+                for (int r = 0; r < 3 && e == cudaSuccess; r++) {
+                    cudaEventRecord(e0, st);
+                    e = pass == 0 ? dp::launch_fwdb_group(D->d, B.b, D->ops, 0, cand[i], st)
+                                  : dp::launch_bwdb_group(D->d, B.b, D->ops, 0, cand[i], st);
+                    cudaEventRecord(e1, st);
+                    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+                    float ms = 0.f;
+                    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+                    if (r > 0 && ms < t) t = ms;
+                }
+                if (e == cudaSuccess && t < least) {
+                    least = t;
+                    (pass == 0 ? B.fwd_group : B.bwd_group) = cand[i];
+                }
+            }
+        }
+    }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -174,6 +245,22 @@ dp_status tune(dp_design *D) {
 }  // namespace
 
 namespace dpi {
+
+cudaError_t batch_forward(dp_design *D, int tr_mode, cudaStream_t s) {
+    dp_batch &B = D->batch;
+    const dp::GroupShape g = group_in_use(D, tr_mode, 0);
+    if (g.v > 0) return dp::launch_fwdb_group(D->d, B.b, D->ops, tr_mode, g, s);
+    dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), tr_mode, B.fwd_shape, s);
+    return cudaGetLastError();
+}
+
+cudaError_t batch_reverse(dp_design *D, int tr_mode, cudaStream_t s) {
+    dp_batch &B = D->batch;
+    const dp::GroupShape g = group_in_use(D, tr_mode, 1);
+    if (g.v > 0) return dp::launch_bwdb_group(D->d, B.b, D->ops, tr_mode, g, s);
+    dp::launch_bwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), tr_mode, B.bwd_shape, s);
+    return cudaGetLastError();
+}
 
 void free_batch(dp_design *D) {
     free_list(D->batch.allocs, D->batch.bytes);
@@ -214,7 +301,8 @@ dp_status batch_propagate(dp_design *D, const dp_config &c) {
         if (s != DP_OK) return s;
     }
     cudaStream_t st = D->ctx->stream;
-    dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), c.tr_mode, B.fwd_shape, st);
+    cudaError_t le = batch_forward(D, c.tr_mode, st);
+    if (le != cudaSuccess) return cuda_err(D->ctx, le, "dp_propagate (batched)");
     dp::launch_powerb(D->d, B.b, c.tr_mode, power_K(c), st);
     dp_status s = launch_check(D->ctx, "dp_propagate (batched)");
     if (s != DP_OK) return s;
@@ -342,7 +430,8 @@ dp_status dp_backward_weighted(dp_design *D, const dp_config *cfg, const double 
     }
     if (e != cudaSuccess) return cuda_err(c, e, "dp_backward_weighted");
     dp::launch_seedb(B.b, power_K(*cfg), wd, st);
-    dp::launch_bwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), cfg->tr_mode, B.bwd_shape, st);
+    e = batch_reverse(D, cfg->tr_mode, st);
+    if (e != cudaSuccess) return cuda_err(c, e, "dp_backward (batched)");
     if ((s = launch_check(c, "dp_backward (batched)")) != DP_OK) return s;
     const bool reduce = cap_reduce != 0;
     const size_t nsS = (size_t)D->d.n_start * (size_t)S;

@@ -33,6 +33,8 @@ struct dp_batch {
     bool fwd_valid = false;
     int fwd_tr_mode = -1;
     dp::BatchShape fwd_shape{128, 1}, bwd_shape{128, 1};
+    dp::GroupShape fwd_group, bwd_group;   // group passes that were faster than the level launches at tuned_S
+    bool shape_from_env = false;   // DP_BATCH_SHAPE fixed the level launches
     int64_t tuned_S = 0;           // S the shapes were tuned for (0: not tuned)
     bool shapes_locked = false;    // keep the shapes whatever S comes (a server fixes them once)
     float tune_ms[2] = {0.f, 0.f}; // best forward / backward time seen by the tuner
@@ -129,6 +131,9 @@ bool capturing(cudaStream_t s);
 void free_batch(dp_design *D);
 // batched halves of dp_propagate, dp_get_power and dp_get_nets (capi_batch.cu)
 dp_status batch_propagate(dp_design *D, const dp_config &c);
+// the forward and the reverse pass of the staged batch (B.S scenarios), by groups or by levels
+cudaError_t batch_forward(dp_design *D, int tr_mode, cudaStream_t s);
+cudaError_t batch_reverse(dp_design *D, int tr_mode, cudaStream_t s);
 dp_status batch_get_power(dp_design *D, int hybrid, double *watts, int on_device);
 dp_status batch_get_nets(dp_design *D, float *sp, float *tr, int on_device);
 // batch buffers for S scenarios plus the host-output staging (synchronises; not under capture)

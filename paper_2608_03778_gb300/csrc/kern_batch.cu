@@ -16,7 +16,7 @@
 // the bytes every gather moves.  The gradient is the model gradient (Sec. III-E,
 // Eq. 7) in binary32, scaled per scenario by a seed K * w_s so that a caller
 // can back-propagate any weighted sum of the scenario powers.
-#include "kern_batch.cuh"
+#include "kern_cells.cuh"
 
 namespace dp {
 namespace {
@@ -38,9 +38,55 @@ __global__ void k_fwdb_start4(const float *__restrict__ sp_in, float2 *pq, int64
     reinterpret_cast<float4 *>(pq + i)[1] = make_float4(a.z, 0.f, a.w, 0.f);
 }
 
+// V consecutive values of a row in 8- or 16-byte accesses
+template <int V>
+__device__ __forceinline__ void row_load(const float2 *src, float2 (&v)[V]) {
+    if constexpr (V == 1) {
+        v[0] = *src;
+    } else {
+#pragma unroll
+        for (int h = 0; h < V / 2; h++) {
+            const float4 t = reinterpret_cast<const float4 *>(src)[h];
+            v[2 * h] = make_float2(t.x, t.y);
+            v[2 * h + 1] = make_float2(t.z, t.w);
+        }
+    }
+}
+template <int V>
+__device__ __forceinline__ void row_store(float2 *dst, const float2 (&v)[V]) {
+    if constexpr (V == 1) {
+        *dst = v[0];
+    } else {
+#pragma unroll
+        for (int h = 0; h < V / 2; h++)
+            reinterpret_cast<float4 *>(dst)[h] = make_float4(v[2 * h].x, v[2 * h].y, v[2 * h + 1].x, v[2 * h + 1].y);
+    }
+}
+template <int V>
+__device__ __forceinline__ void row_add(const float *src, float (&acc)[V]) {
+    if constexpr (V == 1) {
+        acc[0] += *src;
+    } else if constexpr (V == 2) {
+        const float2 t = *reinterpret_cast<const float2 *>(src);
+        acc[0] += t.x, acc[1] += t.y;
+    } else {
+        const float4 t = *reinterpret_cast<const float4 *>(src);
+        acc[0] += t.x, acc[1] += t.y, acc[2] += t.z, acc[3] += t.w;
+    }
+}
+template <int V>
+__device__ __forceinline__ void row_store(float *dst, const float (&v)[V]) {
+    if constexpr (V == 1) *dst = v[0];
+    else if constexpr (V == 2) *reinterpret_cast<float2 *>(dst) = make_float2(v[0], v[1]);
+    else *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// One level, V consecutive scenarios per thread (1, or 2 or 4 with S a multiple of V): each fanin
+// gather is V / 2 16-byte loads of those scenarios' P, so a warp keeps V times the bytes in flight.
+template <int V>
 __global__ void k_fwdb_level(const uint4 *__restrict__ fanin, float2 *pq, int32_t c0, int32_t c1, int64_t ns,
                              int64_t S, OpTable ops) {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t s = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     pdl_trigger();
     if (s >= S) return;
     const int64_t step = (int64_t)gridDim.y * blockDim.y;
@@ -50,10 +96,22 @@ __global__ void k_fwdb_level(const uint4 *__restrict__ fanin, float2 *pq, int32_
     for (int64_t c = cf; c < c1; c += step) {
         if (c != cf) r = fanin[c];
         const uint32_t op = r.x >> 24;
-        const int k = op_arity(ops, op);
-        pair_ff x[4];
-        gather_ffb(pq, r, k, S, s, x);
-        pq[(ns + c) * S + s] = cell_p(k, op_tt(ops, op), x);
+        const uint32_t n[4] = {r.x & kMask24, r.y, r.z, r.w};
+        with_cell(op_arity(ops, op), op_tt(ops, op), [&](const auto f) {
+            constexpr int K = decltype(f)::k;
+            float2 x[K ? K : 1][V], out[V];
+#pragma unroll
+            for (int j = 0; j < K; j++) row_load(pq + (int64_t)n[j] * S + s, x[j]);
+#pragma unroll
+            for (int i = 0; i < V; i++) {
+                pair_ff a[4];
+#pragma unroll
+                for (int j = 0; j < K; j++) a[j] = pair_get(x[j][i]);
+                const ff p = f.prob(a);
+                out[i] = make_float2(p.hi, p.lo);
+            }
+            row_store(pq + (ns + c) * S + s, out);
+        });
     }
 }
 
@@ -69,8 +127,9 @@ __global__ void k_powerb_partials(const float2 *__restrict__ pq, const float *__
                                   int64_t nn, int64_t ns,
                                   int64_t S, int64_t chunk, int nchunks, int tr_mode) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= S) return;
-    const int64_t n0 = (int64_t)blockIdx.y * chunk, n1 = n0 + chunk < nn ? n0 + chunk : nn;
+    const int64_t b = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
+    if (s >= S || b >= nchunks) return;
+    const int64_t n0 = b * chunk, n1 = n0 + chunk < nn ? n0 + chunk : nn;
     ff acc = ff_make(0.f);
     for (int64_t n = n0; n < n1; n += 4) {
         float a[4], c[4];
@@ -95,7 +154,7 @@ __global__ void k_powerb_partials(const float2 *__restrict__ pq, const float *__
             acc = fast_two_sum(t.hi, t.lo + acc.lo);
         }
     }
-    partials[s * nchunks + blockIdx.y] = (double)acc.hi + (double)acc.lo;
+    partials[s * nchunks + b] = (double)acc.hi + (double)acc.lo;
 }
 
 // The same partial sums with four consecutive scenarios per thread (S a
@@ -105,8 +164,9 @@ __global__ void k_powerb_partials4(const float2 *__restrict__ pq, const float *_
                                    const float *__restrict__ cload, const float *__restrict__ dcl, double *partials,
                                    int64_t nn, int64_t ns, int64_t S, int64_t chunk, int nchunks, int tr_mode) {
     const int64_t s = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
-    if (s >= S) return;
-    const int64_t n0 = (int64_t)blockIdx.y * chunk, n1 = n0 + chunk < nn ? n0 + chunk : nn;
+    const int64_t b = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
+    if (s >= S || b >= nchunks) return;
+    const int64_t n0 = b * chunk, n1 = n0 + chunk < nn ? n0 + chunk : nn;
     ff acc[4] = {ff_make(0.f), ff_make(0.f), ff_make(0.f), ff_make(0.f)};
     for (int64_t n = n0; n < n1; n += 2) {
         float a[2][4], c[2][4];
@@ -154,7 +214,7 @@ __global__ void k_powerb_partials4(const float2 *__restrict__ pq, const float *_
             }
     }
 #pragma unroll
-    for (int v = 0; v < 4; v++) partials[(s + v) * nchunks + blockIdx.y] = (double)acc[v].hi + (double)acc[v].lo;
+    for (int v = 0; v < 4; v++) partials[(s + v) * nchunks + b] = (double)acc[v].hi + (double)acc[v].lo;
 }
 
 // one warp per scenario: lane l sums chunks l, l + 32, ... in order, then a fixed shuffle tree
@@ -163,7 +223,14 @@ __global__ void k_sumb_final(const double *__restrict__ partials, int nchunks, i
     const int lane = threadIdx.x & 31;
     if (s >= S) return;
     double acc = 0.0;
-    for (int b = lane; b < nchunks; b += 32) acc += partials[s * nchunks + b];
+    for (int b0 = lane; b0 < nchunks; b0 += 32 * 16) {   // sixteen loads in flight, added in order
+        double v[16];
+#pragma unroll
+        for (int i = 0; i < 16; i++) v[i] = b0 + 32 * i < nchunks ? partials[s * nchunks + b0 + 32 * i] : 0.0;
+#pragma unroll
+        for (int i = 0; i < 16; i++)
+            if (b0 + 32 * i < nchunks) acc += v[i];
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) out[s] = K * acc;
@@ -173,100 +240,16 @@ __global__ void k_seedb(float *ks, const double *__restrict__ w, double K, int64
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s < S) ks[s] = (float)(w ? K * w[s] : K);
 }
-// The same level with V consecutive scenarios per thread (V = 2 or 4, S a
-// multiple of V): each fanin gather is V / 2 16-byte loads of those scenarios'
-// P, so a warp keeps V times the bytes in flight; every (cell, scenario) is
-// computed exactly as above.
-template <int V>
-__global__ void k_fwdb_levelv(const uint4 *__restrict__ fanin, float2 *pq, int32_t c0, int32_t c1, int64_t ns,
-                              int64_t S, OpTable ops) {
-    const int64_t s = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
-    pdl_trigger();
-    if (s >= S) return;
-    const int64_t step = (int64_t)gridDim.y * blockDim.y;
-    const int64_t cf = c0 + (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
-    uint4 r = cf < c1 ? fanin[cf] : make_uint4(0, 0, 0, 0);   // static: before the wait
-    pdl_wait();
-    for (int64_t c = cf; c < c1; c += step) {
-        if (c != cf) r = fanin[c];
-        const uint32_t op = r.x >> 24;
-        const int k = op_arity(ops, op);
-        const uint32_t tt = op_tt(ops, op);
-        const uint32_t n[4] = {r.x & kMask24, r.y, r.z, r.w};
-        float4 v[4][V / 2];
-#pragma unroll
-        for (int j = 0; j < 4; j++)
-#pragma unroll
-            for (int h = 0; h < V / 2; h++)
-                v[j][h] = j < k ? reinterpret_cast<const float4 *>(pq + (int64_t)n[j] * S + s)[h]
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 out[V / 2];
-#pragma unroll
-        for (int h = 0; h < V / 2; h++) {
-            pair_ff x[4], y[4];
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                x[j] = pair_get(make_float2(v[j][h].x, v[j][h].y));
-                y[j] = pair_get(make_float2(v[j][h].z, v[j][h].w));
-            }
-            const float2 a = cell_p(k, tt, x), b = cell_p(k, tt, y);
-            out[h] = make_float4(a.x, a.y, b.x, b.y);
-        }
-#pragma unroll
-        for (int h = 0; h < V / 2; h++) reinterpret_cast<float4 *>(pq + (ns + c) * S + s)[h] = out[h];
-    }
-}
 
 // reverse level: each net's adjoint is its fanout range summed in index order
 // plus its local term d(K_s C 2PQ)/dP = 2 K_s C (Q - P); the cell then writes
-// one contribution per input edge (no atomics)
+// one contribution per input edge (no atomics).  V consecutive scenarios per thread as in the forward level.
+template <int V>
 __global__ void k_bwdb_level(const uint4 *__restrict__ fanin, const int32_t *__restrict__ fptr,
                              const int4 *__restrict__ efpos, const float2 *__restrict__ pq,
                              const float *__restrict__ cload, const float *__restrict__ dcl,
                              const float *__restrict__ ks, float *gfo, int32_t c0, int32_t c1, int64_t ns, int64_t S,
                              OpTable ops) {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    pdl_trigger();
-    if (s >= S) return;
-    const int64_t step = (int64_t)gridDim.y * blockDim.y;
-    const int64_t cf = c0 + (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
-    uint4 rf = cf < c1 ? fanin[cf] : make_uint4(0, 0, 0, 0);   // static: before the wait
-    pdl_wait();
-    const float Ks = ks[s];
-    for (int64_t c = cf; c < c1; c += step) {
-        const int64_t n = ns + c;
-        // everything that does not depend on the fanout sum goes out first, so its loads
-        // overlap the fanout range's
-        const uint4 r = c == cf ? rf : fanin[c];
-        const int4 ep = efpos[c];
-        const int32_t e0 = fptr[n], e1 = fptr[n + 1];
-        const float2 self = pq[n * S + s];
-        const float cl = cl_of(cload, dcl, n, S, s);
-        const uint32_t op = r.x >> 24;
-        const int k = op_arity(ops, op);
-        float p[4], q[4], d[4];
-        gather32(pq, r, k, S, s, p, q);
-        float acc = 0.f;
-        for (int32_t e = e0; e < e1; e++) acc += gfo[(int64_t)e * S + s];
-        const float g = acc + 2.f * Ks * cl * qmp32(self);
-        cell_partials(k, op_tt(ops, op), p, q, d);
-        if (k > 0) gfo[(int64_t)ep.x * S + s] = g * d[0];
-        if (k > 1) gfo[(int64_t)ep.y * S + s] = g * d[1];
-        if (k > 2) gfo[(int64_t)ep.z * S + s] = g * d[2];
-        if (k > 3) gfo[(int64_t)ep.w * S + s] = g * d[3];
-    }
-}
-
-// The same reverse level with V consecutive scenarios per thread (V = 2 or 4,
-// S a multiple of V): 16-byte loads of those scenarios' P, 8- or 16-byte loads
-// and stores of their edge adjoints; every (cell, scenario) is computed
-// exactly as above.
-template <int V>
-__global__ void k_bwdb_levelv(const uint4 *__restrict__ fanin, const int32_t *__restrict__ fptr,
-                              const int4 *__restrict__ efpos, const float2 *__restrict__ pq,
-                              const float *__restrict__ cload, const float *__restrict__ dcl,
-                              const float *__restrict__ ks, float *gfo, int32_t c0, int32_t c1, int64_t ns, int64_t S,
-                              OpTable ops) {
     const int64_t s = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     pdl_trigger();
     if (s >= S) return;
@@ -279,70 +262,46 @@ __global__ void k_bwdb_levelv(const uint4 *__restrict__ fanin, const int32_t *__
     for (int i = 0; i < V; i++) Ks[i] = ks[s + i];
     for (int64_t c = cf; c < c1; c += step) {
         const int64_t n = ns + c;
+        // everything that does not depend on the fanout sum goes out first, so its loads
+        // overlap the fanout range's
         const uint4 r = c == cf ? rf : fanin[c];
         const int4 ep = efpos[c];
         const int32_t e0 = fptr[n], e1 = fptr[n + 1];
         float2 self[V];
-#pragma unroll
-        for (int h = 0; h < V / 2; h++) {
-            const float4 t = reinterpret_cast<const float4 *>(pq + n * S + s)[h];
-            self[2 * h] = make_float2(t.x, t.y);
-            self[2 * h + 1] = make_float2(t.z, t.w);
-        }
+        row_load(pq + n * S + s, self);
         float cl[V];
 #pragma unroll
-        for (int i = 0; i < V; i++) cl[i] = dcl ? cload[n] + dcl[n * S + s + i] : cload[n];
+        for (int i = 0; i < V; i++) cl[i] = cl_of(cload, dcl, n, S, s + i);
         const uint32_t op = r.x >> 24;
-        const int k = op_arity(ops, op);
-        const uint32_t tt = op_tt(ops, op);
         const uint32_t nid[4] = {r.x & kMask24, r.y, r.z, r.w};
-        float4 v[4][V / 2];
-#pragma unroll
-        for (int j = 0; j < 4; j++)
-#pragma unroll
-            for (int h = 0; h < V / 2; h++)
-                v[j][h] = j < k ? reinterpret_cast<const float4 *>(pq + (int64_t)nid[j] * S + s)[h]
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-        float acc[V];
-#pragma unroll
-        for (int i = 0; i < V; i++) acc[i] = 0.f;
-        for (int32_t e = e0; e < e1; e++) {
-            const float *src = gfo + (int64_t)e * S + s;
-            if (V == 4) {
-                const float4 t = *reinterpret_cast<const float4 *>(src);
-                acc[0] += t.x;
-                acc[1 % V] += t.y;
-                acc[2 % V] += t.z;
-                acc[3 % V] += t.w;
-            } else {
-                const float2 t = *reinterpret_cast<const float2 *>(src);
-                acc[0] += t.x;
-                acc[1 % V] += t.y;
-            }
-        }
-        float g[V], d[V][4];
-#pragma unroll
-        for (int i = 0; i < V; i++) {
-            float p[4], q[4];
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const float4 &w = v[j][i / 2];
-                const pair_ff a = pair_get((i & 1) ? make_float2(w.z, w.w) : make_float2(w.x, w.y));
-                p[j] = a.p.hi + a.p.lo;
-                q[j] = a.q.hi + a.q.lo;
-            }
-            g[i] = acc[i] + 2.f * Ks[i] * cl[i] * qmp32(self[i]);
-            cell_partials(k, tt, p, q, d[i]);
-        }
         const int pos[4] = {ep.x, ep.y, ep.z, ep.w};
+        with_cell(op_arity(ops, op), op_tt(ops, op), [&](const auto f) {
+            constexpr int K = decltype(f)::k;
+            float2 x[K ? K : 1][V];
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            if (j >= k) break;
-            float *dst = gfo + (int64_t)pos[j] * S + s;
-            if (V == 4) *reinterpret_cast<float4 *>(dst) = make_float4(g[0] * d[0][j], g[1 % V] * d[1 % V][j],
-                                                                       g[2 % V] * d[2 % V][j], g[3 % V] * d[3 % V][j]);
-            else *reinterpret_cast<float2 *>(dst) = make_float2(g[0] * d[0][j], g[1 % V] * d[1 % V][j]);
-        }
+            for (int j = 0; j < K; j++) row_load(pq + (int64_t)nid[j] * S + s, x[j]);
+            float acc[V];
+#pragma unroll
+            for (int i = 0; i < V; i++) acc[i] = 0.f;
+            for (int32_t e = e0; e < e1; e++) row_add(gfo + (int64_t)e * S + s, acc);
+            float g[K ? K : 1][V];
+#pragma unroll
+            for (int i = 0; i < V; i++) {
+                float p[4], q[4], d[4];
+#pragma unroll
+                for (int j = 0; j < K; j++) {
+                    const pair_ff a = pair_get(x[j][i]);
+                    p[j] = a.p.hi + a.p.lo;
+                    q[j] = a.q.hi + a.q.lo;
+                }
+                f.partials(p, q, d);
+                const float gn = bwdb_adjoint(acc[i], Ks[i], cl[i], self[i]);
+#pragma unroll
+                for (int j = 0; j < K; j++) g[j][i] = __fmul_rn(gn, d[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < K; j++) row_store(gfo + (int64_t)pos[j] * S + s, g[j]);
+        });
     }
 }
 
@@ -361,9 +320,7 @@ __global__ void k_bwdb_start(const int32_t *__restrict__ fptr, const float2 *__r
         const int32_t e0 = fptr[k], e1 = fptr[k + 1];
         float acc = 0.f;
         for (int32_t e = e0; e < e1; e++) acc += gfo[(int64_t)e * S + s];
-        float g = acc;
-        if (tr_mode) g += 2.f * Ks * cl_of(cload, dcl, k, S, s) * qmp32(pq[k * S + s]);
-        gsp[k * S + s] = g;
+        gsp[k * S + s] = tr_mode ? bwdb_adjoint(acc, Ks, cl_of(cload, dcl, k, S, s), pq[k * S + s]) : acc;
     }
 }
 
@@ -406,7 +363,7 @@ __global__ void k_bwdb_start4(const int32_t *__restrict__ fptr, const float2 *__
             const float2 w[4] = {make_float2(u0.x, u0.y), make_float2(u0.z, u0.w), make_float2(u1.x, u1.y),
                                  make_float2(u1.z, u1.w)};
 #pragma unroll
-            for (int v = 0; v < 4; v++) g[v] += 2.f * ksv[v] * cl_of(cload, dcl, k, S, s + v) * qmp32(w[v]);
+            for (int v = 0; v < 4; v++) g[v] = bwdb_adjoint(g[v], ksv[v], cl_of(cload, dcl, k, S, s + v), w[v]);
         }
         *reinterpret_cast<float4 *>(gsp + k * S + s) = make_float4(g[0], g[1], g[2], g[3]);
     }
@@ -613,9 +570,9 @@ void launch_fwdb(const DevDesign &d, const BatchBufs &b, const OpTable &ops, con
         const int32_t c0 = lvl[l - 1], c1 = lvl[l];
         if (c1 <= c0) continue;
         const dim3 g = bgrid(S / v, sh, c1 - c0);
-        if (v == 4) launch_pdl(k_fwdb_levelv<4>, g, blk, s, d.fanin, b.pq, c0, c1, d.n_start, S, ops);
-        else if (v == 2) launch_pdl(k_fwdb_levelv<2>, g, blk, s, d.fanin, b.pq, c0, c1, d.n_start, S, ops);
-        else launch_pdl(k_fwdb_level, g, blk, s, d.fanin, b.pq, c0, c1, d.n_start, S, ops);
+        if (v == 4) launch_pdl(k_fwdb_level<4>, g, blk, s, d.fanin, b.pq, c0, c1, d.n_start, S, ops);
+        else if (v == 2) launch_pdl(k_fwdb_level<2>, g, blk, s, d.fanin, b.pq, c0, c1, d.n_start, S, ops);
+        else launch_pdl(k_fwdb_level<1>, g, blk, s, d.fanin, b.pq, c0, c1, d.n_start, S, ops);
     }
 }
 
@@ -623,14 +580,18 @@ void launch_powerb(const DevDesign &d, const BatchBufs &b, int tr_mode, double K
     const int64_t S = b.S;
     int64_t chunk = 0;
     const int nch = nchunks_of(d.n_nets, &chunk);
-    if (S % 4 == 0)
-        k_powerb_partials4<<<dim3((unsigned)cdiv(S / 4, 128), (unsigned)nch), 128, 0, s>>>(
-            b.pq, tr_mode == 2 ? b.tq : b.tr_in, d.cload, b.dcl, b.partials, d.n_nets, d.n_start, S, chunk, nch,
-            tr_mode);
+    // 128 threads a block over scenarios, or over several chunks where there are fewer (37 scenarios of 21,474
+    // nets: 1,024 blocks of 37 threads before)
+    const int v = S % 4 == 0 ? 4 : 1;
+    const BatchShape sh = fit_shape(BatchShape{128, 1}, S / v);
+    const dim3 g((unsigned)cdiv(S / v, sh.bx), (unsigned)cdiv(nch, sh.by)), blk((unsigned)sh.bx, (unsigned)sh.by);
+    const float *act = tr_mode == 2 ? b.tq : b.tr_in;
+    if (v == 4)
+        k_powerb_partials4<<<g, blk, 0, s>>>(b.pq, act, d.cload, b.dcl, b.partials, d.n_nets, d.n_start, S, chunk, nch,
+                                             tr_mode);
     else
-        k_powerb_partials<<<dim3((unsigned)cdiv(S, 128), (unsigned)nch), 128, 0, s>>>(
-            b.pq, tr_mode == 2 ? b.tq : b.tr_in, d.cload, b.dcl, b.partials, d.n_nets, d.n_start, S, chunk, nch,
-            tr_mode);
+        k_powerb_partials<<<g, blk, 0, s>>>(b.pq, act, d.cload, b.dcl, b.partials, d.n_nets, d.n_start, S, chunk, nch,
+                                            tr_mode);
     k_sumb_final<<<(unsigned)cdiv(S * 32, 256), 256, 0, s>>>(b.partials, nch, S, K, b.power);
 }
 
@@ -654,13 +615,13 @@ void launch_bwdb(const DevDesign &d, const BatchBufs &b, const OpTable &ops, con
         if (c1 <= c0) continue;
         const dim3 g = bgrid(S / v, sh, c1 - c0);
         if (v == 4)
-            launch_pdl(k_bwdb_levelv<4>, g, blk, s, d.fanin, d.fout_ptr, (const int4 *)d.edge_fpos, b.pq, d.cload,
+            launch_pdl(k_bwdb_level<4>, g, blk, s, d.fanin, d.fout_ptr, (const int4 *)d.edge_fpos, b.pq, d.cload,
                        b.dcl, b.ks, b.gfo, c0, c1, d.n_start, S, ops);
         else if (v == 2)
-            launch_pdl(k_bwdb_levelv<2>, g, blk, s, d.fanin, d.fout_ptr, (const int4 *)d.edge_fpos, b.pq, d.cload,
+            launch_pdl(k_bwdb_level<2>, g, blk, s, d.fanin, d.fout_ptr, (const int4 *)d.edge_fpos, b.pq, d.cload,
                        b.dcl, b.ks, b.gfo, c0, c1, d.n_start, S, ops);
         else
-            launch_pdl(k_bwdb_level, g, blk, s, d.fanin, d.fout_ptr, (const int4 *)d.edge_fpos, b.pq, d.cload,
+            launch_pdl(k_bwdb_level<1>, g, blk, s, d.fanin, d.fout_ptr, (const int4 *)d.edge_fpos, b.pq, d.cload,
                        b.dcl, b.ks, b.gfo, c0, c1, d.n_start, S, ops);
     }
     if (d.n_start && S % 4 == 0) {

@@ -13,17 +13,6 @@ __device__ __forceinline__ pair_ff pair_get(const float2 &v) {
     const ff t = fast_two_sum(1.f, -v.x);   // exact: 0 <= P.hi <= 1
     return pair_ff{p, fast_two_sum(t.hi, __fsub_rn(t.lo, v.y))};
 }
-__device__ __forceinline__ float2 p_set(const pair_ff &a) { return make_float2(a.p.hi, a.p.lo); }
-
-__device__ __forceinline__ void gather_ffb(const float2 *pq, const uint4 &r, int k, int64_t S, int64_t s,
-                                           pair_ff (&x)[4]) {
-    const uint32_t n[4] = {r.x & kMask24, r.y, r.z, r.w};
-    float2 v[4];
-#pragma unroll
-    for (int j = 0; j < 4; j++) v[j] = j < k ? pq[(int64_t)n[j] * S + s] : make_float2(0.f, 0.f);
-#pragma unroll
-    for (int j = 0; j < 4; j++) x[j] = pair_get(v[j]);
-}
 
 // P(out = 1) of a cell alone: the multilinear extension of its truth table over
 // the fanin pairs, folded in float-float.  The batched path stores only P and
@@ -48,33 +37,6 @@ __device__ __forceinline__ ff ml_p(uint32_t tt, const pair_ff (&x)[4]) {
     return v[0];
 }
 
-__device__ __forceinline__ float2 cell_p(int k, uint32_t tt, const pair_ff (&x)[4]) {
-    ff p;
-    switch (k) {
-        case 0: p = ff_make((tt & 1u) ? 1.f : 0.f); break;
-        case 1: p = ml_p<1>(tt, x); break;
-        case 2: p = ml_p<2>(tt, x); break;
-        case 3: p = ml_p<3>(tt, x); break;
-        default: p = ml_p<4>(tt, x); break;
-    }
-    return make_float2(p.hi, p.lo);
-}
-
-// binary32 (P, Q) of a cell's inputs for the partial derivatives
-__device__ __forceinline__ void gather32(const float2 *pq, const uint4 &r, int k, int64_t S, int64_t s,
-                                         float (&p)[4], float (&q)[4]) {
-    const uint32_t n[4] = {r.x & kMask24, r.y, r.z, r.w};
-    float2 v[4];
-#pragma unroll
-    for (int j = 0; j < 4; j++) v[j] = j < k ? pq[(int64_t)n[j] * S + s] : make_float2(0.f, 0.f);
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-        const pair_ff a = pair_get(v[j]);
-        p[j] = a.p.hi + a.p.lo;
-        q[j] = a.q.hi + a.q.lo;
-    }
-}
-
 // Q - P of a stored net, rounded once to binary32
 __device__ __forceinline__ float qmp32(const float2 &v) {
     const pair_ff a = pair_get(v);
@@ -90,6 +52,21 @@ __device__ __forceinline__ float alpha32(const float2 *pq, const float *tr_in, i
                                          int64_t s, int tr_mode) {
     if (tr_mode == 2 || (n < ns && tr_mode == 0)) return tr_in[n * S + s];
     return pair_tr(pair_get(pq[n * S + s]));
+}
+
+// a net's adjoint from its fanout sum: plus the local term d(K_s C 2PQ)/dP = 2 K_s C (Q - P), every operation
+// spelled out (no contraction left to the compiler), so that every kernel gives the same bits
+__device__ __forceinline__ float bwdb_adjoint(float acc, float Ks, float cl, const float2 &self) {
+    return fmaf(__fmul_rn(__fmul_rn(2.f, Ks), cl), qmp32(self), acc);
+}
+
+// lag-one weights q(a, b) of a pair and its T: q(1,1) = P - T/2, q(0,0) = P(net=0) - T/2, q(0,1) = q(1,0) = T/2
+__device__ __forceinline__ void lag1_weights(const pair_ff &a, float t, float (&w)[4]) {
+    const float h = 0.5f * t;
+    w[0] = __fsub_rn(a.q.hi + a.q.lo, h);
+    w[1] = h;
+    w[2] = h;
+    w[3] = __fsub_rn(a.p.hi + a.p.lo, h);
 }
 
 // the load of net n in scenario s: C_load plus the scenario's sizing delta (if any)

@@ -1,0 +1,365 @@
+// Batched passes by scenario groups: one launch per pass.  Scenarios do not depend on each other,
+// so a group of them (lanes x V consecutive ones) is walked through all levels by one thread-block
+// cluster (1 to 16 blocks; 1: a single block), with the cluster's barrier between levels, and the
+// groups never wait for each other.  The level launches (kern_batch.cu, kern_lag1.cu) spread every
+// level of all scenarios over the whole grid instead and pay a launch and a drained grid per level.
+//
+// A block is lanes x rows threads: a thread takes V consecutive scenarios of one cell (loads of up
+// to 32 bytes), the lanes of a row the group's scenarios, the rows of all blocks of the cluster
+// consecutive cells of the level.  What other blocks write is read through L2; the static records of
+// a level are loaded between the arrival at the barrier before it and the wait.
+//
+// Every (cell, scenario) is computed by the same code as in the level launches, so the results are
+// bitwise the same in any shape.
+#include <cooperative_groups.h>
+
+#include "kern_cells.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace dp {
+namespace {
+
+constexpr int kGroupThreads = 512;
+
+// V consecutive float2 or float values of a row, through L2
+template <int V>
+struct Row2 {
+    float2 v[V];
+};
+template <int V>
+struct Row1 {
+    float v[V];
+};
+template <int V>
+__device__ __forceinline__ Row2<V> ld2(const float2 *p) {
+    Row2<V> r;
+    if constexpr (V == 1) {
+        r.v[0] = __ldcg(p);
+    } else if constexpr (V == 2) {
+        const float4 t = __ldcg(reinterpret_cast<const float4 *>(p));
+        r.v[0] = make_float2(t.x, t.y), r.v[1] = make_float2(t.z, t.w);
+    } else {
+        asm volatile("ld.global.cg.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=f"(r.v[0].x), "=f"(r.v[0].y), "=f"(r.v[1].x), "=f"(r.v[1].y), "=f"(r.v[2].x), "=f"(r.v[2].y),
+                       "=f"(r.v[3].x), "=f"(r.v[3].y)
+                     : "l"(p)
+                     : "memory");
+    }
+    return r;
+}
+template <int V>
+__device__ __forceinline__ void st2(float2 *p, const Row2<V> &r) {
+    if constexpr (V == 1) {
+        *p = r.v[0];
+    } else if constexpr (V == 2) {
+        *reinterpret_cast<float4 *>(p) = make_float4(r.v[0].x, r.v[0].y, r.v[1].x, r.v[1].y);
+    } else {
+        asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(r.v[0].x), "f"(r.v[0].y),
+                     "f"(r.v[1].x), "f"(r.v[1].y), "f"(r.v[2].x), "f"(r.v[2].y), "f"(r.v[3].x), "f"(r.v[3].y)
+                     : "memory");
+    }
+}
+template <int V>
+__device__ __forceinline__ Row1<V> ld1(const float *p) {
+    Row1<V> r;
+    if constexpr (V == 1) {
+        r.v[0] = __ldcg(p);
+    } else if constexpr (V == 2) {
+        const float2 t = __ldcg(reinterpret_cast<const float2 *>(p));
+        r.v[0] = t.x, r.v[1] = t.y;
+    } else {
+        const float4 t = __ldcg(reinterpret_cast<const float4 *>(p));
+        r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
+    }
+    return r;
+}
+template <int V>
+__device__ __forceinline__ void st1(float *p, const Row1<V> &r) {
+    if constexpr (V == 1) *p = r.v[0];
+    else if constexpr (V == 2) *reinterpret_cast<float2 *>(p) = make_float2(r.v[0], r.v[1]);
+    else *reinterpret_cast<float4 *>(p) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
+}
+
+// this thread's place: scenario, first cell of a level, distance to its next one
+struct Place {
+    int64_t s;
+    int first, stride, C;
+    __device__ __forceinline__ Place(int lanes, int V) {
+        const cg::cluster_group cl = cg::this_cluster();
+        C = (int)cl.num_blocks();
+        const int rows = (int)blockDim.x / lanes, row = (int)threadIdx.x / lanes;
+        s = ((int64_t)((int)blockIdx.x / C) * lanes + (int)threadIdx.x % lanes) * V;
+        first = (int)cl.block_rank() * rows + row;
+        stride = C * rows;
+    }
+    __device__ __forceinline__ void arrive() const {
+        __syncwarp();
+        if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    }
+    __device__ __forceinline__ void wait() const {
+        __syncwarp();
+        if (C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        else __syncthreads();
+    }
+};
+
+template <int V, bool LAG>
+__global__ void __launch_bounds__(kGroupThreads) k_fwdb_group(const uint4 *__restrict__ fanin, float2 *pq, float *tq,
+                                                             const float *__restrict__ sp_in,
+                                                             const float *__restrict__ tr_in,
+                                                             const int32_t *__restrict__ lvl, int L, int64_t ns,
+                                                             int64_t S, int lanes, OpTable ops) {
+    const Place at(lanes, V);
+    const bool on = at.s < S;
+    pq += at.s;
+    if (LAG) tq += at.s;
+    if (on)
+        for (int64_t k = at.first; k < ns; k += at.stride) {
+            const Row1<V> a = ld1<V>(sp_in + k * S + at.s);
+            Row2<V> o;
+#pragma unroll
+            for (int i = 0; i < V; i++) o.v[i] = make_float2(a.v[i], 0.f);
+            st2<V>(pq + k * S, o);
+            if (LAG) st1<V>(tq + k * S, ld1<V>(tr_in + k * S + at.s));
+        }
+    int32_t c1 = lvl[0];
+    for (int l = 1; l <= L; l++) {
+        int32_t c = c1 + at.first;
+        c1 = lvl[l];
+        at.arrive();
+        uint4 r = on && c < c1 ? fanin[c] : make_uint4(0, 0, 0, 0);
+        at.wait();
+        if (!on) continue;
+        while (c < c1) {
+            const uint4 cur = r;
+            float2 *const out = pq + (ns + c) * S;
+            float *const out_t = LAG ? tq + (ns + c) * S : nullptr;
+            c += at.stride;
+            if (c < c1) r = fanin[c];
+            const uint32_t op = cur.x >> 24;
+            const uint32_t n[4] = {cur.x & kMask24, cur.y, cur.z, cur.w};
+            const int k = op_arity(ops, op);
+            Row2<V> x[4], o;
+            Row1<V> t[4], ot;
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (j < k) {
+                    x[j] = ld2<V>(pq + (int64_t)n[j] * S);
+                    if (LAG) t[j] = ld1<V>(tq + (int64_t)n[j] * S);
+                }
+            with_cell(k, op_tt(ops, op), [&](const auto f) {
+                constexpr int K = decltype(f)::k;
+#pragma unroll
+                for (int i = 0; i < V; i++) {
+                    pair_ff a[4];
+                    float w[4][4];
+#pragma unroll
+                    for (int j = 0; j < K; j++) {
+                        a[j] = pair_get(x[j].v[i]);
+                        if (LAG) lag1_weights(a[j], t[j].v[i], w[j]);
+                    }
+                    const ff p = f.prob(a);
+                    o.v[i] = make_float2(p.hi, p.lo);
+                    if (LAG) ot.v[i] = f.toggle(w);
+                }
+            });
+            st2<V>(out, o);
+            if (LAG) st1<V>(out_t, ot);
+        }
+    }
+}
+
+template <int V, bool LAG>
+__global__ void __launch_bounds__(kGroupThreads) k_bwdb_group(
+    const uint4 *__restrict__ fanin, const int32_t *__restrict__ fptr, const int4 *__restrict__ efpos,
+    const float2 *pq, const float *tq, const float *__restrict__ cload, const float *__restrict__ dcl,
+    const float *__restrict__ ks, float *gfo, float2 *gfo2, float *gsp, float *gtr, const int32_t *__restrict__ lvl,
+    int L, int64_t ns, int64_t S, int lanes, int tr_mode, OpTable ops) {
+    const Place at(lanes, V);
+    const bool on = at.s < S;
+    pq += at.s;
+    gsp += at.s;
+    if (dcl) dcl += at.s;
+    if (LAG) tq += at.s, gfo2 += at.s, gtr += at.s;
+    else gfo += at.s;
+    Row1<V> Ks;
+#pragma unroll
+    for (int i = 0; i < V; i++) Ks.v[i] = on ? ks[at.s + i] : 0.f;
+    // the sum of a net's fanout range (P adjoint in a, T adjoint in b), four edges' loads in flight
+    auto fanout = [&](int32_t e0, int32_t e1, Row1<V> &a, Row1<V> &b) {
+#pragma unroll
+        for (int i = 0; i < V; i++) a.v[i] = b.v[i] = 0.f;
+        for (int32_t e = e0; e < e1; e += 4) {
+            Row1<V> u[4];
+            Row2<V> u2[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (e + k < e1) {
+                    if constexpr (LAG) u2[k] = ld2<V>(gfo2 + (int64_t)(e + k) * S);
+                    else u[k] = ld1<V>(gfo + (int64_t)(e + k) * S);
+                }
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (e + k < e1)
+#pragma unroll
+                    for (int i = 0; i < V; i++) {
+                        if constexpr (LAG) a.v[i] += u2[k].v[i].x, b.v[i] += u2[k].v[i].y;
+                        else a.v[i] += u[k].v[i];
+                    }
+        }
+    };
+    auto load_of = [&](int64_t n) {
+        Row1<V> c;
+#pragma unroll
+        for (int i = 0; i < V; i++) c.v[i] = dcl ? cload[n] + dcl[n * S + i] : cload[n];
+        return c;
+    };
+    for (int l = L; l >= 1; l--) {
+        const int32_t c0 = lvl[l - 1], c1 = lvl[l];
+        int32_t c = c0 + at.first;
+        if (l < L) at.arrive();
+        uint4 r = make_uint4(0, 0, 0, 0);
+        int4 ep = make_int4(0, 0, 0, 0);
+        int32_t e0 = 0, e1 = 0;
+        auto record = [&] {
+            if (!on || c >= c1) return;
+            r = fanin[c];
+            ep = efpos[c];
+            e0 = fptr[ns + c];
+            e1 = fptr[ns + c + 1];
+        };
+        record();
+        if (l < L) at.wait();
+        if (!on) continue;
+        while (c < c1) {
+            const uint4 cur = r;
+            const int4 pos4 = ep;
+            const int32_t f0 = e0, f1 = e1;
+            const int64_t n = ns + c;
+            c += at.stride;
+            record();
+            const uint32_t op = cur.x >> 24;
+            const uint32_t nid[4] = {cur.x & kMask24, cur.y, cur.z, cur.w};
+            const int pos[4] = {pos4.x, pos4.y, pos4.z, pos4.w};
+            const int k = op_arity(ops, op);
+            Row2<V> x[4], self;
+            Row1<V> t[4], a, b;
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (j < k) {
+                    x[j] = ld2<V>(pq + (int64_t)nid[j] * S);
+                    if (LAG) t[j] = ld1<V>(tq + (int64_t)nid[j] * S);
+                }
+            if (!LAG) self = ld2<V>(pq + n * S);
+            const Row1<V> cl = load_of(n);
+            fanout(f0, f1, a, b);
+            Row1<V> g[4];
+            Row2<V> g2[4];
+            with_cell(k, op_tt(ops, op), [&](const auto f) {
+                constexpr int K = decltype(f)::k;
+#pragma unroll
+                for (int i = 0; i < V; i++) {
+                    float p[4], q[4], d[4], w[4][4], dp[4], dt[4];
+#pragma unroll
+                    for (int j = 0; j < K; j++) {
+                        const pair_ff v = pair_get(x[j].v[i]);
+                        p[j] = v.p.hi + v.p.lo;
+                        q[j] = v.q.hi + v.q.lo;
+                        if (LAG) lag1_weights(v, t[j].v[i], w[j]);
+                    }
+                    f.partials(p, q, d);
+                    if constexpr (LAG) {
+                        f.toggle_partials(w, dp, dt);
+                        const float gt = fmaf(Ks.v[i], cl.v[i], b.v[i]);
+#pragma unroll
+                        for (int j = 0; j < K; j++)
+                            g2[j].v[i] = make_float2(fmaf(a.v[i], d[j], __fmul_rn(gt, dp[j])), __fmul_rn(gt, dt[j]));
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < K; j++) g[j].v[i] = d[j];
+                    }
+                }
+            });
+            if (!LAG)
+#pragma unroll
+                for (int i = 0; i < V; i++) {
+                    const float gn = bwdb_adjoint(a.v[i], Ks.v[i], cl.v[i], self.v[i]);
+#pragma unroll
+                    for (int j = 0; j < 4; j++) g[j].v[i] = __fmul_rn(gn, g[j].v[i]);
+                }
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (j < k) {
+                    if constexpr (LAG) st2<V>(gfo2 + (int64_t)pos[j] * S, g2[j]);
+                    else st1<V>(gfo + (int64_t)pos[j] * S, g[j]);
+                }
+        }
+    }
+    at.arrive();
+    at.wait();
+    if (!on) return;
+    for (int64_t k = at.first; k < ns; k += at.stride) {
+        Row1<V> a, b;
+        fanout(fptr[k], fptr[k + 1], a, b);
+        if (LAG || tr_mode) {
+            const Row1<V> cl = load_of(k);
+            Row2<V> self;
+            if (!LAG) self = ld2<V>(pq + k * S);
+#pragma unroll
+            for (int i = 0; i < V; i++) {
+                if constexpr (LAG) b.v[i] = fmaf(Ks.v[i], cl.v[i], b.v[i]);
+                else a.v[i] = bwdb_adjoint(a.v[i], Ks.v[i], cl.v[i], self.v[i]);
+            }
+        }
+        st1<V>(gsp + k * S, a);
+        if (LAG) st1<V>(gtr + k * S, b);
+    }
+}
+
+template <class... KArgs, class... Args>
+cudaError_t launch_group(void (*kern)(KArgs...), GroupShape sh, int64_t S, cudaStream_t s, Args... args) {
+    cudaError_t e = cudaSuccess;
+    if (sh.blocks > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    const int64_t per = (int64_t)sh.lanes * sh.v;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((S + per - 1) / per * sh.blocks));
+    cfg.blockDim = dim3((unsigned)sh.threads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)sh.blocks;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
+}  // namespace
+
+cudaError_t launch_fwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
+                              cudaStream_t s) {
+    if (tr_mode == 2 && sh.v == 4) sh.v = 2, sh.lanes *= 2;   // the lag-one state takes two scenarios' registers
+    auto go = [&](auto kern) {
+        return launch_group(kern, sh, b.S, s, d.fanin, b.pq, b.tq, b.sp_in, b.tr_in, d.lvl, d.n_levels, d.n_start, b.S,
+                            sh.lanes, ops);
+    };
+    if (tr_mode == 2) return sh.v >= 2 ? go(k_fwdb_group<2, true>) : go(k_fwdb_group<1, true>);
+    return sh.v == 4 ? go(k_fwdb_group<4, false>) : sh.v == 2 ? go(k_fwdb_group<2, false>) : go(k_fwdb_group<1, false>);
+}
+
+cudaError_t launch_bwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
+                              cudaStream_t s) {
+    if (tr_mode == 2 && sh.v == 4) sh.v = 2, sh.lanes *= 2;
+    auto go = [&](auto kern) {
+        return launch_group(kern, sh, b.S, s, d.fanin, d.fout_ptr, (const int4 *)d.edge_fpos, b.pq, b.tq, d.cload, b.dcl,
+                            b.ks, b.gfo, b.gfo2, b.gsp, b.gtr, d.lvl, d.n_levels, d.n_start, b.S, sh.lanes, tr_mode,
+                            ops);
+    };
+    if (tr_mode == 2) return sh.v >= 2 ? go(k_bwdb_group<2, true>) : go(k_bwdb_group<1, true>);
+    return sh.v == 4 ? go(k_bwdb_group<4, false>) : sh.v == 2 ? go(k_bwdb_group<2, false>) : go(k_bwdb_group<1, false>);
+}
+
+}  // namespace dp

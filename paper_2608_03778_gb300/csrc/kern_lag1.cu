@@ -15,75 +15,10 @@
 // dq/dT = (-1/2, 1/2, 1/2, -1/2).  The reverse pass carries two adjoints per
 // net (of P and of T); edge contributions are float2 in fanout-CSR order, so a
 // net sums one contiguous range, without atomics, as in the other modes.
-#include "kern_batch.cuh"
+#include "kern_cells.cuh"
 
 namespace dp {
 namespace {
-
-// q weights of a stored pair and its T
-__device__ __forceinline__ void lag1_weights(const float2 &pv, float t, float (&w)[4]) {
-    const pair_ff a = pair_get(pv);
-    const float h = 0.5f * t;
-    w[0] = (a.q.hi + a.q.lo) - h;
-    w[1] = h;
-    w[2] = h;
-    w[3] = (a.p.hi + a.p.lo) - h;
-}
-
-// the fold, with input `sub` (if 0 <= sub < K) weighted by dv instead of its own weights
-template <int K>
-__device__ __forceinline__ float lag1_fold(uint32_t tt, const float (&w)[4][4], int sub, const float (&dv)[4]) {
-    constexpr int M = 1 << (2 * K);
-    float v[M];
-#pragma unroll
-    for (int m = 0; m < M; m++) {
-        int a = 0, b = 0;
-#pragma unroll
-        for (int i = 0; i < K; i++) {
-            const int dgt = (m >> (2 * i)) & 3;
-            a |= (dgt >> 1) << i;
-            b |= (dgt & 1) << i;
-        }
-        v[m] = (((tt >> a) ^ (tt >> b)) & 1u) ? 1.f : 0.f;
-    }
-#pragma unroll
-    for (int i = 0; i < K; i++) {
-        float c[4];
-#pragma unroll
-        for (int d = 0; d < 4; d++) c[d] = i == sub ? dv[d] : w[i][d];
-#pragma unroll
-        for (int m = 0; m < (M >> (2 * (i + 1))); m++)
-            v[m] = fmaf(c[3], v[4 * m + 3], fmaf(c[2], v[4 * m + 2], fmaf(c[1], v[4 * m + 1], c[0] * v[4 * m])));
-    }
-    return v[0];
-}
-
-__device__ __forceinline__ float lag1_t(int k, uint32_t tt, const float (&w)[4][4], int sub, const float (&dv)[4]) {
-    switch (k) {
-        case 0: return 0.f;   // a constant never toggles
-        case 1: return lag1_fold<1>(tt, w, sub, dv);
-        case 2: return lag1_fold<2>(tt, w, sub, dv);
-        case 3: return lag1_fold<3>(tt, w, sub, dv);
-        default: return lag1_fold<4>(tt, w, sub, dv);
-    }
-}
-
-__device__ __forceinline__ void gather_lag1(const float2 *pq, const float *tq, const uint4 &r, int k, int64_t S,
-                                            int64_t s, pair_ff (&x)[4], float (&w)[4][4]) {
-    const uint32_t n[4] = {r.x & kMask24, r.y, r.z, r.w};
-    float2 v[4];
-    float t[4];
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-        v[j] = j < k ? pq[(int64_t)n[j] * S + s] : make_float2(0.f, 0.f);
-        t[j] = j < k ? tq[(int64_t)n[j] * S + s] : 0.f;
-    }
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-        x[j] = pair_get(v[j]);
-        lag1_weights(v[j], t[j], w[j]);
-    }
-}
 
 __global__ void k_fwdl_start(const float *__restrict__ sp_in, const float *__restrict__ tr_in, float2 *pq, float *tq,
                              int64_t n) {
@@ -98,7 +33,6 @@ __global__ void k_fwdl_level(const uint4 *__restrict__ fanin, float2 *pq, float 
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     pdl_trigger();
     if (s >= S) return;
-    const float none[4] = {0.f, 0.f, 0.f, 0.f};
     const int64_t step = (int64_t)gridDim.y * blockDim.y;
     const int64_t cf = c0 + (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     const uint4 rf = cf < c1 ? fanin[cf] : make_uint4(0, 0, 0, 0);   // static: before the wait
@@ -106,13 +40,20 @@ __global__ void k_fwdl_level(const uint4 *__restrict__ fanin, float2 *pq, float 
     for (int64_t c = cf; c < c1; c += step) {
         const uint4 r = c == cf ? rf : fanin[c];
         const uint32_t op = r.x >> 24;
-        const int k = op_arity(ops, op);
-        const uint32_t tt = op_tt(ops, op);
-        pair_ff x[4];
-        float w[4][4];
-        gather_lag1(pq, tq, r, k, S, s, x, w);
-        pq[(ns + c) * S + s] = cell_p(k, tt, x);
-        tq[(ns + c) * S + s] = lag1_t(k, tt, w, -1, none);
+        const uint32_t n[4] = {r.x & kMask24, r.y, r.z, r.w};
+        with_cell(op_arity(ops, op), op_tt(ops, op), [&](const auto f) {
+            constexpr int K = decltype(f)::k;
+            pair_ff x[4];
+            float w[4][4];
+#pragma unroll
+            for (int j = 0; j < K; j++) {
+                x[j] = pair_get(pq[(int64_t)n[j] * S + s]);
+                lag1_weights(x[j], tq[(int64_t)n[j] * S + s], w[j]);
+            }
+            const ff p = f.prob(x);
+            pq[(ns + c) * S + s] = make_float2(p.hi, p.lo);
+            tq[(ns + c) * S + s] = f.toggle(w);
+        });
     }
 }
 
@@ -129,8 +70,6 @@ __global__ void k_bwdl_level(const uint4 *__restrict__ fanin, const int32_t *__r
     if (s >= S) return;
     pdl_wait();
     const float Ks = ks[s];
-    const float dP[4] = {-1.f, 0.f, 0.f, 1.f};
-    const float dT[4] = {-0.5f, 0.5f, 0.5f, -0.5f};
     const int64_t step = (int64_t)gridDim.y * blockDim.y;
     for (int64_t c = c0 + (int64_t)blockIdx.y * blockDim.y + threadIdx.y; c < c1; c += step) {
         const int64_t n = ns + c;
@@ -140,28 +79,28 @@ __global__ void k_bwdl_level(const uint4 *__restrict__ fanin, const int32_t *__r
             gp += g.x;
             gt += g.y;
         }
-        gt += Ks * cl_of(cload, dcl, n, S, s);
+        gt = fmaf(Ks, cl_of(cload, dcl, n, S, s), gt);
         const uint4 r = fanin[c];
         const uint32_t op = r.x >> 24;
-        const int k = op_arity(ops, op);
-        const uint32_t tt = op_tt(ops, op);
-        pair_ff x[4];
-        float w[4][4], p[4], q[4], d[4];
-        gather_lag1(pq, tq, r, k, S, s, x, w);
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            p[j] = x[j].p.hi + x[j].p.lo;
-            q[j] = x[j].q.hi + x[j].q.lo;
-        }
-        cell_partials(k, tt, p, q, d);
+        const uint32_t nid[4] = {r.x & kMask24, r.y, r.z, r.w};
         const int4 ep = efpos[c];
         const int pos[4] = {ep.x, ep.y, ep.z, ep.w};
+        with_cell(op_arity(ops, op), op_tt(ops, op), [&](const auto f) {
+            constexpr int K = decltype(f)::k;
+            float w[4][4], p[4], q[4], d[4], dp[4], dt[4];
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            if (j >= k) break;
-            const float dtp = lag1_t(k, tt, w, j, dP), dtt = lag1_t(k, tt, w, j, dT);
-            gfo2[(int64_t)pos[j] * S + s] = make_float2(fmaf(gp, d[j], gt * dtp), gt * dtt);
-        }
+            for (int j = 0; j < K; j++) {
+                const pair_ff v = pair_get(pq[(int64_t)nid[j] * S + s]);
+                lag1_weights(v, tq[(int64_t)nid[j] * S + s], w[j]);
+                p[j] = v.p.hi + v.p.lo;
+                q[j] = v.q.hi + v.q.lo;
+            }
+            f.partials(p, q, d);
+            f.toggle_partials(w, dp, dt);
+#pragma unroll
+            for (int j = 0; j < K; j++)
+                gfo2[(int64_t)pos[j] * S + s] = make_float2(fmaf(gp, d[j], __fmul_rn(gt, dp[j])), __fmul_rn(gt, dt[j]));
+        });
     }
 }
 
@@ -182,7 +121,7 @@ __global__ void k_bwdl_start(const int32_t *__restrict__ fptr, const float *__re
             gt += g.y;
         }
         gsp[k * S + s] = gp;
-        gtr[k * S + s] = gt + Ks * cl_of(cload, dcl, k, S, s);
+        gtr[k * S + s] = fmaf(Ks, cl_of(cload, dcl, k, S, s), gt);
     }
 }
 

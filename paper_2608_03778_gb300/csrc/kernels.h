@@ -187,6 +187,15 @@ void launch_fwdl(const DevDesign &d, const BatchBufs &b, const OpTable &ops, con
                  cudaStream_t s);
 void launch_bwdl(const DevDesign &d, const BatchBufs &b, const OpTable &ops, const int32_t *lvl_host, BatchShape sh,
                  cudaStream_t s);
+// the same passes by scenario groups, one launch each (kern_group.cu): groups of lanes x v scenarios, each on a
+// cluster of `blocks` blocks of `threads` threads (v = 0: not used; S a multiple of v)
+struct GroupShape {
+    int lanes = 0, v = 0, blocks = 0, threads = 0;
+};
+cudaError_t launch_fwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
+                              cudaStream_t s);
+cudaError_t launch_bwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
+                              cudaStream_t s);
 void launch_powerb(const DevDesign &d, const BatchBufs &b, int tr_mode, double K, cudaStream_t s);
 // ks[s] = K * weights[s] (weights NULL: K)
 void launch_seedb(const BatchBufs &b, double K, const double *weights, cudaStream_t s);

@@ -265,12 +265,12 @@ cudaError_t capture_batch_graph(dp_server *srv, Slot *sl, int64_t Sg, bool grad,
     } else {
         dp::launch_transpose(sl->d_in_sp, B.b.sp_in, Sg, ns, st);
         dp::launch_transpose(sl->d_in_tr, B.b.tr_in, Sg, ns, st);
-        dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), c.tr_mode, B.fwd_shape, st);
+        e = batch_forward(D, c.tr_mode, st);
     }
     dp::launch_powerb(D->d, B.b, c.tr_mode, power_K(c), st);
     if (grad) {
         dp::launch_seedb(B.b, power_K(c), nullptr, st);
-        dp::launch_bwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), c.tr_mode, B.bwd_shape, st);
+        if (e == cudaSuccess) e = batch_reverse(D, c.tr_mode, st);
         dp::launch_transpose(B.b.gsp, sl->d_out_sp, ns, Sg, st);
         dp::launch_gradb(D->d, B.b, D->ops, c.tr_mode, false, B.stage, nullptr, nullptr, st);
         dp::launch_transpose(B.stage, sl->d_out_tr, ns, Sg, st);
@@ -278,7 +278,9 @@ cudaError_t capture_batch_graph(dp_server *srv, Slot *sl, int64_t Sg, bool grad,
         dp::launch_transpose(B.stage, sl->d_out_pin, nc, Sg, st);
     }
     cudaMemcpyAsync(sl->h_power, B.b.power, sizeof(double) * (size_t)Sg, cudaMemcpyDeviceToHost, st);
+    const cudaError_t le = e;   // of the passes' own launches
     e = cudaStreamEndCapture(st, &g);
+    if (e == cudaSuccess) e = le;
     if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
     // upload now: the first launch of an executable graph otherwise uploads it, and the
     // worker would pay that (milliseconds for a large design's level chain) inside a batch
@@ -696,8 +698,8 @@ dp_status make_slot(dp_server *srv, const dp_compiled *cp, const float *ref_sp, 
         if (e == cudaSuccess && ns)
             e = cudaMemcpyAsync(B.b.tr_in, sl->d_ref_tr, sizeof(float) * (size_t)ns, cudaMemcpyDeviceToDevice, sl->stream);
         if (e == cudaSuccess) {
-            dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), srv->cfg.analysis.tr_mode, B.fwd_shape, sl->stream);
-            e = cudaMemcpyAsync(sl->d_ref_pq, B.b.pq, sizeof(float2) * (size_t)nn, cudaMemcpyDeviceToDevice, sl->stream);
+            e = batch_forward(D, srv->cfg.analysis.tr_mode, sl->stream);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(sl->d_ref_pq, B.b.pq, sizeof(float2) * (size_t)nn, cudaMemcpyDeviceToDevice, sl->stream);
         }
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(sl->stream);
