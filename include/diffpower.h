@@ -382,8 +382,8 @@ dp_status dp_virus_eval(dp_design *d, const float *sp, int32_t n_scen, uint8_t *
  *   mode 1: the chain rule through Eq. 2, SP adjoint / (2 - 4 SP), |2 - 4 SP| >= 1e-6.
  * scores[n_cells] (may be NULL).  k > 0: the k highest-scoring cell lines, best
  * first, ties by cell index, into top_cells[k] and top_scores[k] (may be NULL);
- * found by a radix select on the device, the candidates ordered on the host
- * (synchronises).  Single-scenario inputs only. */
+ * found by a radix select on the device and ordered there, or on the host when
+ * more than 8,192 cells are at or above the k-th score (synchronises).  Single-scenario inputs only. */
 dp_status dp_sizing_scores(dp_design *d, const dp_config *cfg, int32_t mode, float *scores, int32_t k,
                            int32_t *top_cells, float *top_scores, int on_device);
 

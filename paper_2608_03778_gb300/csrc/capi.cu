@@ -1241,66 +1241,58 @@ dp_status dp_sizing_scores(dp_design *D, const dp_config *cfg, int32_t mode, flo
         return set_err(c, DP_ESTATE, "sizing scores need dp_backward (or dp_step) with the same config");
     DeviceGuard g(c->device);
     cudaStream_t st = c->stream;
-    if (!D->sc_scores) {
-        if ((s = dalloc(D, &D->sc_scores, (size_t)nc)) != DP_OK) return s;
-        if ((s = dalloc(D, &D->sc_idx, (size_t)nc)) != DP_OK) return s;
-        if ((s = dalloc(D, &D->sc_hist, 257)) != DP_OK) return s;
+    const int64_t kk = k < nc ? k : nc;
+    if (!D->sc_tops) {   // the last one
+        if (!D->sc_scores && (s = dalloc(D, &D->sc_scores, (size_t)nc)) != DP_OK) return s;
+        if (!D->sc_idx && (s = dalloc(D, &D->sc_idx, (size_t)nc)) != DP_OK) return s;
+        if (!D->sc_state && (s = dalloc(D, &D->sc_state, (size_t)dp::kSelectWords)) != DP_OK) return s;
+        if (!D->sc_keys && (s = dalloc(D, &D->sc_keys, (size_t)dp::kSelectMax)) != DP_OK) return s;
+        if (!D->sc_top && (s = dalloc(D, &D->sc_top, (size_t)dp::kSelectMax)) != DP_OK) return s;
+        if ((s = dalloc(D, &D->sc_tops, (size_t)dp::kSelectMax)) != DP_OK) return s;
     }
-    dp::launch_scores(D->d, cfg->grad_mode != 0, (float)power_K(*cfg), mode, D->sc_scores, st);
-    if ((s = launch_check(c, "dp_sizing_scores")) != DP_OK) return s;
-    cudaError_t e = cudaSuccess;
-    if (scores && nc)
-        e = cudaMemcpyAsync(scores, D->sc_scores, sizeof(float) * (size_t)nc,
-                            on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st);
+    float *sc = on_device && scores ? scores : D->sc_scores;   // a device caller's array is written in place
+    cudaError_t e = dp::launch_scores(D->d, cfg->grad_mode != 0, (float)power_K(*cfg), mode, sc, D->sc_state, kk, st);
+    if (e == cudaSuccess && scores && nc && !on_device)
+        e = cudaMemcpyAsync(scores, sc, sizeof(float) * (size_t)nc, cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return cuda_err(c, e, "dp_sizing_scores");
-    if (k == 0 || nc == 0) {
+    if (kk == 0) {
         if (!on_device && (e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_err(c, e, "dp_sizing_scores");
         return on_device ? DP_OK : check_device_error(c);
     }
-    const int64_t kk = k < nc ? k : nc;
-    // radix select of the kk-th largest score: 8-bit digits, most significant first
-    uint32_t prefix = 0, mask = 0;
-    int64_t remaining = kk;
-    unsigned hist[256];
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        e = cudaMemsetAsync(D->sc_hist, 0, 256 * sizeof(unsigned), st);
-        if (e == cudaSuccess) dp::launch_radix_hist(D->sc_scores, nc, prefix, mask, shift, D->sc_hist, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(hist, D->sc_hist, sizeof hist, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return cuda_err(c, e, "dp_sizing_scores (select)");
-        int64_t above = 0;
-        int b = 255;
-        for (; b > 0; b--) {
-            if (above + (int64_t)hist[b] >= remaining) break;
-            above += hist[b];
-        }
-        remaining -= above;
-        prefix |= (uint32_t)b << shift;
-        mask |= 0xFFu << shift;
-    }
-    // every cell at or above the threshold (the kk-th score), then exact ordering on the host
+    // the select, and the order of its candidates, into a device caller's arrays if they hold all of them
+    const bool direct = on_device && kk <= dp::kSelectMax;
+    int32_t *top = direct ? top_cells : D->sc_top;
+    float *tops = direct ? top_scores : D->sc_tops;
+    e = dp::launch_select(sc, nc, kk <= dp::kSelectMax ? kk : dp::kSelectMax, D->sc_state, D->sc_idx, D->sc_keys, top, tops,
+                          st);
     unsigned cnt = 0;
-    e = cudaMemsetAsync(D->sc_hist + 256, 0, sizeof(unsigned), st);
-    if (e == cudaSuccess) dp::launch_radix_collect(D->sc_scores, nc, prefix, D->sc_idx, D->sc_hist + 256, nc, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&cnt, D->sc_hist + 256, sizeof cnt, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_err(c, e, "dp_sizing_scores (collect)");
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&cnt, D->sc_state + dp::kSelectWords - 1, sizeof cnt, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && !on_device && kk <= dp::kSelectMax) {
+        e = cudaMemcpyAsync(top_cells, top, sizeof(int32_t) * (size_t)kk, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess && top_scores)
+            e = cudaMemcpyAsync(top_scores, tops, sizeof(float) * (size_t)kk, cudaMemcpyDeviceToHost, st);
+    }
+    if (e != cudaSuccess) return cuda_err(c, e, "dp_sizing_scores (select)");
+    if ((s = check_device_error(c)) != DP_OK) return s;   // synchronises
+    if ((int64_t)cnt < kk) return set_err(c, DP_ECUDA, "top-k selection lost candidates");
+    if (cnt <= (unsigned)dp::kSelectMax) return DP_OK;
+    // more candidates than one block orders (a large k, or many equal scores): exact ordering on the host
     std::vector<int32_t> idx(cnt);
     std::vector<float> all((size_t)nc);
-    if (cnt) e = cudaMemcpy(idx.data(), D->sc_idx, sizeof(int32_t) * cnt, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaMemcpy(all.data(), D->sc_scores, sizeof(float) * (size_t)nc, cudaMemcpyDeviceToHost);
+    e = cudaMemcpy(idx.data(), D->sc_idx, sizeof(int32_t) * cnt, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(all.data(), sc, sizeof(float) * (size_t)nc, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_err(c, e, "dp_sizing_scores (collect)");
     std::sort(idx.begin(), idx.end(), [&](int32_t a, int32_t b) {
         return all[(size_t)a] != all[(size_t)b] ? all[(size_t)a] > all[(size_t)b] : a < b;
     });
-    if ((int64_t)idx.size() < kk) return set_err(c, DP_ECUDA, "top-k selection lost candidates");
     std::vector<float> ts((size_t)kk);
     for (int64_t i = 0; i < kk; i++) ts[(size_t)i] = all[(size_t)idx[(size_t)i]];
     const cudaMemcpyKind kind = on_device ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost;
     e = cudaMemcpy(top_cells, idx.data(), sizeof(int32_t) * (size_t)kk, kind);
     if (e == cudaSuccess && top_scores) e = cudaMemcpy(top_scores, ts.data(), sizeof(float) * (size_t)kk, kind);
     if (e != cudaSuccess) return cuda_err(c, e, "dp_sizing_scores (top)");
-    return check_device_error(c);
+    return DP_OK;
 }
 
 dp_status dp_step_kernels(const dp_design *D, int64_t *k) {

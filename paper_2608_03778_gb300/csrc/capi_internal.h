@@ -74,10 +74,14 @@ struct dp_design {
     float *pc_caps = nullptr;
     int64_t pc_cap = 0;
     cudaEvent_t pc_done = nullptr;
-    // sizing-score scratch (lazy): scores [n_cells], candidates [n_cells], histogram [256] + count
+    // sizing-score scratch (lazy): scores [n_cells], candidates [n_cells], selection state, and for the ordering
+    // the candidates' keys and the ordered cells and scores
     float *sc_scores = nullptr;
     int32_t *sc_idx = nullptr;
-    unsigned *sc_hist = nullptr;
+    unsigned *sc_state = nullptr;
+    unsigned long long *sc_keys = nullptr;
+    int32_t *sc_top = nullptr;
+    float *sc_tops = nullptr;
     dp_batch batch;
     // graph of the whole step for one config
     cudaGraphExec_t graph = nullptr;

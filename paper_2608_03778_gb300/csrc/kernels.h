@@ -237,12 +237,15 @@ void launch_ascent(float *x, const float *g, int64_t n, float eta, cudaStream_t 
 void launch_virus(const DevDesign &d, const OpTable &ops, const int32_t *lvl_host, const float *sp, int64_t S,
                   uint64_t *words, uint8_t *v0, double *partials, double *out, cudaStream_t s);
 
-// sizing score (kern_size.cu): Eq. 8 per cell line, and the radix select of its top k
-void launch_scores(const DevDesign &d, bool hybrid, float K, int mode, float *out, cudaStream_t s);
-void launch_radix_hist(const float *scores, int64_t n, uint32_t prefix, uint32_t mask, int shift, unsigned *hist,
-                       cudaStream_t s);
-void launch_radix_collect(const float *scores, int64_t n, uint32_t thr, int32_t *idx, unsigned *count, int64_t cap,
+// sizing score (kern_size.cu): Eq. 8 per cell line, and the radix select of its top k.  state: kSelectWords words;
+// [kSelectWords - 1] the number of candidates (at or above the k-th score) once launch_select has run, in idx in
+// no order; where they are at most kSelectMax, top and top_scores (may be NULL) hold the k best in order
+constexpr int kSelectWords = 1031;
+constexpr int kSelectMax = 8192;
+cudaError_t launch_scores(const DevDesign &d, bool hybrid, float K, int mode, float *out, unsigned *state, int64_t k,
                           cudaStream_t s);
+cudaError_t launch_select(const float *scores, int64_t n, int64_t k, unsigned *state, int32_t *idx,
+                          unsigned long long *keys, int32_t *top, float *top_scores, cudaStream_t s);
 
 // simulation by slices of lanes and cycles, the live nets in shared memory (kern_slice.cu)
 struct SlicePlan {

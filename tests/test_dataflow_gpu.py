@@ -86,3 +86,27 @@ def test_sliced_simulation_matches_the_others(dp, ctx, library_text, T):  # noqa
                 np.testing.assert_array_equal(got[0][1], other[1])
         finally:
             dp.dp_design_free(d)
+
+
+# one candidate, around one block's sort of 8,192 on both sides, every cell; host and device arrays
+@pytest.mark.parametrize("k", [1, 2, 1000, 8191, 8192, 8193, 12_000])
+@pytest.mark.parametrize("on_device", [0, 1])
+def test_top_k_is_the_full_order(dp, ctx, library_text, k, on_device):  # noqa: F811
+    import torch
+    spec = netgen.NetlistSpec(12_000, 100, 300, 9, 16, 14)
+    sp, tr = netgen.scenario_inputs(spec.n_start, 60)
+    d = dp.dp_design_load(ctx, netgen.netlist_text(spec), library_text)
+    try:
+        cfg = dp.config(grad_mode=0)
+        dp.dp_set_inputs(ctx, d, sp[:, 0].copy(), tr[:, 0].copy())
+        dp.dp_propagate(ctx, d, cfg)
+        dp.dp_backward(ctx, d, cfg)
+        s, top, ts = np.zeros(12_000, np.float32), np.zeros(k, np.int32), np.zeros(k, np.float32)
+        a = [torch.from_numpy(x).cuda() for x in (s, top, ts)] if on_device else [s, top, ts]
+        dp.dp_sizing_scores(ctx, d, cfg, 0, a[0], k, a[1], a[2], on_device)
+        s, top, ts = (x.cpu().numpy() if on_device else x for x in a)
+    finally:
+        dp.dp_design_free(d)
+    want = np.lexsort((np.arange(len(s)), -s))[:k]
+    np.testing.assert_array_equal(top, want.astype(np.int32))
+    np.testing.assert_array_equal(ts, s[want])
