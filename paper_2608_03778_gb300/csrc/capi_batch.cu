@@ -71,6 +71,9 @@ dp_status ensure_batch(dp_design *D, int64_t S) {
     TRYB(balloc(D, &B.b.power, s));
     TRYB(balloc(D, &B.b.ks, s));
     TRYB(balloc(D, &B.weights, s));
+    TRYB(balloc(D, &B.b.state, 8));
+    const cudaError_t e = cudaMemsetAsync(B.b.state, 0, sizeof(uint32_t) * 8, c->stream);
+    if (e != cudaSuccess) return cuda_err(c, e, "batch buffers");
 #undef TRYB
     B.cap = S;
     return DP_OK;
@@ -124,6 +127,13 @@ bool parse_group_env(dp::GroupShape *g) {
            g->lanes >= 1 && g->lanes <= 32 && g->threads % g->lanes == 0;
 }
 
+// DP_BATCH_FLOW = "v": the dataflow passes wherever v divides S
+int flow_env(int64_t S) {
+    const char *v = std::getenv("DP_BATCH_FLOW");
+    const int n = v ? std::atoi(v) : 0;
+    return (n == 1 || n == 2 || n == 4) && S % n == 0 ? n : 0;
+}
+
 // The group shape of a batch that was not tuned, v = 0 for the level launches.  Groups win where a level's
 // work is small (W cells of a level times S scenarios) and a launch per level costs more than it: level
 // launches against groups, forward with power + reverse, 5,000 cells / 30 levels S = 1 85 + 146 / 55 + 74 us, S = 64
@@ -154,20 +164,44 @@ dp::GroupShape group_in_use(const dp_design *D, int tr_mode, int pass) {
     return group_rule(D, B.S);
 }
 
-// Autotuner: times the forward and the reverse pass of this design at this S
-// for every candidate shape (CUDA events, best of two after a warm-up) and
-// keeps the fastest of each; where the rule above takes groups, or nearly, a few group shapes too.  Runs on the staged inputs; the results it
+// scenarios per thread of the staged batch's dataflow pass (0 forward, 1 reverse); 0: not used.  The tuner takes them
+// where they are fastest; the results are bitwise those of the other passes.  (A design without startpoints has no
+// launch that would tell them of a pass by level launches.)
+int flow_in_use(const dp_design *D, int tr_mode, int pass) {
+    const dp_batch &B = D->batch;
+    if (tr_mode == 2 || D->d.n_start == 0) return 0;
+    if (const int v = flow_env(B.S)) return v;
+    dp::GroupShape g;
+    if (B.shape_from_env || parse_group_env(&g) || B.tuned_S != B.S || B.shapes_locked) return 0;
+    return pass == 0 ? B.fwd_flow : B.bwd_flow;
+}
+
+// Scenarios per thread of the dataflow passes of a design with W cells per level: as many as leave whole warps and
+// about a thousand items a level (forward with power + reverse, us, v = 1 / 2 / 4: 120,000 cells / 48 levels S = 512
+// 599 + 834 / 424 + 579 / 348 + 441, S = 64 166 + 136 / 160 + 115 / 168 + 129; 50,000 / 44 S = 128 107 + 121 /
+// 105 + 106 / 104 + 103; 2,000 / 24 S = 512 48 + 48 / 51 + 51 / 53 + 55).
+int flow_v(int64_t S, int64_t W) {
+    for (int v : {4, 2})
+        if (S % v == 0 && S >= 32 * v && W * S >= 1000 * 32 * v) return v;
+    return 1;
+}
+
+// Autotuner: times the forward and the reverse pass of this design at this S (CUDA events) for every candidate shape
+// of the level launches, for the dataflow passes, and for a small batch for a few group shapes, and keeps the
+// fastest of each.  The first shape of a kernel runs once before it is timed; a shape that is
+// more than a tenth slower than the best is not timed twice.  Runs on the staged inputs; the results it
 // leaves are overwritten by the next dp_propagate.
 dp_status tune(dp_design *D) {
     dp_batch &B = D->batch;
     dp_ctx *c = D->ctx;
     B.fwd_group = B.bwd_group = dp::GroupShape{};
+    B.fwd_flow = B.bwd_flow = 0;
     B.shape_from_env = parse_shape_env(&B.fwd_shape, &B.bwd_shape);
     if (B.shape_from_env) {
         B.tuned_S = B.S;
         return DP_OK;
     }
-    const int64_t S = B.S;
+    const int64_t S = B.S, W = D->d.n_cells / (D->d.n_levels > 0 ? D->d.n_levels : 1);
     const int64_t limit = S <= 32 ? 32 : ((S + 31) / 32) * 32;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaEventCreate(&e0);
@@ -177,58 +211,79 @@ dp_status tune(dp_design *D) {
     const double K = power_K(cfg);
     cudaStream_t st = c->stream;
     dp::launch_seedb(B.b, K, nullptr, st);
+    auto timed = [&](const auto &run, bool warm, float best) {
+        float t = 1e30f;
+        for (int r = warm ? 0 : 1; r < 3 && e == cudaSuccess; r++) {
+            cudaEventRecord(e0, st);
+            e = run();
+            cudaEventRecord(e1, st);
+            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+            float ms = 0.f;
+            if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+            if (r > 0 && ms < t) t = ms;
+            if (r > 0 && t > 1.1f * best) break;
+        }
+        return e == cudaSuccess ? t : 1e30f;
+    };
     float best[2] = {1e30f, 1e30f};
     dp::BatchShape pick[2] = {B.fwd_shape, B.bwd_shape};
     for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
         if (pass == 1) dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), 0, pick[0], st);
+        int seen = 0;
         for (const dp::BatchShape &sh : kShapes) {
             if (sh.bx > limit) continue;
-            float t = 1e30f;
-            for (int r = 0; r < 3 && e == cudaSuccess; r++) {
-                cudaEventRecord(e0, st);
-                if (pass == 0) dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), 0, sh, st);
-                else dp::launch_bwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), 0, sh, st);
-                cudaEventRecord(e1, st);
-                e = cudaEventSynchronize(e1);
-                float ms = 0.f;
-                if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-                if (r > 0 && ms < t) t = ms;   // first run warms up
-            }
-            if (e == cudaSuccess && t < best[pass]) {
+            const int v = S % sh.v ? 1 : sh.v;
+            const float t = timed(
+                [&] {
+                    if (pass == 0) dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), 0, sh, st);
+                    else dp::launch_bwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), 0, sh, st);
+                    return cudaSuccess;
+                },
+                (seen & v) == 0, best[pass]);
+            seen |= v;
+            if (t < best[pass]) {
                 best[pass] = t;
                 pick[pass] = sh;
             }
         }
     }
-    const int64_t W = D->d.n_cells / (D->d.n_levels > 0 ? D->d.n_levels : 1);
-    if (D->d.n_levels > 0 && W * S <= 150000 && W <= 6000) {
-        dp::GroupShape cand[8];
-        int n = 0;
-        for (int lanes : {2, 4, 8, 16})
-            if (W * lanes <= 16384 && cdiv(S, lanes) <= 8) cand[n++] = dp::GroupShape{lanes, 1, 16, 512};
-        if (S % 2 == 0 && cdiv(S, 8) <= 8) cand[n++] = dp::GroupShape{4, 2, 16, 512};
-        if (cdiv(S, 8) <= 18) cand[n++] = dp::GroupShape{8, 1, 8, 512};
-        if (S % 2 == 0 && cdiv(S, 16) <= 18) cand[n++] = dp::GroupShape{8, 2, 8, 512};
+    float least[2] = {best[0], best[1]};
+    if (D->d.n_levels > 0 && D->d.n_start > 0)
         for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
-            float least = best[pass];
-            for (int i = 0; i < n && e == cudaSuccess; i++) {
-                float t = 1e30f;
-                for (int r = 0; r < 3 && e == cudaSuccess; r++) {
-                    cudaEventRecord(e0, st);
-                    e = pass == 0 ? dp::launch_fwdb_group(D->d, B.b, D->ops, 0, cand[i], st)
-                                  : dp::launch_bwdb_group(D->d, B.b, D->ops, 0, cand[i], st);
-                    cudaEventRecord(e1, st);
-                    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-                    float ms = 0.f;
-                    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-                    if (r > 0 && ms < t) t = ms;
-                }
-                if (e == cudaSuccess && t < least) {
-                    least = t;
-                    (pass == 0 ? B.fwd_group : B.bwd_group) = cand[i];
-                }
+            const int v = flow_v(S, W);
+            const float t = timed(   // the first run also brings the arrays to rest
+                [&] {
+                    return pass == 0 ? dp::launch_fwdb_flow(D->d, B.b, D->ops, v, c->sm_count, st)
+                                     : dp::launch_bwdb_flow(D->d, B.b, D->ops, 0, v, D->n_edges * B.cap, c->sm_count, st);
+                },
+                true, least[pass]);
+            if (t < least[pass]) {
+                least[pass] = t;
+                (pass == 0 ? B.fwd_flow : B.bwd_flow) = v;
             }
         }
+    // groups: from eight scenarios the dataflow passes were faster at every size
+    if (D->d.n_levels > 0 && S < 8 && W * S <= 150000 && W <= 6000) {
+        dp::GroupShape cand[4];
+        int n = 0;
+        for (int lanes : {2, 4})
+            if (W * lanes <= 16384) cand[n++] = dp::GroupShape{lanes, 1, 16, 512};
+        if (W * 8 <= 16384) cand[n++] = dp::GroupShape{8, 1, 16, 512};
+        cand[n++] = dp::GroupShape{8, 1, 8, 512};
+        for (int pass = 0; pass < 2 && e == cudaSuccess; pass++)
+            for (int i = 0; i < n; i++) {
+                const float t = timed(
+                    [&] {
+                        return pass == 0 ? dp::launch_fwdb_group(D->d, B.b, D->ops, 0, cand[i], st)
+                                         : dp::launch_bwdb_group(D->d, B.b, D->ops, 0, cand[i], st);
+                    },
+                    i == 0, least[pass]);
+                if (t < least[pass]) {
+                    least[pass] = t;
+                    (pass == 0 ? B.fwd_group : B.bwd_group) = cand[i];
+                    (pass == 0 ? B.fwd_flow : B.bwd_flow) = 0;
+                }
+            }
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
@@ -248,6 +303,8 @@ namespace dpi {
 
 cudaError_t batch_forward(dp_design *D, int tr_mode, cudaStream_t s) {
     dp_batch &B = D->batch;
+    const int v = flow_in_use(D, tr_mode, 0);
+    if (v > 0) return dp::launch_fwdb_flow(D->d, B.b, D->ops, v, D->ctx->sm_count, s);
     const dp::GroupShape g = group_in_use(D, tr_mode, 0);
     if (g.v > 0) return dp::launch_fwdb_group(D->d, B.b, D->ops, tr_mode, g, s);
     dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), tr_mode, B.fwd_shape, s);
@@ -256,6 +313,8 @@ cudaError_t batch_forward(dp_design *D, int tr_mode, cudaStream_t s) {
 
 cudaError_t batch_reverse(dp_design *D, int tr_mode, cudaStream_t s) {
     dp_batch &B = D->batch;
+    const int v = flow_in_use(D, tr_mode, 1);
+    if (v > 0) return dp::launch_bwdb_flow(D->d, B.b, D->ops, tr_mode, v, D->n_edges * B.cap, D->ctx->sm_count, s);
     const dp::GroupShape g = group_in_use(D, tr_mode, 1);
     if (g.v > 0) return dp::launch_bwdb_group(D->d, B.b, D->ops, tr_mode, g, s);
     dp::launch_bwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), tr_mode, B.bwd_shape, s);

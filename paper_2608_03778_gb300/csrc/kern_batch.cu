@@ -23,15 +23,17 @@ namespace {
 
 __host__ __device__ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-__global__ void k_fwdb_start(const float *__restrict__ sp_in, float2 *pq, int64_t n) {
+__global__ void k_fwdb_start(const float *__restrict__ sp_in, float2 *pq, int64_t n, uint32_t *state) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) state[0] = 0u;   // no dataflow pass wrote these
     if (i >= n) return;
     pq[i] = make_float2(sp_in[i], 0.f);
 }
 
 // the same, four values per thread (n a multiple of 4): one 16-byte load, two 16-byte stores
-__global__ void k_fwdb_start4(const float *__restrict__ sp_in, float2 *pq, int64_t n) {
+__global__ void k_fwdb_start4(const float *__restrict__ sp_in, float2 *pq, int64_t n, uint32_t *state) {
     const int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    if (i == 0) state[0] = 0u;
     if (i >= n) return;
     const float4 a = *reinterpret_cast<const float4 *>(sp_in + i);
     reinterpret_cast<float4 *>(pq + i)[0] = make_float4(a.x, 0.f, a.y, 0.f);
@@ -97,7 +99,7 @@ __global__ void k_fwdb_level(const uint4 *__restrict__ fanin, float2 *pq, int32_
         if (c != cf) r = fanin[c];
         const uint32_t op = r.x >> 24;
         const uint32_t n[4] = {r.x & kMask24, r.y, r.z, r.w};
-        with_cell(op_arity(ops, op), op_tt(ops, op), [&](const auto f) {
+        with_cell(ops.e[op], [&](const auto f) {
             constexpr int K = decltype(f)::k;
             float2 x[K ? K : 1][V], out[V];
 #pragma unroll
@@ -122,99 +124,74 @@ __global__ void k_fwdb_level(const uint4 *__restrict__ fanin, float2 *pq, int32_
 // P = 1; about 1e-7 relative per term) and adds it with TwoSum into a
 // float-float sum (about 48 significant bits), so the FP64 pipe, slow on this
 // part, sees one conversion per chunk instead of several operations per term.
+// V consecutive scenarios per thread (S a multiple of V), kPowerNets nets' loads in flight before their terms are
+// added in net order.
+template <class R, class T>
+__device__ __forceinline__ R read_row(const T *p) {   // through L1: a few scenarios' rows share its lines
+    R r;
+    constexpr int n = sizeof(R) / sizeof(float);
+    float *const o = reinterpret_cast<float *>(&r);
+    const float *const a = reinterpret_cast<const float *>(p);
+    if constexpr (n == 1) {
+        o[0] = a[0];
+    } else if constexpr (n == 2) {
+        const float2 t = *reinterpret_cast<const float2 *>(a);
+        o[0] = t.x, o[1] = t.y;
+    } else {
+#pragma unroll
+        for (int i = 0; i < n; i += 4) {
+            const float4 t = *reinterpret_cast<const float4 *>(a + i);
+            o[i] = t.x, o[i + 1] = t.y, o[i + 2] = t.z, o[i + 3] = t.w;
+        }
+    }
+    return r;
+}
+template <int V>
 __global__ void k_powerb_partials(const float2 *__restrict__ pq, const float *__restrict__ tr_in,
                                   const float *__restrict__ cload, const float *__restrict__ dcl, double *partials,
-                                  int64_t nn, int64_t ns,
-                                  int64_t S, int64_t chunk, int nchunks, int tr_mode) {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+                                  int64_t nn, int64_t ns, int64_t S, int64_t chunk, int nchunks, int tr_mode) {
+    const int64_t s = V * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     const int64_t b = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     if (s >= S || b >= nchunks) return;
+    constexpr int kPowerNets = V == 1 ? 8 : 4;
     const int64_t n0 = b * chunk, n1 = n0 + chunk < nn ? n0 + chunk : nn;
-    ff acc = ff_make(0.f);
-    for (int64_t n = n0; n < n1; n += 4) {
-        float a[4], c[4];
+    ff acc[V];
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
+    for (int v = 0; v < V; v++) acc[v] = ff_make(0.f);
+    auto stored = [&](int64_t m) { return tr_mode == 2 || (m < ns && tr_mode == 0); };   // its TR, not its P
+    for (int64_t n = n0; n < n1; n += kPowerNets) {
+        Row2<V> w[kPowerNets];
+        Row1<V> t[kPowerNets], d[kPowerNets];
+        float c[kPowerNets];
+#pragma unroll
+        for (int i = 0; i < kPowerNets; i++) {
             const int64_t m = n + i;
-            a[i] = 0.f;
-            c[i] = 0.f;
-            if (m < n1) {
-                if (tr_mode == 2 || (m < ns && tr_mode == 0)) {
-                    a[i] = tr_in[m * S + s];
-                } else {
-                    const pair_ff pr = pair_get(pq[m * S + s]);
-                    a[i] = 2.f * (pr.p.hi + pr.p.lo) * (pr.q.hi + pr.q.lo);
-                }
-                c[i] = cl_of(cload, dcl, m, S, s);
-            }
+            if (m >= n1) continue;
+            if (stored(m)) t[i] = read_row<Row1<V>>(tr_in + m * S + s);
+            else w[i] = read_row<Row2<V>>(pq + m * S + s);
+            if (dcl) d[i] = read_row<Row1<V>>(dcl + m * S + s);
+            c[i] = cload[m];
         }
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-            const ff t = two_sum(acc.hi, a[i] * c[i]);
-            acc = fast_two_sum(t.hi, t.lo + acc.lo);
+        for (int i = 0; i < kPowerNets; i++) {
+            if (n + i >= n1) continue;
+            const bool st = stored(n + i);
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                float a;
+                if (st) {
+                    a = t[i].v[v];
+                } else {
+                    const pair_ff pr = pair_get(w[i].v[v]);
+                    a = 2.f * (pr.p.hi + pr.p.lo) * (pr.q.hi + pr.q.lo);
+                }
+                const ff u = two_sum(acc[v].hi, a * (dcl ? c[i] + d[i].v[v] : c[i]));
+                acc[v] = fast_two_sum(u.hi, u.lo + acc[v].lo);
+            }
         }
     }
-    partials[s * nchunks + b] = (double)acc.hi + (double)acc.lo;
-}
-
-// The same partial sums with four consecutive scenarios per thread (S a
-// multiple of 4): one 32-byte load of their P per net, four accumulators, each
-// scenario's terms added in the same net order as above (bitwise the same).
-__global__ void k_powerb_partials4(const float2 *__restrict__ pq, const float *__restrict__ tr_in,
-                                   const float *__restrict__ cload, const float *__restrict__ dcl, double *partials,
-                                   int64_t nn, int64_t ns, int64_t S, int64_t chunk, int nchunks, int tr_mode) {
-    const int64_t s = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
-    const int64_t b = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
-    if (s >= S || b >= nchunks) return;
-    const int64_t n0 = b * chunk, n1 = n0 + chunk < nn ? n0 + chunk : nn;
-    ff acc[4] = {ff_make(0.f), ff_make(0.f), ff_make(0.f), ff_make(0.f)};
-    for (int64_t n = n0; n < n1; n += 2) {
-        float a[2][4], c[2][4];
 #pragma unroll
-        for (int i = 0; i < 2; i++) {
-            const int64_t m = n + i;
-#pragma unroll
-            for (int v = 0; v < 4; v++) a[i][v] = c[i][v] = 0.f;
-            if (m < n1) {
-                if (tr_mode == 2 || (m < ns && tr_mode == 0)) {
-                    const float4 t = *reinterpret_cast<const float4 *>(tr_in + m * S + s);
-                    a[i][0] = t.x;
-                    a[i][1] = t.y;
-                    a[i][2] = t.z;
-                    a[i][3] = t.w;
-                } else {
-                    const float4 u0 = reinterpret_cast<const float4 *>(pq + m * S + s)[0];
-                    const float4 u1 = reinterpret_cast<const float4 *>(pq + m * S + s)[1];
-                    const float2 w[4] = {make_float2(u0.x, u0.y), make_float2(u0.z, u0.w), make_float2(u1.x, u1.y),
-                                         make_float2(u1.z, u1.w)};
-#pragma unroll
-                    for (int v = 0; v < 4; v++) {
-                        const pair_ff pr = pair_get(w[v]);
-                        a[i][v] = 2.f * (pr.p.hi + pr.p.lo) * (pr.q.hi + pr.q.lo);
-                    }
-                }
-                if (dcl) {
-                    const float4 t = *reinterpret_cast<const float4 *>(dcl + m * S + s);
-                    c[i][0] = cload[m] + t.x;
-                    c[i][1] = cload[m] + t.y;
-                    c[i][2] = cload[m] + t.z;
-                    c[i][3] = cload[m] + t.w;
-                } else {
-#pragma unroll
-                    for (int v = 0; v < 4; v++) c[i][v] = cload[m];
-                }
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 2; i++)
-#pragma unroll
-            for (int v = 0; v < 4; v++) {
-                const ff t = two_sum(acc[v].hi, a[i][v] * c[i][v]);
-                acc[v] = fast_two_sum(t.hi, t.lo + acc[v].lo);
-            }
-    }
-#pragma unroll
-    for (int v = 0; v < 4; v++) partials[(s + v) * nchunks + b] = (double)acc[v].hi + (double)acc[v].lo;
+    for (int v = 0; v < V; v++) partials[(s + v) * nchunks + b] = (double)acc[v].hi + (double)acc[v].lo;
 }
 
 // one warp per scenario: lane l sums chunks l, l + 32, ... in order, then a fixed shuffle tree
@@ -275,7 +252,7 @@ __global__ void k_bwdb_level(const uint4 *__restrict__ fanin, const int32_t *__r
         const uint32_t op = r.x >> 24;
         const uint32_t nid[4] = {r.x & kMask24, r.y, r.z, r.w};
         const int pos[4] = {ep.x, ep.y, ep.z, ep.w};
-        with_cell(op_arity(ops, op), op_tt(ops, op), [&](const auto f) {
+        with_cell(ops.e[op], [&](const auto f) {
             constexpr int K = decltype(f)::k;
             float2 x[K ? K : 1][V];
 #pragma unroll
@@ -309,11 +286,13 @@ __global__ void k_bwdb_level(const uint4 *__restrict__ fanin, const int32_t *__r
 __global__ void k_bwdb_start(const int32_t *__restrict__ fptr, const float2 *__restrict__ pq,
                              const float *__restrict__ cload, const float *__restrict__ dcl,
                              const float *__restrict__ ks,
-                             const float *__restrict__ gfo, float *gsp, int64_t ns, int64_t S, int tr_mode) {
+                             const float *__restrict__ gfo, float *gsp, int64_t ns, int64_t S, int tr_mode,
+                             uint32_t *state) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     pdl_trigger();
     if (s >= S) return;
     pdl_wait();
+    if (s == 0 && blockIdx.y == 0 && threadIdx.y == 0) state[2] = 0u;   // gfo holds values
     const float Ks = ks[s];
     const int64_t step = (int64_t)gridDim.y * blockDim.y;
     for (int64_t k = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; k < ns; k += step) {
@@ -330,11 +309,12 @@ __global__ void k_bwdb_start(const int32_t *__restrict__ fptr, const float2 *__r
 __global__ void k_bwdb_start4(const int32_t *__restrict__ fptr, const float2 *__restrict__ pq,
                               const float *__restrict__ cload, const float *__restrict__ dcl,
                               const float *__restrict__ ks, const float *__restrict__ gfo, float *gsp, int64_t ns,
-                              int64_t S, int tr_mode) {
+                              int64_t S, int tr_mode, uint32_t *state) {
     const int64_t s = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
     pdl_trigger();
     if (s >= S) return;
     pdl_wait();
+    if (s == 0 && blockIdx.y == 0 && threadIdx.y == 0) state[2] = 0u;
     const float4 Ks = *reinterpret_cast<const float4 *>(ks + s);
     const int64_t step = (int64_t)gridDim.y * blockDim.y;
     for (int64_t k = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; k < ns; k += step) {
@@ -463,7 +443,7 @@ __global__ void k_netb_user(const float2 *__restrict__ pq, const float *__restri
     for (int64_t u = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; u < nn; u += step) {
         const int64_t n = net_of_user[u];
         if (sp_out) {
-            const float2 v = pq[n * S + s];
+            const float2 v = untag(pq[n * S + s]);
             sp_out[u * S + s] = v.x + v.y;
         }
         if (tr_out) tr_out[u * S + s] = alpha32(pq, tr_in, n, ns, S, s, tr_mode);
@@ -560,9 +540,9 @@ void launch_fwdb(const DevDesign &d, const BatchBufs &b, const OpTable &ops, con
     }
     const int64_t S = b.S;
     if (d.n_start && (d.n_start * S) % 4 == 0)
-        k_fwdb_start4<<<(unsigned)cdiv(d.n_start * S / 4, 256), 256, 0, s>>>(b.sp_in, b.pq, d.n_start * S);
+        k_fwdb_start4<<<(unsigned)cdiv(d.n_start * S / 4, 256), 256, 0, s>>>(b.sp_in, b.pq, d.n_start * S, b.state);
     else if (d.n_start)
-        k_fwdb_start<<<(unsigned)cdiv(d.n_start * S, 256), 256, 0, s>>>(b.sp_in, b.pq, d.n_start * S);
+        k_fwdb_start<<<(unsigned)cdiv(d.n_start * S, 256), 256, 0, s>>>(b.sp_in, b.pq, d.n_start * S, b.state);
     const int v = scen_per_thread(sh, S);
     sh = fit_shape(sh, S / v);
     const dim3 blk((unsigned)sh.bx, (unsigned)sh.by);
@@ -580,18 +560,22 @@ void launch_powerb(const DevDesign &d, const BatchBufs &b, int tr_mode, double K
     const int64_t S = b.S;
     int64_t chunk = 0;
     const int nch = nchunks_of(d.n_nets, &chunk);
-    // 128 threads a block over scenarios, or over several chunks where there are fewer (37 scenarios of 21,474
-    // nets: 1,024 blocks of 37 threads before)
-    const int v = S % 4 == 0 ? 4 : 1;
-    const BatchShape sh = fit_shape(BatchShape{128, 1}, S / v);
-    const dim3 g((unsigned)cdiv(S / v, sh.bx), (unsigned)cdiv(nch, sh.by)), blk((unsigned)sh.bx, (unsigned)sh.by);
+    const int v = S % 4 == 0 && S >= 256 ? 4 : S % 2 == 0 && S >= 128 ? 2 : 1;
+    // 65,536 threads and more take two or four scenarios each (forward with power, us, v = 1 / 2 / 4: 50,000 cells x 256
+    // 226 / 218 / 207, 120,000 x 64 155 / 166 / 177), and fewer go into smaller blocks, for every SM to have some
+    // (2,000,000 x 2: 587 with blocks of 128, 484 so)
+    int width = 1, bx = 1;
+    while (width < 128 && (int64_t)width * 608 < nch * (S / v)) width <<= 1;
+    while (bx < width && bx * v < S) bx <<= 1;
+    const int by = width / bx;
+    const dim3 g((unsigned)cdiv(S / v, bx), (unsigned)cdiv(nch, by)), blk((unsigned)bx, (unsigned)by);
     const float *act = tr_mode == 2 ? b.tq : b.tr_in;
-    if (v == 4)
-        k_powerb_partials4<<<g, blk, 0, s>>>(b.pq, act, d.cload, b.dcl, b.partials, d.n_nets, d.n_start, S, chunk, nch,
-                                             tr_mode);
-    else
-        k_powerb_partials<<<g, blk, 0, s>>>(b.pq, act, d.cload, b.dcl, b.partials, d.n_nets, d.n_start, S, chunk, nch,
-                                            tr_mode);
+    auto go = [&](auto kern) {
+        kern<<<g, blk, 0, s>>>(b.pq, act, d.cload, b.dcl, b.partials, d.n_nets, d.n_start, S, chunk, nch, tr_mode);
+    };
+    if (v == 4) go(k_powerb_partials<4>);
+    else if (v == 2) go(k_powerb_partials<2>);
+    else go(k_powerb_partials<1>);
     k_sumb_final<<<(unsigned)cdiv(S * 32, 256), 256, 0, s>>>(b.partials, nch, S, K, b.power);
 }
 
@@ -627,10 +611,10 @@ void launch_bwdb(const DevDesign &d, const BatchBufs &b, const OpTable &ops, con
     if (d.n_start && S % 4 == 0) {
         const BatchShape s4 = fit_shape(BatchShape{128, 1, 4}, S / 4);
         launch_pdl(k_bwdb_start4, bgrid(S / 4, s4, d.n_start), dim3((unsigned)s4.bx, (unsigned)s4.by), s, d.fout_ptr,
-                   b.pq, d.cload, b.dcl, b.ks, b.gfo, b.gsp, d.n_start, S, tr_mode);
+                   b.pq, d.cload, b.dcl, b.ks, b.gfo, b.gsp, d.n_start, S, tr_mode, b.state);
     } else if (d.n_start) {
         launch_pdl(k_bwdb_start, bgrid(S, sh1, d.n_start), dim3((unsigned)sh1.bx, (unsigned)sh1.by), s, d.fout_ptr,
-                   b.pq, d.cload, b.dcl, b.ks, b.gfo, b.gsp, d.n_start, S, tr_mode);
+                   b.pq, d.cload, b.dcl, b.ks, b.gfo, b.gsp, d.n_start, S, tr_mode, b.state);
     }
 }
 

@@ -7,8 +7,16 @@ namespace dp {
 
 __host__ __device__ inline int64_t bcdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// Bit 30 of a stored P's low part is no part of it (clear for |P| < 2^25): the dataflow passes tag what they
+// write with it.
+constexpr uint32_t kTagBit = 0x40000000u;
+__device__ __forceinline__ float2 untag(const float2 &v) {
+    return make_float2(v.x, __uint_as_float(__float_as_uint(v.y) & ~kTagBit));
+}
+
 // the stored float-float P of a net and its pair (P, 1 - P)
-__device__ __forceinline__ pair_ff pair_get(const float2 &v) {
+__device__ __forceinline__ pair_ff pair_get(const float2 &stored) {
+    const float2 v = untag(stored);
     const ff p{v.x, v.y};
     const ff t = fast_two_sum(1.f, -v.x);   // exact: 0 <= P.hi <= 1
     return pair_ff{p, fast_two_sum(t.hi, __fsub_rn(t.lo, v.y))};

@@ -14,22 +14,28 @@ namespace dp {
 // ---- P(out = 1) in float-float: a fold whose operands may be known to be 0 or 1
 enum Known { kZero, kOne, kAny };
 
+// Q a + P b: fold_pq without the operations that a known operand makes exact, and the others in its order, so the
+// result is fold_pq's to the last bit
 template <int A, int B>
-__device__ __forceinline__ ff fold_known(const pair_ff &x, const ff &a, const ff &b) {   // Q a + P b
+__device__ __forceinline__ ff fold_known(const pair_ff &x, const ff &a, const ff &b) {
     if (A == kZero && B == kZero) return ff_make(0.f);
-    if (A == kOne && B == kOne) return ff_make(1.f);
     if (A == kZero && B == kOne) return x.p;
     if (A == kOne && B == kZero) return x.q;
     if (A == kAny && B == kAny) return fold_pq(x, a, b);
     if (A == kZero) return ff_mul(x.p, b);
     if (B == kZero) return ff_mul(x.q, a);
+    if (A == kOne && B == kOne) {   // Q + P, 1 to about 4e-15
+        const ff u = two_sum(x.q.hi, x.p.hi);
+        return fast_two_sum(u.hi, __fadd_rn(__fadd_rn(u.lo, x.q.lo), x.p.lo));
+    }
     const ff &s = A == kOne ? x.q : x.p, &f = A == kOne ? x.p : x.q, &g = A == kOne ? b : a;   // s + f g
     const float t = __fmul_rn(f.hi, g.hi);
     const ff u = two_sum(s.hi, t);
     float lo = __fadd_rn(u.lo, fmaf(f.hi, g.hi, -t));
-    lo = __fadd_rn(lo, s.lo);
+    if (A == kOne) lo = __fadd_rn(lo, s.lo);
     lo = fmaf(f.hi, g.lo, lo);
     lo = fmaf(f.lo, g.hi, lo);
+    if (B == kOne) lo = __fadd_rn(lo, s.lo);
     return fast_two_sum(u.hi, lo);
 }
 
@@ -37,7 +43,7 @@ template <uint32_t TT, int I, int M>
 struct ProbNode {   // inputs 0 .. I folded, entry M of what is left
     using A = ProbNode<TT, I - 1, 2 * M>;
     using B = ProbNode<TT, I - 1, 2 * M + 1>;
-    static constexpr int kind = A::kind == B::kind && A::kind != kAny ? A::kind : kAny;
+    static constexpr int kind = A::kind == kZero && B::kind == kZero ? kZero : kAny;
     __device__ __forceinline__ static ff val(const pair_ff (&x)[4]) {
         return fold_known<A::kind, B::kind>(x[I], A::val(x), B::val(x));
     }
@@ -219,33 +225,201 @@ struct CellAny {
 // Calls f with the cell's function; consecutive cells of a level mostly share theirs, so a warp takes one
 // branch.  f is inlined 22 times: it computes, and loads and stores stay outside.
 template <class F>
-__device__ __forceinline__ void with_cell(int k, uint32_t tt, const F &f) {
-    switch ((uint32_t)k << 16 | tt) {
-        case 0x10001u: return f(CellFn<1, 0x1u>{});    // INV
-        case 0x10002u: return f(CellFn<1, 0x2u>{});    // BUF
-        case 0x20008u: return f(CellFn<2, 0x8u>{});    // AND2
-        case 0x20007u: return f(CellFn<2, 0x7u>{});    // NAND2
-        case 0x2000Eu: return f(CellFn<2, 0xEu>{});    // OR2
-        case 0x20001u: return f(CellFn<2, 0x1u>{});    // NOR2
-        case 0x20006u: return f(CellFn<2, 0x6u>{});    // XOR2
-        case 0x20009u: return f(CellFn<2, 0x9u>{});    // XNOR2
-        case 0x30080u: return f(CellFn<3, 0x80u>{});   // AND3
-        case 0x3007Fu: return f(CellFn<3, 0x7Fu>{});   // NAND3
-        case 0x300FEu: return f(CellFn<3, 0xFEu>{});   // OR3
-        case 0x30001u: return f(CellFn<3, 0x01u>{});   // NOR3
-        case 0x30007u: return f(CellFn<3, 0x07u>{});   // AOI21
-        case 0x300F8u: return f(CellFn<3, 0xF8u>{});   // AO21
-        case 0x3001Fu: return f(CellFn<3, 0x1Fu>{});   // OAI21
-        case 0x300E0u: return f(CellFn<3, 0xE0u>{});   // OA21
-        case 0x300E2u: return f(CellFn<3, 0xE2u>{});   // MUX2
-        default: break;
+__device__ __forceinline__ void with_cell(uint32_t e, const F &f) {
+    switch ((e >> 19) & 31u) {
+#define DP_CELL(I, K, TT) case I: return f(CellFn<K, TT>{});
+        DP_CELL_CLASSES(DP_CELL)
+#undef DP_CELL
+        case 18: return f(CellAny<0>{e & 0xFFFFu});
+        case 19: return f(CellAny<1>{e & 0xFFFFu});
+        case 20: return f(CellAny<2>{e & 0xFFFFu});
+        case 21: return f(CellAny<3>{e & 0xFFFFu});
+        default: return f(CellAny<4>{e & 0xFFFFu});
     }
-    switch (k) {
-        case 0: return f(CellAny<0>{tt});
-        case 1: return f(CellAny<1>{tt});
-        case 2: return f(CellAny<2>{tt});
-        case 3: return f(CellAny<3>{tt});
-        default: return f(CellAny<4>{tt});
+}
+
+// ---- rows of V consecutive scenarios
+
+// row n of an array of S columns: one multiply-add
+template <class T>
+__device__ __forceinline__ T *row_at(T *base, uint32_t n, uint32_t S) {
+    return reinterpret_cast<T *>(reinterpret_cast<uint64_t>(base) + (uint64_t)n * (uint64_t)(S * (uint32_t)sizeof(T)));
+}
+
+// V consecutive float2 or float values of a row, through L2
+template <int V>
+struct Row2 {
+    float2 v[V];
+};
+template <int V>
+struct Row1 {
+    float v[V];
+};
+template <int V>
+__device__ __forceinline__ Row2<V> ld2(const float2 *p) {
+    Row2<V> r;
+    if constexpr (V == 1) {
+        r.v[0] = __ldcg(p);
+    } else if constexpr (V == 2) {
+        const float4 t = __ldcg(reinterpret_cast<const float4 *>(p));
+        r.v[0] = make_float2(t.x, t.y), r.v[1] = make_float2(t.z, t.w);
+    } else {
+        asm volatile("ld.global.cg.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=f"(r.v[0].x), "=f"(r.v[0].y), "=f"(r.v[1].x), "=f"(r.v[1].y), "=f"(r.v[2].x), "=f"(r.v[2].y),
+                       "=f"(r.v[3].x), "=f"(r.v[3].y)
+                     : "l"(p)
+                     : "memory");
+    }
+    return r;
+}
+template <int V>
+__device__ __forceinline__ void st2(float2 *p, const Row2<V> &r) {
+    if constexpr (V == 1) {
+        *p = r.v[0];
+    } else if constexpr (V == 2) {
+        *reinterpret_cast<float4 *>(p) = make_float4(r.v[0].x, r.v[0].y, r.v[1].x, r.v[1].y);
+    } else {
+        asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(r.v[0].x), "f"(r.v[0].y),
+                     "f"(r.v[1].x), "f"(r.v[1].y), "f"(r.v[2].x), "f"(r.v[2].y), "f"(r.v[3].x), "f"(r.v[3].y)
+                     : "memory");
+    }
+}
+template <int V>
+__device__ __forceinline__ Row1<V> ld1(const float *p) {
+    Row1<V> r;
+    if constexpr (V == 1) {
+        r.v[0] = __ldcg(p);
+    } else if constexpr (V == 2) {
+        const float2 t = __ldcg(reinterpret_cast<const float2 *>(p));
+        r.v[0] = t.x, r.v[1] = t.y;
+    } else {
+        const float4 t = __ldcg(reinterpret_cast<const float4 *>(p));
+        r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
+    }
+    return r;
+}
+template <int V>
+__device__ __forceinline__ void st1(float *p, const Row1<V> &r) {
+    if constexpr (V == 1) *p = r.v[0];
+    else if constexpr (V == 2) *reinterpret_cast<float2 *>(p) = make_float2(r.v[0], r.v[1]);
+    else *reinterpret_cast<float4 *>(p) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
+}
+
+// P (LAG: and T) of a cell of table entry e from its inputs' rows; get(j, x, t) reads input j's
+template <int V, bool LAG, class G>
+__device__ __forceinline__ void cell_value(uint32_t e, const G &get, Row2<V> &o, Row1<V> &ot) {
+    with_cell(e, [&](const auto f) {
+        constexpr int K = decltype(f)::k;
+        Row2<V> x[4];
+        Row1<V> t[4];
+#pragma unroll
+        for (int j = 0; j < K; j++) get(j, x[j], t[j]);
+#pragma unroll
+        for (int i = 0; i < V; i++) {
+            pair_ff a[4];
+            float w[4][4];
+#pragma unroll
+            for (int j = 0; j < K; j++) {
+                a[j] = pair_get(x[j].v[i]);
+                if (LAG) lag1_weights(a[j], t[j].v[i], w[j]);
+            }
+            const ff p = f.prob(a);
+            o.v[i] = make_float2(p.hi, p.lo);
+            if (LAG) ot.v[i] = f.toggle(w);
+        }
+    });
+}
+
+// What a cell adds to its inputs' adjoints, from the fanout sums a (LAG: and b, of T) of its net: g, LAG: (of P, of T)
+// in g2.  self: the net's own P, cl: its load.
+template <int V, bool LAG>
+__device__ __forceinline__ void cell_adjoints(uint32_t e, const Row2<V> (&x)[4],
+                                              const Row1<V> (&t)[4], const Row2<V> &self, const Row1<V> &Ks,
+                                              const Row1<V> &cl, const Row1<V> &a, const Row1<V> &b, Row1<V> (&g)[4],
+                                              Row2<V> (&g2)[4]) {
+    with_cell(e, [&](const auto f) {
+        constexpr int K = decltype(f)::k;
+#pragma unroll
+        for (int i = 0; i < V; i++) {
+            float p[4], q[4], d[4], w[4][4];
+#pragma unroll
+            for (int j = 0; j < K; j++) {
+                const pair_ff v = pair_get(x[j].v[i]);
+                p[j] = v.p.hi + v.p.lo;
+                q[j] = v.q.hi + v.q.lo;
+                if (LAG) lag1_weights(v, t[j].v[i], w[j]);
+            }
+            f.partials(p, q, d);
+            if constexpr (LAG) {
+                float dp[4], dt[4];
+                f.toggle_partials(w, dp, dt);
+                const float gt = fmaf(Ks.v[i], cl.v[i], b.v[i]);
+#pragma unroll
+                for (int j = 0; j < K; j++)
+                    g2[j].v[i] = make_float2(fmaf(a.v[i], d[j], __fmul_rn(gt, dp[j])), __fmul_rn(gt, dt[j]));
+            } else {
+#pragma unroll
+                for (int j = 0; j < K; j++) g[j].v[i] = d[j];
+            }
+        }
+    });
+    if (!LAG)
+#pragma unroll
+        for (int i = 0; i < V; i++) {
+            const float gn = bwdb_adjoint(a.v[i], Ks.v[i], cl.v[i], self.v[i]);
+#pragma unroll
+            for (int j = 0; j < 4; j++) g[j].v[i] = __fmul_rn(gn, g[j].v[i]);
+        }
+}
+
+// the partial derivatives of a cell's P with respect to its inputs' (get(j) reads input j)
+template <int V, class G>
+__device__ __forceinline__ void cell_partials(uint32_t e, const G &get, Row1<V> (&d)[4]) {
+    with_cell(e, [&](const auto f) {
+        constexpr int K = decltype(f)::k;
+        Row2<V> x[4];
+#pragma unroll
+        for (int j = 0; j < K; j++) x[j] = get(j);
+#pragma unroll
+        for (int i = 0; i < V; i++) {
+            float p[4], q[4], g[4];
+#pragma unroll
+            for (int j = 0; j < K; j++) {
+                const pair_ff v = pair_get(x[j].v[i]);
+                p[j] = v.p.hi + v.p.lo;
+                q[j] = v.q.hi + v.q.lo;
+            }
+            f.partials(p, q, g);
+#pragma unroll
+            for (int j = 0; j < K; j++) d[j].v[i] = g[j];
+        }
+    });
+}
+
+// the sums over a net's fanout range [e0, e1) in index order, four edges' loads in flight: the adjoints of P in a, LAG:
+// of T in b
+template <int V, bool LAG>
+__device__ __forceinline__ void fanout_sum(const float *gfo, const float2 *gfo2, int32_t e0, int32_t e1, uint32_t S,
+                                           Row1<V> &a, Row1<V> &b) {
+#pragma unroll
+    for (int i = 0; i < V; i++) a.v[i] = b.v[i] = 0.f;
+    for (int32_t e = e0; e < e1; e += 4) {
+        Row1<V> u[4];
+        Row2<V> u2[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (e + k < e1) {
+                if constexpr (LAG) u2[k] = ld2<V>(row_at(gfo2, (uint32_t)(e + k), S));
+                else u[k] = ld1<V>(row_at(gfo, (uint32_t)(e + k), S));
+            }
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (e + k < e1)
+#pragma unroll
+                for (int i = 0; i < V; i++) {
+                    if constexpr (LAG) a.v[i] += u2[k].v[i].x, b.v[i] += u2[k].v[i].y;
+                    else a.v[i] += u[k].v[i];
+                }
     }
 }
 

@@ -22,65 +22,6 @@ namespace {
 
 constexpr int kGroupThreads = 512;
 
-// V consecutive float2 or float values of a row, through L2
-template <int V>
-struct Row2 {
-    float2 v[V];
-};
-template <int V>
-struct Row1 {
-    float v[V];
-};
-template <int V>
-__device__ __forceinline__ Row2<V> ld2(const float2 *p) {
-    Row2<V> r;
-    if constexpr (V == 1) {
-        r.v[0] = __ldcg(p);
-    } else if constexpr (V == 2) {
-        const float4 t = __ldcg(reinterpret_cast<const float4 *>(p));
-        r.v[0] = make_float2(t.x, t.y), r.v[1] = make_float2(t.z, t.w);
-    } else {
-        asm volatile("ld.global.cg.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=f"(r.v[0].x), "=f"(r.v[0].y), "=f"(r.v[1].x), "=f"(r.v[1].y), "=f"(r.v[2].x), "=f"(r.v[2].y),
-                       "=f"(r.v[3].x), "=f"(r.v[3].y)
-                     : "l"(p)
-                     : "memory");
-    }
-    return r;
-}
-template <int V>
-__device__ __forceinline__ void st2(float2 *p, const Row2<V> &r) {
-    if constexpr (V == 1) {
-        *p = r.v[0];
-    } else if constexpr (V == 2) {
-        *reinterpret_cast<float4 *>(p) = make_float4(r.v[0].x, r.v[0].y, r.v[1].x, r.v[1].y);
-    } else {
-        asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(r.v[0].x), "f"(r.v[0].y),
-                     "f"(r.v[1].x), "f"(r.v[1].y), "f"(r.v[2].x), "f"(r.v[2].y), "f"(r.v[3].x), "f"(r.v[3].y)
-                     : "memory");
-    }
-}
-template <int V>
-__device__ __forceinline__ Row1<V> ld1(const float *p) {
-    Row1<V> r;
-    if constexpr (V == 1) {
-        r.v[0] = __ldcg(p);
-    } else if constexpr (V == 2) {
-        const float2 t = __ldcg(reinterpret_cast<const float2 *>(p));
-        r.v[0] = t.x, r.v[1] = t.y;
-    } else {
-        const float4 t = __ldcg(reinterpret_cast<const float4 *>(p));
-        r.v[0] = t.x, r.v[1] = t.y, r.v[2] = t.z, r.v[3] = t.w;
-    }
-    return r;
-}
-template <int V>
-__device__ __forceinline__ void st1(float *p, const Row1<V> &r) {
-    if constexpr (V == 1) *p = r.v[0];
-    else if constexpr (V == 2) *reinterpret_cast<float2 *>(p) = make_float2(r.v[0], r.v[1]);
-    else *reinterpret_cast<float4 *>(p) = make_float4(r.v[0], r.v[1], r.v[2], r.v[3]);
-}
-
 // this thread's place: scenario, first cell of a level, distance to its next one
 struct Place {
     int64_t s;
@@ -109,8 +50,9 @@ __global__ void __launch_bounds__(kGroupThreads) k_fwdb_group(const uint4 *__res
                                                              const float *__restrict__ sp_in,
                                                              const float *__restrict__ tr_in,
                                                              const int32_t *__restrict__ lvl, int L, int64_t ns,
-                                                             int64_t S, int lanes, OpTable ops) {
+                                                             int64_t S, int lanes, OpTable ops, uint32_t *state) {
     const Place at(lanes, V);
+    if (blockIdx.x == 0 && threadIdx.x == 0) state[0] = 0u;   // no dataflow pass wrote these
     const bool on = at.s < S;
     pq += at.s;
     if (LAG) tq += at.s;
@@ -148,22 +90,8 @@ __global__ void __launch_bounds__(kGroupThreads) k_fwdb_group(const uint4 *__res
                     x[j] = ld2<V>(pq + (int64_t)n[j] * S);
                     if (LAG) t[j] = ld1<V>(tq + (int64_t)n[j] * S);
                 }
-            with_cell(k, op_tt(ops, op), [&](const auto f) {
-                constexpr int K = decltype(f)::k;
-#pragma unroll
-                for (int i = 0; i < V; i++) {
-                    pair_ff a[4];
-                    float w[4][4];
-#pragma unroll
-                    for (int j = 0; j < K; j++) {
-                        a[j] = pair_get(x[j].v[i]);
-                        if (LAG) lag1_weights(a[j], t[j].v[i], w[j]);
-                    }
-                    const ff p = f.prob(a);
-                    o.v[i] = make_float2(p.hi, p.lo);
-                    if (LAG) ot.v[i] = f.toggle(w);
-                }
-            });
+            cell_value<V, LAG>(
+                ops.e[op], [&](int j, Row2<V> &xj, Row1<V> &tj) { xj = x[j], tj = t[j]; }, o, ot);
             st2<V>(out, o);
             if (LAG) st1<V>(out_t, ot);
         }
@@ -175,8 +103,9 @@ __global__ void __launch_bounds__(kGroupThreads) k_bwdb_group(
     const uint4 *__restrict__ fanin, const int32_t *__restrict__ fptr, const int4 *__restrict__ efpos,
     const float2 *pq, const float *tq, const float *__restrict__ cload, const float *__restrict__ dcl,
     const float *__restrict__ ks, float *gfo, float2 *gfo2, float *gsp, float *gtr, const int32_t *__restrict__ lvl,
-    int L, int64_t ns, int64_t S, int lanes, int tr_mode, OpTable ops) {
+    int L, int64_t ns, int64_t S, int lanes, int tr_mode, OpTable ops, uint32_t *state) {
     const Place at(lanes, V);
+    if (!LAG && blockIdx.x == 0 && threadIdx.x == 0) state[2] = 0u;   // gfo will hold values
     const bool on = at.s < S;
     pq += at.s;
     gsp += at.s;
@@ -186,29 +115,6 @@ __global__ void __launch_bounds__(kGroupThreads) k_bwdb_group(
     Row1<V> Ks;
 #pragma unroll
     for (int i = 0; i < V; i++) Ks.v[i] = on ? ks[at.s + i] : 0.f;
-    // the sum of a net's fanout range (P adjoint in a, T adjoint in b), four edges' loads in flight
-    auto fanout = [&](int32_t e0, int32_t e1, Row1<V> &a, Row1<V> &b) {
-#pragma unroll
-        for (int i = 0; i < V; i++) a.v[i] = b.v[i] = 0.f;
-        for (int32_t e = e0; e < e1; e += 4) {
-            Row1<V> u[4];
-            Row2<V> u2[4];
-#pragma unroll
-            for (int k = 0; k < 4; k++)
-                if (e + k < e1) {
-                    if constexpr (LAG) u2[k] = ld2<V>(gfo2 + (int64_t)(e + k) * S);
-                    else u[k] = ld1<V>(gfo + (int64_t)(e + k) * S);
-                }
-#pragma unroll
-            for (int k = 0; k < 4; k++)
-                if (e + k < e1)
-#pragma unroll
-                    for (int i = 0; i < V; i++) {
-                        if constexpr (LAG) a.v[i] += u2[k].v[i].x, b.v[i] += u2[k].v[i].y;
-                        else a.v[i] += u[k].v[i];
-                    }
-        }
-    };
     auto load_of = [&](int64_t n) {
         Row1<V> c;
 #pragma unroll
@@ -253,41 +159,10 @@ __global__ void __launch_bounds__(kGroupThreads) k_bwdb_group(
                 }
             if (!LAG) self = ld2<V>(pq + n * S);
             const Row1<V> cl = load_of(n);
-            fanout(f0, f1, a, b);
+            fanout_sum<V, LAG>(gfo, gfo2, f0, f1, (uint32_t)S, a, b);
             Row1<V> g[4];
             Row2<V> g2[4];
-            with_cell(k, op_tt(ops, op), [&](const auto f) {
-                constexpr int K = decltype(f)::k;
-#pragma unroll
-                for (int i = 0; i < V; i++) {
-                    float p[4], q[4], d[4], w[4][4], dp[4], dt[4];
-#pragma unroll
-                    for (int j = 0; j < K; j++) {
-                        const pair_ff v = pair_get(x[j].v[i]);
-                        p[j] = v.p.hi + v.p.lo;
-                        q[j] = v.q.hi + v.q.lo;
-                        if (LAG) lag1_weights(v, t[j].v[i], w[j]);
-                    }
-                    f.partials(p, q, d);
-                    if constexpr (LAG) {
-                        f.toggle_partials(w, dp, dt);
-                        const float gt = fmaf(Ks.v[i], cl.v[i], b.v[i]);
-#pragma unroll
-                        for (int j = 0; j < K; j++)
-                            g2[j].v[i] = make_float2(fmaf(a.v[i], d[j], __fmul_rn(gt, dp[j])), __fmul_rn(gt, dt[j]));
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < K; j++) g[j].v[i] = d[j];
-                    }
-                }
-            });
-            if (!LAG)
-#pragma unroll
-                for (int i = 0; i < V; i++) {
-                    const float gn = bwdb_adjoint(a.v[i], Ks.v[i], cl.v[i], self.v[i]);
-#pragma unroll
-                    for (int j = 0; j < 4; j++) g[j].v[i] = __fmul_rn(gn, g[j].v[i]);
-                }
+            cell_adjoints<V, LAG>(ops.e[op], x, t, self, Ks, cl, a, b, g, g2);
 #pragma unroll
             for (int j = 0; j < 4; j++)
                 if (j < k) {
@@ -301,7 +176,7 @@ __global__ void __launch_bounds__(kGroupThreads) k_bwdb_group(
     if (!on) return;
     for (int64_t k = at.first; k < ns; k += at.stride) {
         Row1<V> a, b;
-        fanout(fptr[k], fptr[k + 1], a, b);
+        fanout_sum<V, LAG>(gfo, gfo2, fptr[k], fptr[k + 1], (uint32_t)S, a, b);
         if (LAG || tr_mode) {
             const Row1<V> cl = load_of(k);
             Row2<V> self;
@@ -344,7 +219,7 @@ cudaError_t launch_fwdb_group(const DevDesign &d, const BatchBufs &b, const OpTa
     if (tr_mode == 2 && sh.v == 4) sh.v = 2, sh.lanes *= 2;   // the lag-one state takes two scenarios' registers
     auto go = [&](auto kern) {
         return launch_group(kern, sh, b.S, s, d.fanin, b.pq, b.tq, b.sp_in, b.tr_in, d.lvl, d.n_levels, d.n_start, b.S,
-                            sh.lanes, ops);
+                            sh.lanes, ops, b.state);
     };
     if (tr_mode == 2) return sh.v >= 2 ? go(k_fwdb_group<2, true>) : go(k_fwdb_group<1, true>);
     return sh.v == 4 ? go(k_fwdb_group<4, false>) : sh.v == 2 ? go(k_fwdb_group<2, false>) : go(k_fwdb_group<1, false>);
@@ -356,7 +231,7 @@ cudaError_t launch_bwdb_group(const DevDesign &d, const BatchBufs &b, const OpTa
     auto go = [&](auto kern) {
         return launch_group(kern, sh, b.S, s, d.fanin, d.fout_ptr, (const int4 *)d.edge_fpos, b.pq, b.tq, d.cload, b.dcl,
                             b.ks, b.gfo, b.gfo2, b.gsp, b.gtr, d.lvl, d.n_levels, d.n_start, b.S, sh.lanes, tr_mode,
-                            ops);
+                            ops, b.state);
     };
     if (tr_mode == 2) return sh.v >= 2 ? go(k_bwdb_group<2, true>) : go(k_bwdb_group<1, true>);
     return sh.v == 4 ? go(k_bwdb_group<4, false>) : sh.v == 2 ? go(k_bwdb_group<2, false>) : go(k_bwdb_group<1, false>);

@@ -21,8 +21,9 @@ namespace dp {
 namespace {
 
 __global__ void k_fwdl_start(const float *__restrict__ sp_in, const float *__restrict__ tr_in, float2 *pq, float *tq,
-                             int64_t n) {
+                             int64_t n, uint32_t *state) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) state[0] = 0u;   // no dataflow pass wrote these
     if (i >= n) return;
     pq[i] = make_float2(sp_in[i], 0.f);
     tq[i] = tr_in[i];
@@ -41,7 +42,7 @@ __global__ void k_fwdl_level(const uint4 *__restrict__ fanin, float2 *pq, float 
         const uint4 r = c == cf ? rf : fanin[c];
         const uint32_t op = r.x >> 24;
         const uint32_t n[4] = {r.x & kMask24, r.y, r.z, r.w};
-        with_cell(op_arity(ops, op), op_tt(ops, op), [&](const auto f) {
+        with_cell(ops.e[op], [&](const auto f) {
             constexpr int K = decltype(f)::k;
             pair_ff x[4];
             float w[4][4];
@@ -85,7 +86,7 @@ __global__ void k_bwdl_level(const uint4 *__restrict__ fanin, const int32_t *__r
         const uint32_t nid[4] = {r.x & kMask24, r.y, r.z, r.w};
         const int4 ep = efpos[c];
         const int pos[4] = {ep.x, ep.y, ep.z, ep.w};
-        with_cell(op_arity(ops, op), op_tt(ops, op), [&](const auto f) {
+        with_cell(ops.e[op], [&](const auto f) {
             constexpr int K = decltype(f)::k;
             float w[4][4], p[4], q[4], d[4], dp[4], dt[4];
 #pragma unroll
@@ -131,7 +132,7 @@ void launch_fwdl(const DevDesign &d, const BatchBufs &b, const OpTable &ops, con
                  cudaStream_t s) {
     const int64_t S = b.S;
     if (d.n_start)
-        k_fwdl_start<<<(unsigned)bcdiv(d.n_start * S, 256), 256, 0, s>>>(b.sp_in, b.tr_in, b.pq, b.tq, d.n_start * S);
+        k_fwdl_start<<<(unsigned)bcdiv(d.n_start * S, 256), 256, 0, s>>>(b.sp_in, b.tr_in, b.pq, b.tq, d.n_start * S, b.state);
     sh = fit_shape(sh, S);
     const dim3 blk((unsigned)sh.bx, (unsigned)sh.by);
     for (int l = 1; l <= d.n_levels; l++) {

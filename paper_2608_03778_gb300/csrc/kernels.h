@@ -6,8 +6,22 @@
 
 namespace dp {
 
+// The functions whose truth tables are compiled into the batched passes (kern_cells.cuh): class, inputs, table.
+// Any other function of k inputs: class 18 + k.
+#define DP_CELL_CLASSES(X)                                                                                     \
+    X(1, 1, 0x1u) X(2, 1, 0x2u)                                                           /* INV BUF */         \
+    X(3, 2, 0x8u) X(4, 2, 0x7u) X(5, 2, 0xEu) X(6, 2, 0x1u) X(7, 2, 0x6u) X(8, 2, 0x9u)   /* AND..XNOR, 2 */    \
+    X(9, 3, 0x80u) X(10, 3, 0x7Fu) X(11, 3, 0xFEu) X(12, 3, 0x01u)                        /* AND..NOR, 3 */     \
+    X(13, 3, 0x07u) X(14, 3, 0xF8u) X(15, 3, 0x1Fu) X(16, 3, 0xE0u) X(17, 3, 0xE2u)       /* AOI21 AO21 OAI21 OA21 MUX2 */
+inline uint32_t cell_class(uint32_t k, uint32_t tt) {
+#define DP_CELL(I, K, TT) if (k == K && tt == TT) return I;
+    DP_CELL_CLASSES(DP_CELL)
+#undef DP_CELL
+    return 18 + k;
+}
+
 // Per-design function table passed by value to kernels (lives in the
-// constant bank): entry = truth table (bits 0..15) | arity << 16 |
+// constant bank): entry = truth table (bits 0..15) | arity << 16 | class << 19 |
 // (for arity <= 3) the 8-bit LOP3 table of the function << 24, whose entry
 // 4 x2 + 2 x1 + x0 is f(x0, x1, x2) (inputs beyond the arity ignored).
 struct OpTable {
@@ -161,13 +175,15 @@ cudaError_t launch_probe_chase(const uint32_t *next, int hops, uint32_t *sink, c
 struct BatchBufs {
     int64_t S;
     float *sp_in, *tr_in;   // [n_start * S] staged inputs
-    float2 *pq;             // [n_nets * S] float-float P(net=1) (hi, lo); P(net=0) = 1 - P re-derived
+    float2 *pq;             // [n_nets * S] float-float P(net=1) (hi, lo; bit 30 of lo: tag); P(net=0) = 1 - P re-derived
     float *gfo;             // [n_edges * S] edge adjoints in fanout-CSR order
     float *gsp;             // [n_start * S] SP adjoint of the startpoints
     double *partials;       // [kBatchPowerChunks * S]
     double *power;          // [S] model power per scenario
     float *ks;              // [S] per-scenario seed of the backward (K * weight), binary32
     const float *dcl;       // [n_nets * S] per-scenario change of C_load (sizing deltas), or NULL
+    uint32_t *state;        // [8] the dataflow passes' (0 at rest): [0] columns of pq if such a pass wrote it, else 0;
+                            // [1] forward passes; [2] 1: every word of gfo is at rest; [3], [4] blocks done
     // lag-one mode (tr_mode 2) only, else NULL:
     float *tq;              // [n_nets * S] TR of every net
     float2 *gfo2;           // [n_edges * S] edge adjoints of (P, TR)
@@ -196,6 +212,12 @@ cudaError_t launch_fwdb_group(const DevDesign &d, const BatchBufs &b, const OpTa
                               cudaStream_t s);
 cudaError_t launch_bwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
                               cudaStream_t s);
+// the same passes (tr_mode 0 and 1) in one launch each without barriers between levels (kern_flowb.cu): v scenarios
+// per thread (S a multiple of v); edges: the words of gfo
+cudaError_t launch_fwdb_flow(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int v, int sms,
+                             cudaStream_t s);
+cudaError_t launch_bwdb_flow(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, int v,
+                             int64_t edges, int sms, cudaStream_t s);
 void launch_powerb(const DevDesign &d, const BatchBufs &b, int tr_mode, double K, cudaStream_t s);
 // ks[s] = K * weights[s] (weights NULL: K)
 void launch_seedb(const BatchBufs &b, double K, const double *weights, cudaStream_t s);
