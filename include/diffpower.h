@@ -333,12 +333,12 @@ dp_status dp_phase_times(dp_design *d, float *ms5);
  * with a new n_scen outside capture also runs the launch-shape autotuner
  * (times every candidate shape of the forward and reverse kernels on the
  * staged inputs and keeps the fastest; synchronises).  The environment
- * variable DP_BATCH_SHAPE="bx,by[,bx2,by2]" fixes the shapes instead.  In
- * tr_mode 0 and 1 it also times the passes without level barriers, one cooperative
- * launch each (DP_BATCH_FLOW="v" takes them with v scenarios per thread wherever
- * v divides n_scen), and for up to seven scenarios those by scenario groups
- * (DP_BATCH_GROUP="lanes,v,blocks,threads" fixes them); a wait in the former that
- * gives up is reported as DP_ETIMEOUT by the next synchronising call.
+ * variable DP_BATCH_SHAPE="bx,by[,bx2,by2]" fixes the shapes instead.  It
+ * also times the passes without level barriers, one cooperative launch each
+ * (DP_BATCH_FLOW="v" takes them with v scenarios per thread wherever v divides
+ * n_scen), and for up to seven scenarios those by scenario groups
+ * (DP_BATCH_GROUP="lanes,v,blocks,threads" fixes them); a wait in the former
+ * that gives up is reported as DP_ETIMEOUT by the next synchronising call.
  * Every shape gives bitwise identical results. */
 dp_status dp_set_inputs_batch(dp_design *d, const float *sp, const float *tr, int32_t n_scen, int on_device);
 

@@ -169,11 +169,12 @@ dp::GroupShape group_in_use(const dp_design *D, int tr_mode, int pass) {
 // launch that would tell them of a pass by level launches.)
 int flow_in_use(const dp_design *D, int tr_mode, int pass) {
     const dp_batch &B = D->batch;
-    if (tr_mode == 2 || D->d.n_start == 0) return 0;
-    if (const int v = flow_env(B.S)) return v;
+    if (D->d.n_start == 0) return 0;
     dp::GroupShape g;
-    if (B.shape_from_env || parse_group_env(&g) || B.tuned_S != B.S || B.shapes_locked) return 0;
-    return pass == 0 ? B.fwd_flow : B.bwd_flow;
+    int v = flow_env(B.S);
+    if (v == 0 && !B.shape_from_env && !parse_group_env(&g) && B.tuned_S == B.S && !B.shapes_locked)
+        v = pass == 0 ? B.fwd_flow : B.bwd_flow;
+    return tr_mode == 2 && v > 2 ? 2 : v;
 }
 
 // Scenarios per thread of the dataflow passes of a design with W cells per level: as many as leave whole warps and
@@ -253,7 +254,7 @@ dp_status tune(dp_design *D) {
             const int v = flow_v(S, W);
             const float t = timed(   // the first run also brings the arrays to rest
                 [&] {
-                    return pass == 0 ? dp::launch_fwdb_flow(D->d, B.b, D->ops, v, c->sm_count, st)
+                    return pass == 0 ? dp::launch_fwdb_flow(D->d, B.b, D->ops, 0, v, c->sm_count, st)
                                      : dp::launch_bwdb_flow(D->d, B.b, D->ops, 0, v, D->n_edges * B.cap, c->sm_count, st);
                 },
                 true, least[pass]);
@@ -304,7 +305,7 @@ namespace dpi {
 cudaError_t batch_forward(dp_design *D, int tr_mode, cudaStream_t s) {
     dp_batch &B = D->batch;
     const int v = flow_in_use(D, tr_mode, 0);
-    if (v > 0) return dp::launch_fwdb_flow(D->d, B.b, D->ops, v, D->ctx->sm_count, s);
+    if (v > 0) return dp::launch_fwdb_flow(D->d, B.b, D->ops, tr_mode, v, D->ctx->sm_count, s);
     const dp::GroupShape g = group_in_use(D, tr_mode, 0);
     if (g.v > 0) return dp::launch_fwdb_group(D->d, B.b, D->ops, tr_mode, g, s);
     dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), tr_mode, B.fwd_shape, s);

@@ -372,26 +372,36 @@ __device__ __forceinline__ void cell_adjoints(uint32_t e, const Row2<V> (&x)[4],
         }
 }
 
-// the partial derivatives of a cell's P with respect to its inputs' (get(j) reads input j)
-template <int V, class G>
-__device__ __forceinline__ void cell_partials(uint32_t e, const G &get, Row1<V> (&d)[4]) {
+// the partial derivatives of a cell with respect to its inputs (get(j, x, t) reads input j): of P by P in d, LAG: of T by
+// P and by T in dp and dt
+template <int V, bool LAG, class G>
+__device__ __forceinline__ void cell_partials(uint32_t e, const G &get, Row1<V> (&d)[4], Row1<V> (&dp)[4],
+                                              Row1<V> (&dt)[4]) {
     with_cell(e, [&](const auto f) {
         constexpr int K = decltype(f)::k;
         Row2<V> x[4];
+        Row1<V> t[4];
 #pragma unroll
-        for (int j = 0; j < K; j++) x[j] = get(j);
+        for (int j = 0; j < K; j++) get(j, x[j], t[j]);
 #pragma unroll
         for (int i = 0; i < V; i++) {
-            float p[4], q[4], g[4];
+            float p[4], q[4], g[4], w[4][4];
 #pragma unroll
             for (int j = 0; j < K; j++) {
                 const pair_ff v = pair_get(x[j].v[i]);
                 p[j] = v.p.hi + v.p.lo;
                 q[j] = v.q.hi + v.q.lo;
+                if (LAG) lag1_weights(v, t[j].v[i], w[j]);
             }
             f.partials(p, q, g);
 #pragma unroll
             for (int j = 0; j < K; j++) d[j].v[i] = g[j];
+            if constexpr (LAG) {
+                float gp[4], gt[4];
+                f.toggle_partials(w, gp, gt);
+#pragma unroll
+                for (int j = 0; j < K; j++) dp[j].v[i] = gp[j], dt[j].v[i] = gt[j];
+            }
         }
     });
 }

@@ -5,8 +5,9 @@
 // Forward: the low part of a stored P never has bit 30 set (|lo| < 2 for |P| < 2^25), so the bit carries the
 // parity of the pass that wrote it, in the same single-copy atomic word; everything that reads a
 // stored P drops it (pair_get).  Reverse: an edge's contribution is written once and read once, and its
-// reader leaves kNotYet behind for the next pass.  launch_flowb_prep brings both to rest where another pass wrote
-// the arrays in between.
+// reader leaves kNotYet behind for the next pass.  k_flowb_prep brings both to rest where another pass wrote
+// the arrays in between.  Lag-one mode: a net's T has no bit to spare; it starts as kNotYet in every pass (27 MB, 6 us
+// at 50,000 x 128).
 //
 // What bounds it: the level launches end a grid and start the next per level, about 3 us, with 58 instructions per
 // (cell, scenario) to do in between (30 % of the issue slots used, 38 % of the warps active).  Without them a pass
@@ -17,7 +18,8 @@
 // partial derivatives before it waits for the fanout, so only sums and products are on the way from level to level.
 // Forward with the model power + reverse, level launches against this: 120,000 x 512 404 + 575 us -> 366 + 435;
 // 50,000 x 256 172 + 220 -> 124 + 137; 50,000 x 128 145 + 189 -> 104 + 103; 20,000 / 38 x 37 84 + 105 -> 66 + 68; 2,000 /
-// 24 x 512 67 + 83 -> 50 + 50 (the power pass's own gain, 16 us at 50,000 x 256, included).
+// 24 x 512 67 + 83 -> 50 + 50 (the power pass's own gain, 16 us at 50,000 x 256, included).  Lag-one mode: 50,000 x
+// 128 142 + 257 -> 115 + 135, 120,000 x 256 555 + 1197 (level launches, general cell functions) -> 304 + 448.
 //
 // Progress: an item depends on lower levels only (reverse: higher), every warp takes its items in that
 // order and the cooperative launch keeps all warps resident, so the lowest unfinished item can always
@@ -83,6 +85,30 @@ __device__ __forceinline__ bool gives_up(unsigned &spins, long long t0, int *err
     return __any_sync(kAll, lost);
 }
 
+// an edge's adjoint: of P, in the lag-one mode of P and T
+template <bool LAG>
+struct Edge {
+    using T = float;
+    template <int V>
+    using Row = Row1<V>;
+    __device__ __forceinline__ static float rest() { return __uint_as_float(kNotYet); }
+};
+template <>
+struct Edge<true> {
+    using T = float2;
+    template <int V>
+    using Row = Row2<V>;
+    __device__ __forceinline__ static float2 rest() {
+        return make_float2(__uint_as_float(kNotYet), __uint_as_float(kNotYet));
+    }
+};
+__device__ __forceinline__ bool waits(float v) { return __float_as_uint(v) == kNotYet; }
+__device__ __forceinline__ bool waits(const float2 &v) { return waits(v.x) || waits(v.y); }
+template <int V>
+__device__ __forceinline__ void put(float *p, const Row1<V> &r) { st1<V>(p, r); }
+template <int V>
+__device__ __forceinline__ void put(float2 *p, const Row2<V> &r) { st2<V>(p, r); }
+
 // A warp's walk through the items: a net of the level and one of m chunks of 32 V scenarios.
 struct Walk {
     const int *first;   // level l's nets are first[l] .. first[l + 1] (level 0: the startpoints)
@@ -140,10 +166,10 @@ __device__ __forceinline__ bool last_block(uint32_t *done) {
     return true;
 }
 
-template <int V, int THREADS, int BLOCKS>
+template <int V, bool LAG, int THREADS, int BLOCKS>
 __global__ void __launch_bounds__(THREADS, BLOCKS)
-    k_fwdb_flow(const uint4 *__restrict__ fanin, float2 *pq, const float *__restrict__ sp_in,
-                const int32_t *__restrict__ lvl, int L, uint32_t ns, uint32_t S, uint32_t *state, OpTable ops, int *err,
+    k_fwdb_flow(const uint4 *__restrict__ fanin, float2 *pq, float *tq, const float *__restrict__ sp_in,
+                const float *__restrict__ tr_in, const int32_t *__restrict__ lvl, int L, uint32_t ns, uint32_t S, uint32_t *state, OpTable ops, int *err,
                 long long limit) {
     extern __shared__ int bounds[];
     level_bounds(bounds, lvl, L, ns);
@@ -168,24 +194,38 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
         const bool on = s < S;
         const uint32_t sc = on ? s : 0;   // a lane past the batch goes along with the first columns
         float2 *const pqs = pq + sc;
+        float *const tqs = LAG ? tq + sc : nullptr;
         at.next();
         Row2<V> o;
+        Row1<V> ot;
         if (c < ns) {
             const Row1<V> a = ld1<V>(row_at(sp_in + sc, c, S));
 #pragma unroll
             for (int i = 0; i < V; i++) o.v[i] = make_float2(a.v[i], 0.f);
+            if (LAG) {
+                ot = ld1<V>(row_at(tr_in + sc, c, S));
+#pragma unroll
+                for (int i = 0; i < V; i++)   // a caller's NaN of these bits is stored as another
+                    if (__float_as_uint(ot.v[i]) == kNotYet) ot.v[i] = __uint_as_float(0x7FFFFFFFu);
+            }
         } else {
             const int k = (int)((e >> 16) & 7u);
             Row2<V> x[4];
+            Row1<V> t[4];
             bool late[4];
             auto look = [&](int j) {
-                x[j] = ld_row<V>(row_at(pqs, n[j], S));
+                x[j] = ld_row<V>(row_at((const float2 *)pqs, n[j], S));
+                if (LAG) t[j] = ld_row<V>(row_at((const float *)tqs, n[j], S));
             };
             auto check = [&](int j) {
                 uint32_t bad = 0;
 #pragma unroll
                 for (int i = 0; i < V; i++) bad |= __float_as_uint(x[j].v[i].y) ^ tag;
-                return (bad & kTagBit) != 0;
+                bool b = (bad & kTagBit) != 0;
+                if (LAG)
+#pragma unroll
+                    for (int i = 0; i < V; i++) b = b || __float_as_uint(t[j].v[i]) == kNotYet;
+                return b;
             };
 #pragma unroll
             for (int j = 0; j < 4; j++)
@@ -205,15 +245,20 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
                     if (gives_up(spins, t0, err, limit)) ok = false;
                 } while (ok && __any_sync(kAll, late[0] || late[1] || late[2] || late[3]));
             }
-            Row1<V> none;
-            cell_value<V, false>(
-                e, [&](int j, Row2<V> &xj, Row1<V> &) { xj = x[j]; }, o, none);
+            cell_value<V, LAG>(
+                e,
+                [&](int j, Row2<V> &xj, Row1<V> &tj) {
+                    xj = x[j];
+                    if (LAG) tj = t[j];
+                },
+                o, ot);
         }
         if (on) {
 #pragma unroll
             for (int i = 0; i < V; i++)
                 o.v[i].y = __uint_as_float((__float_as_uint(o.v[i].y) & ~kTagBit) | tag);
             st2<V>(row_at(pqs, c, S), o);
+            if (LAG) st1<V>(row_at(tqs, c, S), ot);
         }
     }
     if (last_block(state + 3)) {
@@ -222,11 +267,12 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
     }
 }
 
-template <int V, int THREADS, int BLOCKS>
+template <int V, bool LAG, int THREADS, int BLOCKS>
 __global__ void __launch_bounds__(THREADS, BLOCKS)
     k_bwdb_flow(const uint4 *__restrict__ fanin, const int32_t *__restrict__ fptr, const int4 *__restrict__ efpos,
-                const float2 *__restrict__ pq, const float *__restrict__ cload, const float *__restrict__ dcl,
-                const float *__restrict__ ks, float *gfo, float *gsp, const int32_t *__restrict__ lvl, int L,
+                const float2 *__restrict__ pq, const float *__restrict__ tq, const float *__restrict__ cload, const float *__restrict__ dcl,
+                const float *__restrict__ ks, typename Edge<LAG>::T *gfo, float *gsp, float *gtr,
+                const int32_t *__restrict__ lvl, int L,
                 uint32_t ns, uint32_t S, int tr_mode, uint32_t *state, OpTable ops, int *err, long long limit) {
     extern __shared__ int bounds[];
     level_bounds(bounds, lvl, L, ns);
@@ -257,36 +303,50 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
         const uint32_t sc = on ? s : 0;
         at.next();
         const float2 *const pqs = pq + sc;
-        float *const gs = gfo + sc;
+        typename Edge<LAG>::T *const gs = gfo + sc;
         const int k = c < ns ? 0 : (int)((e >> 16) & 7u);
-        // what does not wait for the fanout: the partial derivatives, and the local term's factors (bwdb_adjoint)
-        Row1<V> two_kc = ld1<V>(ks + sc), qmp, d[4];
+        // what does not wait for the fanout: the partial derivatives, the load, the local term's factor (bwdb_adjoint)
+        const Row1<V> Ks = ld1<V>(ks + sc);
+        Row1<V> cl, qmp, d[4], dp[4], dt[4];
         {
-            Row1<V> dc;
-            if (dcl) dc = ld1<V>(row_at(dcl + sc, c, S));
-            const float cl = cload[c];
-            const Row2<V> self = ld2<V>(row_at(pqs, c, S));
-            if (c >= ns) cell_partials<V>(e, [&](int j) { return ld2<V>(row_at(pqs, n[j], S)); }, d);
+            if (dcl) cl = ld1<V>(row_at(dcl + sc, c, S));
+            const float c0 = cload[c];
+            Row2<V> self;
+            if (!LAG) self = ld2<V>(row_at(pqs, c, S));
+            if (c >= ns)
+                cell_partials<V, LAG>(
+                    e,
+                    [&](int j, Row2<V> &x, Row1<V> &t) {
+                        x = ld2<V>(row_at(pqs, n[j], S));
+                        if (LAG) t = ld1<V>(row_at(tq + sc, n[j], S));
+                    },
+                    d, dp, dt);
 #pragma unroll
             for (int i = 0; i < V; i++) {
-                two_kc.v[i] = __fmul_rn(__fmul_rn(2.f, two_kc.v[i]), dcl ? cl + dc.v[i] : cl);
-                qmp.v[i] = qmp32(self.v[i]);
+                cl.v[i] = dcl ? c0 + cl.v[i] : c0;
+                if (!LAG) {
+                    cl.v[i] = __fmul_rn(__fmul_rn(2.f, Ks.v[i]), cl.v[i]);
+                    qmp.v[i] = qmp32(self.v[i]);
+                }
             }
         }
         // the fanout sum in index order, F edges in flight
-        constexpr int F = V == 4 ? 2 : 4;
-        Row1<V> a;
+        constexpr int F = V == 4 || (LAG && V == 2) ? 2 : 4;
+        Row1<V> a, b;
 #pragma unroll
-        for (int i = 0; i < V; i++) a.v[i] = 0.f;
+        for (int i = 0; i < V; i++) a.v[i] = b.v[i] = 0.f;
         for (int32_t p = f0; p < f1 && ok; p += F) {
-            Row1<V> u[F];
+            using R = typename Edge<LAG>::template Row<V>;
+            R u[F];
             bool late[F];
-            auto look = [&](int j) { u[j] = ld_row<V>(row_at((const float *)gs, (uint32_t)(p + j), S)); };
+            auto look = [&](int j) {
+                u[j] = ld_row<V>(row_at((const typename Edge<LAG>::T *)gs, (uint32_t)(p + j), S));
+            };
             auto check = [&](int j) {
-                bool b = false;
+                bool w = false;
 #pragma unroll
-                for (int i = 0; i < V; i++) b = b || __float_as_uint(u[j].v[i]) == kNotYet;
-                return b && on;
+                for (int i = 0; i < V; i++) w = w || waits(u[j].v[i]);
+                return w && on;
             };
 #pragma unroll
             for (int j = 0; j < F; j++)
@@ -294,10 +354,10 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
 #pragma unroll
             for (int j = 0; j < F; j++) late[j] = p + j < f1 && check(j);
             auto any = [&] {
-                bool b = false;
+                bool w = false;
 #pragma unroll
-                for (int j = 0; j < F; j++) b = b || late[j];
-                return __any_sync(kAll, b) != 0;
+                for (int j = 0; j < F; j++) w = w || late[j];
+                return __any_sync(kAll, w) != 0;
             };
             if (any()) {
                 const long long t0 = clock64();
@@ -311,58 +371,74 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
                     if (gives_up(spins, t0, err, limit)) ok = false;
                 } while (ok && any());
             }
-            Row1<V> rest;
+            R rest;
 #pragma unroll
-            for (int i = 0; i < V; i++) rest.v[i] = __uint_as_float(kNotYet);
+            for (int i = 0; i < V; i++) rest.v[i] = Edge<LAG>::rest();
 #pragma unroll
             for (int j = 0; j < F; j++)
                 if (p + j < f1) {
 #pragma unroll
-                    for (int i = 0; i < V; i++) a.v[i] += u[j].v[i];
-                    if (on) st1<V>(row_at(gs, (uint32_t)(p + j), S), rest);
+                    for (int i = 0; i < V; i++) {
+                        if constexpr (LAG) a.v[i] += u[j].v[i].x, b.v[i] += u[j].v[i].y;
+                        else a.v[i] += u[j].v[i];
+                    }
+                    if (on) put(row_at(gs, (uint32_t)(p + j), S), rest);
                 }
         }
         if (!on) continue;
-        if (c >= ns || tr_mode) {
+        if (LAG) {
 #pragma unroll
-            for (int i = 0; i < V; i++) a.v[i] = fmaf(two_kc.v[i], qmp.v[i], a.v[i]);
+            for (int i = 0; i < V; i++) b.v[i] = fmaf(Ks.v[i], cl.v[i], b.v[i]);
+        } else if (c >= ns || tr_mode) {
+#pragma unroll
+            for (int i = 0; i < V; i++) a.v[i] = fmaf(cl.v[i], qmp.v[i], a.v[i]);
         }
         if (c < ns) {
             st1<V>(row_at(gsp + sc, c, S), a);
+            if (LAG) st1<V>(row_at(gtr + sc, c, S), b);
             continue;
         }
 #pragma unroll
         for (int j = 0; j < 4; j++)
             if (j < k) {
+                typename Edge<LAG>::template Row<V> g;
 #pragma unroll
-                for (int i = 0; i < V; i++) d[j].v[i] = __fmul_rn(a.v[i], d[j].v[i]);
-                st1<V>(row_at(gs, pos[j], S), d[j]);
+                for (int i = 0; i < V; i++) {
+                    if constexpr (LAG)
+                        g.v[i] = make_float2(fmaf(a.v[i], d[j].v[i], __fmul_rn(b.v[i], dp[j].v[i])),
+                                             __fmul_rn(b.v[i], dt[j].v[i]));
+                    else g.v[i] = __fmul_rn(a.v[i], d[j].v[i]);
+                }
+                put(row_at(gs, pos[j], S), g);
             }
     }
-    if (last_block(state + 4)) state[2] = ld_word(err) ? 0u : 1u;
+    if (last_block(state + 4)) state[LAG ? 5 : 2] = ld_word(err) ? 0u : 1u;
 }
 
-// The arrays of a pass (0 forward: the pairs of the batch; 1 reverse: all edges) as the pass expects them, where the
-// last to write them was not a dataflow pass (forward: of the same S).
-__global__ void k_flowb_prep(int which, float2 *pq, int64_t n, uint32_t S, float *gfo, int64_t m,
-                             const uint32_t *state) {
+// The arrays of a pass as it expects them: which 0, the forward pass's pairs, where the last to write them was not a
+// dataflow pass of the same S (and tq, n words, always); 1, the reverse pass's edges, m words, where the last was not one
+// (clean: its mark)
+__global__ void k_flowb_prep(int which, float2 *pq, float *tq, int64_t n, uint32_t S, float *gfo, int64_t m,
+                             const uint32_t *state, const uint32_t *clean) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, T = (int64_t)gridDim.x * blockDim.x;
     if (which == 0) {
+        if (tq)
+            for (int64_t i = t; i < n; i += T) tq[i] = __uint_as_float(kNotYet);
         if (state[0] == S) return;
         const float2 v = make_float2(0.f, __uint_as_float((state[1] & 1u) << 30));
         for (int64_t i = t; i < n; i += T) pq[i] = v;
     } else {
-        if (state[2] == 1u) return;
+        if (*clean == 1u) return;
         for (int64_t i = t; i < m; i += T) gfo[i] = __uint_as_float(kNotYet);
     }
 }
 
 // threads per block and blocks per SM by scenarios per thread (see above; 50,000 x 256 reverse, v = 4: 512 threads per
 // SM 137 us, 640 137, 768 150; 120,000 x 512 485, 441, 467)
-template <int V>
+template <int V, bool LAG>
 struct Cfg {
-    static constexpr int fthreads = V == 4 ? 384 : 512, fblocks = 2;
-    static constexpr int bthreads = V == 4 ? 320 : 448, bblocks = 2;
+    static constexpr int fthreads = V == 4 || LAG ? 384 : 512, fblocks = 2;
+    static constexpr int bthreads = V == 4 ? 320 : LAG ? 256 : 448, bblocks = 2;
 };
 
 template <class... KArgs, class... Args>
@@ -380,31 +456,44 @@ cudaError_t launch_flowb(void (*kern)(KArgs...), int threads, int blocks, int L,
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+template <int V, bool LAG>
+cudaError_t fwd(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int sms, cudaStream_t s) {
+    using C = Cfg<V, LAG>;
+    k_flowb_prep<<<(unsigned)(sms * 4), 512, 0, s>>>(0, b.pq, LAG ? b.tq : nullptr, d.n_nets * b.S, (uint32_t)b.S,
+                                                     nullptr, 0, b.state, nullptr);
+    return launch_flowb(k_fwdb_flow<V, LAG, C::fthreads, C::fblocks>, C::fthreads, C::fblocks * sms, d.n_levels, s,
+                        d.fanin, b.pq, b.tq, b.sp_in, b.tr_in, d.lvl, d.n_levels, d.n_start, b.S, b.state, ops, d.err,
+                        kWaitLimitCycles);
+}
+template <int V, bool LAG>
+cudaError_t bwd(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, int64_t edges, int sms,
+                cudaStream_t s) {
+    using C = Cfg<V, LAG>;
+    typename Edge<LAG>::T *gfo;
+    if constexpr (LAG) gfo = b.gfo2;
+    else gfo = b.gfo;
+    k_flowb_prep<<<(unsigned)(sms * 4), 512, 0, s>>>(1, nullptr, nullptr, 0, (uint32_t)b.S, (float *)gfo,
+                                                     edges * (LAG ? 2 : 1), b.state, b.state + (LAG ? 5 : 2));
+    return launch_flowb(k_bwdb_flow<V, LAG, C::bthreads, C::bblocks>, C::bthreads, C::bblocks * sms, d.n_levels, s,
+                        d.fanin, d.fout_ptr, (const int4 *)d.edge_fpos, b.pq, b.tq, d.cload, b.dcl, b.ks, gfo, b.gsp,
+                        b.gtr, d.lvl, d.n_levels, d.n_start, b.S, tr_mode, b.state, ops, d.err, kWaitLimitCycles);
+}
+
 }  // namespace
 
-cudaError_t launch_fwdb_flow(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int v, int sms,
+cudaError_t launch_fwdb_flow(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, int v, int sms,
                              cudaStream_t s) {
-    k_flowb_prep<<<(unsigned)(sms * 4), 512, 0, s>>>(0, b.pq, d.n_nets * b.S, (uint32_t)b.S, b.gfo, 0, b.state);
-    auto go = [&](auto kern, int threads, int blocks) {
-        return launch_flowb(kern, threads, blocks * sms, d.n_levels, s, d.fanin, b.pq, b.sp_in, d.lvl, d.n_levels,
-                            d.n_start, b.S, b.state, ops, d.err, kWaitLimitCycles);
-    };
-#define GO(V) go(k_fwdb_flow<V, Cfg<V>::fthreads, Cfg<V>::fblocks>, Cfg<V>::fthreads, Cfg<V>::fblocks)
-    return v == 4 ? GO(4) : v == 2 ? GO(2) : GO(1);
-#undef GO
+    if (tr_mode == 2) return v == 1 ? fwd<1, true>(d, b, ops, sms, s) : fwd<2, true>(d, b, ops, sms, s);
+    if (v == 4) return fwd<4, false>(d, b, ops, sms, s);
+    return v == 2 ? fwd<2, false>(d, b, ops, sms, s) : fwd<1, false>(d, b, ops, sms, s);
 }
 
 cudaError_t launch_bwdb_flow(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, int v,
                              int64_t edges, int sms, cudaStream_t s) {
-    k_flowb_prep<<<(unsigned)(sms * 4), 512, 0, s>>>(1, b.pq, 0, (uint32_t)b.S, b.gfo, edges, b.state);
-    auto go = [&](auto kern, int threads, int blocks) {
-        return launch_flowb(kern, threads, blocks * sms, d.n_levels, s, d.fanin, d.fout_ptr, (const int4 *)d.edge_fpos,
-                            b.pq, d.cload, b.dcl, b.ks, b.gfo, b.gsp, d.lvl, d.n_levels, d.n_start, b.S, tr_mode,
-                            b.state, ops, d.err, kWaitLimitCycles);
-    };
-#define GO(V) go(k_bwdb_flow<V, Cfg<V>::bthreads, Cfg<V>::bblocks>, Cfg<V>::bthreads, Cfg<V>::bblocks)
-    return v == 4 ? GO(4) : v == 2 ? GO(2) : GO(1);
-#undef GO
+    if (tr_mode == 2)
+        return v == 1 ? bwd<1, true>(d, b, ops, tr_mode, edges, sms, s) : bwd<2, true>(d, b, ops, tr_mode, edges, sms, s);
+    if (v == 4) return bwd<4, false>(d, b, ops, tr_mode, edges, sms, s);
+    return v == 2 ? bwd<2, false>(d, b, ops, tr_mode, edges, sms, s) : bwd<1, false>(d, b, ops, tr_mode, edges, sms, s);
 }
 
 }  // namespace dp

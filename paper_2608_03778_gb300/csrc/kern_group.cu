@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kGroupThreads) k_bwdb_group(
     const float *__restrict__ ks, float *gfo, float2 *gfo2, float *gsp, float *gtr, const int32_t *__restrict__ lvl,
     int L, int64_t ns, int64_t S, int lanes, int tr_mode, OpTable ops, uint32_t *state) {
     const Place at(lanes, V);
-    if (!LAG && blockIdx.x == 0 && threadIdx.x == 0) state[2] = 0u;   // gfo will hold values
+    if (blockIdx.x == 0 && threadIdx.x == 0) state[LAG ? 5 : 2] = 0u;   // the edges will hold values
     const bool on = at.s < S;
     pq += at.s;
     gsp += at.s;

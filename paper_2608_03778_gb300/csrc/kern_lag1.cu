@@ -107,11 +107,13 @@ __global__ void k_bwdl_level(const uint4 *__restrict__ fanin, const int32_t *__r
 
 __global__ void k_bwdl_start(const int32_t *__restrict__ fptr, const float *__restrict__ cload,
                              const float *__restrict__ dcl, const float *__restrict__ ks,
-                             const float2 *__restrict__ gfo2, float *gsp, float *gtr, int64_t ns, int64_t S) {
+                             const float2 *__restrict__ gfo2, float *gsp, float *gtr, int64_t ns, int64_t S,
+                             uint32_t *state) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     pdl_trigger();
     if (s >= S) return;
     pdl_wait();
+    if (s == 0 && blockIdx.y == 0 && threadIdx.y == 0) state[5] = 0u;   // gfo2 holds values
     const float Ks = ks[s];
     const int64_t step = (int64_t)gridDim.y * blockDim.y;
     for (int64_t k = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; k < ns; k += step) {
@@ -155,7 +157,7 @@ void launch_bwdl(const DevDesign &d, const BatchBufs &b, const OpTable &ops, con
     }
     if (d.n_start)
         launch_pdl(k_bwdl_start, bgrid(S, sh, d.n_start), blk, s, d.fout_ptr, d.cload, b.dcl, b.ks, b.gfo2, b.gsp,
-                   b.gtr, d.n_start, S);
+                   b.gtr, d.n_start, S, b.state);
 }
 
 }  // namespace dp

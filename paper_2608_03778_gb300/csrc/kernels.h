@@ -183,7 +183,7 @@ struct BatchBufs {
     float *ks;              // [S] per-scenario seed of the backward (K * weight), binary32
     const float *dcl;       // [n_nets * S] per-scenario change of C_load (sizing deltas), or NULL
     uint32_t *state;        // [8] the dataflow passes' (0 at rest): [0] columns of pq if such a pass wrote it, else 0;
-                            // [1] forward passes; [2] 1: every word of gfo is at rest; [3], [4] blocks done
+                            // [1] forward passes; [2] 1: every word of gfo is at rest; [3], [4] blocks done; [5] as [2], of gfo2
     // lag-one mode (tr_mode 2) only, else NULL:
     float *tq;              // [n_nets * S] TR of every net
     float2 *gfo2;           // [n_edges * S] edge adjoints of (P, TR)
@@ -212,9 +212,9 @@ cudaError_t launch_fwdb_group(const DevDesign &d, const BatchBufs &b, const OpTa
                               cudaStream_t s);
 cudaError_t launch_bwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
                               cudaStream_t s);
-// the same passes (tr_mode 0 and 1) in one launch each without barriers between levels (kern_flowb.cu): v scenarios
-// per thread (S a multiple of v); edges: the words of gfo
-cudaError_t launch_fwdb_flow(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int v, int sms,
+// the same passes in one launch each without barriers between levels (kern_flowb.cu): v scenarios
+// per thread (S a multiple of v; in the lag-one mode at most 2); edges: the elements of gfo
+cudaError_t launch_fwdb_flow(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, int v, int sms,
                              cudaStream_t s);
 cudaError_t launch_bwdb_flow(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, int v,
                              int64_t edges, int sms, cudaStream_t s);

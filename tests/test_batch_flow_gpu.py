@@ -8,7 +8,7 @@ import pytest
 from oracle.oracle import Oracle
 from paper_2608_03778_gb300 import netgen
 from tests._netlists import custom_case
-from tests.test_batch_gpu import check_scenarios, ctx, dp, run_batch  # noqa: F401
+from tests.test_batch_gpu import check_lag1, check_scenarios, ctx, dp, run_batch  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -48,7 +48,7 @@ def netlists(library_text, S):
 
 
 # one lane, a ragged chunk, whole chunks, a ragged last chunk of 64 and of 128 columns
-@pytest.mark.parametrize("tr_mode", [0, 1])
+@pytest.mark.parametrize("tr_mode", [0, 1, 2])
 @pytest.mark.parametrize("S", [1, 33, 64, 130, 260])
 def test_dataflow_matches_level_launches(dp, ctx, library_text, S, tr_mode):  # noqa: F811
     for i, (text, lib) in enumerate(netlists(library_text, S)):
@@ -58,7 +58,10 @@ def test_dataflow_matches_level_launches(dp, ctx, library_text, S, tr_mode):  # 
         for v in (1, 2, 4):
             if S % v == 0:
                 same(run(dp, ctx, text, lib, v, sp, tr, tr_mode), ref, f"netlist {i} v {v}")
-        check_scenarios(o, ref, sp, tr, dp.config(grad_mode=0, tr_mode=tr_mode), range(min(S, 3)))
+        if tr_mode == 2:
+            check_lag1(o, ref, sp, tr, range(min(S, 3)))
+        else:
+            check_scenarios(o, ref, sp, tr, dp.config(grad_mode=0, tr_mode=tr_mode), range(min(S, 3)))
 
 
 def test_dataflow_after_other_passes(dp, ctx, library_text):  # noqa: F811
@@ -69,7 +72,8 @@ def test_dataflow_after_other_passes(dp, ctx, library_text):  # noqa: F811
     d = dp.dp_design_load(ctx, text, library_text)
     try:
         for i, (how, S, m) in enumerate([(2, 96, 0), (2, 96, 0), (1, 64, 0), (4, 96, 0), ("level", 64, 0), (2, 64, 0),
-                                         ("level", 64, 2), (2, 64, 0), (1, 32, 0), ("level", 32, 0), (2, 96, 0)]):
+                                         ("level", 64, 2), (2, 64, 0), (1, 32, 0), ("level", 32, 0), (2, 96, 0),
+                                         (2, 96, 2), (1, 64, 2), ("level", 96, 2), (1, 96, 2), (4, 96, 0)]):
             with forced(how):
                 got = run_batch(dp, ctx, d, *inputs[S], dp.config(grad_mode=0, tr_mode=m))
             same(got, ref[S, m], f"step {i}")
@@ -77,13 +81,15 @@ def test_dataflow_after_other_passes(dp, ctx, library_text):  # noqa: F811
         dp.dp_design_free(d)
 
 
-def test_dataflow_nan_inputs(dp, ctx, library_text):  # noqa: F811
+@pytest.mark.parametrize("tr_mode", [1, 2])
+def test_dataflow_nan_inputs(dp, ctx, library_text, tr_mode):  # noqa: F811
     torch = pytest.importorskip("torch")
     text = netgen.netlist_text(netgen.NetlistSpec(900, 20, 40, 9, 16, 4))
     sp, tr = netgen.scenario_inputs(60, 5, 64)
     sp[3, 5], sp[7, 9], sp[11, 40] = np.nan, np.inf, -np.inf
+    tr[8, 12] = np.array([0xFFFFFFFF], np.uint32).view(np.float32)[0]
     x, t = torch.from_numpy(sp).cuda(), torch.from_numpy(tr).cuda()
-    cfg = dp.config(grad_mode=0, tr_mode=1)
+    cfg = dp.config(grad_mode=0, tr_mode=tr_mode)
     got = {}
     for how in ("level", 1, 4):
         d = dp.dp_design_load(ctx, text, library_text)
@@ -99,7 +105,7 @@ def test_dataflow_nan_inputs(dp, ctx, library_text):  # noqa: F811
         finally:
             dp.dp_design_free(d)
     clean = np.ones(64, bool)
-    clean[[5, 9, 40]] = False
+    clean[[5, 9, 12, 40]] = False
     for how in (1, 4):
         np.testing.assert_array_equal(got[how][0], got["level"][0])
         np.testing.assert_array_equal(got[how][1][clean], got["level"][1][clean])
