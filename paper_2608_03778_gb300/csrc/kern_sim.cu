@@ -82,56 +82,52 @@ __device__ __forceinline__ uint64_t chain_block16(ChainState &c, uint32_t k, int
 // (no probability of exactly 1): a 16-bit draw d is compared in the high half
 // of a 32-bit word against thr << 16, which holds whatever the low half is, so
 // the high-half draws need no extraction.  Each lane keeps only the threshold
-// of its current state (t10 in state 1, t01 in state 0; a flip toggles it by
-// one XOR).  The warp votes on the flips, and the cycle's word is the previous
-// word XOR the flip word, so no lane state is formed.  Ones and toggles are
-// counted from the finished words.
-struct FastChain {
-    uint32_t thr[4];
-    uint64_t word;   // lane states of the previous cycle (this half-warp's startpoint)
-};
-
-// one cycle on draws d[r] (in the high half); FIRST draws the initial state
-template <bool FIRST>
-__device__ __forceinline__ uint64_t fast_cycle(FastChain &c, const uint32_t (&d)[4], uint32_t ti16, uint32_t t10_16,
-                                               uint32_t t01_16, uint32_t sel) {
-    bool b[4];   // FIRST: the initial state; else: a flip
-#pragma unroll
-    for (int r = 0; r < 4; r++) {
-        if (FIRST) {
-            b[r] = d[r] < ti16;
-            c.thr[r] = b[r] ? t10_16 : t01_16;
-        } else {
-            b[r] = d[r] < c.thr[r];
-            c.thr[r] ^= b[r] ? (t10_16 ^ t01_16) : 0u;
-        }
-    }
-    const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, b[0]), b1 = __ballot_sync(0xFFFFFFFFu, b[1]);
-    const uint32_t b2 = __ballot_sync(0xFFFFFFFFu, b[2]), b3 = __ballot_sync(0xFFFFFFFFu, b[3]);
-    const uint64_t w = (uint64_t)__byte_perm(b0, b1, sel) | ((uint64_t)__byte_perm(b2, b3, sel) << 32);
-    c.word = FIRST ? w : c.word ^ w;
-    return c.word;
+// of its current state (t10 in state 1, t01 in state 0; a flip exchanges it for
+// their sum less it).  The warp votes on the flips and its first lane stores the four votes of the
+// cycle; after sixteen cycles thread q takes those of cycle t0 + q, and the words are the running
+// XOR over the half-warp.  Ones and toggles are counted from the words and the flips.
+//
+// What bounds it: the ALU pipe (ten rounds of Philox take 20 of its instructions, the eight draws of a call
+// a comparison, a vote and a change of threshold each; with the word of every cycle formed and kept by its thread at
+// once it took 65 per call, now 40) and the 64-bit products of Philox, which leave every other issue slot unused.
+// 147,456 startpoints x 64 words 333 -> 245 us; 2,000,000-cell step 1,367 -> 1,288 us.
+//
+// the flips of one cycle of lane r on draw d (in the high half)
+__device__ __forceinline__ uint32_t fast_flips(uint32_t &thr, uint32_t d, uint32_t sum) {
+    const bool f = d < thr;
+    if (f) thr = sum - thr;
+    return __ballot_sync(0xFFFFFFFFu, f);
 }
 
+// sixteen cycles from cycle t0 (a multiple of 16) into votes[16]; FIRST draws the initial state
 template <bool FIRST>
-__device__ __forceinline__ uint64_t fast_block16(FastChain &c, uint32_t k, int t0, int q, uint32_t key0,
-                                                 uint32_t key1, uint32_t ti16, uint32_t t10_16, uint32_t t01_16,
-                                                 uint32_t sel) {
-    uint64_t mine = 0;
+__device__ __forceinline__ void fast_block16(uint32_t (&thr)[4], uint4 *votes, uint32_t k, int t0, int q, uint32_t key0,
+                                             uint32_t key1, uint32_t ti16, uint32_t t10_16, uint32_t t01_16) {
+    const uint32_t sum = t10_16 + t01_16;
+    const bool first_lane = (threadIdx.x & 31) == 0;
     // unrolled by 4, not 8: fully unrolled, the compiler keeps several calls' draws live
-    // (124 registers); at 4 the kernel needs 48 and more warps fit on an SM
 #pragma unroll 4
     for (int i = 0; i < 8; i++) {
         const uint4 u = philox4x32_10(make_uint4(k, (uint32_t)((t0 >> 1) + i), (uint32_t)q, 0u), key0, key1);
         const uint32_t lo[4] = {u.x << 16, u.y << 16, u.z << 16, u.w << 16};
         const uint32_t hi[4] = {u.x, u.y, u.z, u.w};
-        const uint64_t w0 = (FIRST && i == 0) ? fast_cycle<true>(c, lo, ti16, t10_16, t01_16, sel)
-                                              : fast_cycle<false>(c, lo, ti16, t10_16, t01_16, sel);
-        const uint64_t w1 = fast_cycle<false>(c, hi, ti16, t10_16, t01_16, sel);
-        if (q == 2 * i) mine = w0;
-        if (q == 2 * i + 1) mine = w1;
+        uint32_t b[4];
+        if (FIRST && i == 0) {
+#pragma unroll
+            for (int r = 0; r < 4; r++) {
+                const bool one = lo[r] < ti16;
+                thr[r] = one ? t10_16 : t01_16;
+                b[r] = __ballot_sync(0xFFFFFFFFu, one);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < 4; r++) b[r] = fast_flips(thr[r], lo[r], sum);
+        }
+        if (first_lane) votes[2 * i] = make_uint4(b[0], b[1], b[2], b[3]);
+#pragma unroll
+        for (int r = 0; r < 4; r++) b[r] = fast_flips(thr[r], hi[r], sum);
+        if (first_lane) votes[2 * i + 1] = make_uint4(b[0], b[1], b[2], b[3]);
     }
-    return mine;
 }
 
 __global__ void __launch_bounds__(256) k_sim_start(const float *__restrict__ sp_in, const float *__restrict__ tr_in,
@@ -167,12 +163,36 @@ __global__ void __launch_bounds__(256) k_sim_start(const float *__restrict__ sp_
         carry = __shfl_sync(0xFFFFFFFFu, w, 15, 16);
     };
     if (!__any_sync(0xFFFFFFFFu, (t_init | t10 | t01) >= 65536u)) {   // warp-uniform
-        FastChain c{};
-        for (int t0 = 0; t0 < T; t0 += 16)
-            take(t0 == 0 ? fast_block16<true>(c, (uint32_t)k, 0, q, key0, key1, t_init << 16, t10 << 16, t01 << 16, sel)
-                         : fast_block16<false>(c, (uint32_t)k, t0, q, key0, key1, t_init << 16, t10 << 16, t01 << 16,
-                                               sel),
-                 t0 + q);
+        __shared__ uint4 votes[8][16];
+        uint4 *const mine = votes[threadIdx.x >> 5];
+        uint32_t thr[4] = {0, 0, 0, 0};
+        uint32_t last_lo = 0, last_hi = 0;   // the word before this block
+        for (int t0 = 0; t0 < T; t0 += 16) {
+            if (t0 == 0)
+                fast_block16<true>(thr, mine, (uint32_t)k, 0, q, key0, key1, t_init << 16, t10 << 16, t01 << 16);
+            else
+                fast_block16<false>(thr, mine, (uint32_t)k, t0, q, key0, key1, t_init << 16, t10 << 16, t01 << 16);
+            __syncwarp();
+            const uint4 v = mine[q];
+            __syncwarp();   // read before the next block's votes
+            const uint32_t f_lo = __byte_perm(v.x, v.y, sel), f_hi = __byte_perm(v.z, v.w, sel);
+            uint32_t w_lo = f_lo, w_hi = f_hi;
+#pragma unroll
+            for (int o = 1; o < 16; o <<= 1) {
+                const uint32_t a = __shfl_up_sync(0xFFFFFFFFu, w_lo, o, 16), b = __shfl_up_sync(0xFFFFFFFFu, w_hi, o, 16);
+                if (q >= o) w_lo ^= a, w_hi ^= b;
+            }
+            w_lo ^= last_lo;
+            w_hi ^= last_hi;
+            last_lo = __shfl_sync(0xFFFFFFFFu, w_lo, 15, 16);
+            last_hi = __shfl_sync(0xFFFFFFFFu, w_hi, 15, 16);
+            const int t = t0 + q;
+            if (t < T) {
+                if (valid) out[t] = (uint64_t)w_lo | (uint64_t)w_hi << 32;
+                n_one += __popc(w_lo) + __popc(w_hi);
+                if (t > 0) n_flip += __popc(f_lo) + __popc(f_hi);
+            }
+        }
     } else {
         ChainState c{0u};
         take(chain_block16<true>(c, (uint32_t)k, 0, q, key0, key1, t_init, t10, t01, sel), q);
