@@ -245,6 +245,21 @@ struct SizingDeltas {
 void launch_sizing_deltas(const DevDesign &d, const OpTable &ops, const SizingDeltas &z, int64_t ne, int64_t S,
                           float *dcl, cudaStream_t s);
 // returns win, dpin, flag and dcl to rest after the batch
+// A request's host buffers, as the device reads and writes them (sp, tr NULL: the reference inputs; nd resized cells
+// from entry off of the batch's on; a gradient NULL: not wanted)
+struct ServeIo {
+    const float *sp, *tr;
+    const int32_t *cells;
+    const float *caps;
+    float *gsp, *gtr, *gpin;
+    int32_t nd, off;
+};
+// the inputs (in_sp NULL: not needed) and resized cells (off NULL: none) of the batch's S requests into its buffers
+void launch_serve_in(const ServeIo *io, int64_t S, int64_t ns, int64_t most_nd, const float *ref_sp, const float *ref_tr,
+                     float *in_sp, float *in_tr, int32_t *cell, float *cap, int32_t *off, cudaStream_t s);
+// its gradients, request-major, into the requests' buffers
+void launch_serve_out(const ServeIo *io, int64_t S, int64_t ns, int64_t nc, const float *sp, const float *tr,
+                      const float *pin, cudaStream_t s);
 // the reference inputs' forward state (P of every net, TR of every startpoint) into every
 // scenario column of a batch: a batch of requests on the reference inputs skips the forward pass
 void launch_bcast_ref(const float2 *ref_pq, const float *ref_tr, float2 *pq, float *tr_in, int64_t nn, int64_t ns,
