@@ -1,0 +1,44 @@
+"""The step's sliced simulation beside its forward pass: the same results as the phases called one after the other, for
+forward passes in one block and in one cluster, whole and ragged word counts, and repeated steps with changed inputs."""
+import numpy as np
+import pytest
+
+from paper_2608_03778_gb300 import netgen
+from tests.test_batch_gpu import ctx, dp  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def nets(dp, ctx, d, info):  # noqa: F811
+    out = [np.zeros(info.n_nets, t) for t in (np.float32, np.float32, np.uint32, np.uint32)]
+    dp.dp_get_nets(ctx, d, beta=out[0], tr_hyb=out[1], toggles=out[2], ones=out[3])
+    return out
+
+
+@pytest.mark.parametrize("spec", [(900, 60, 9), (6000, 400, 24), (16000, 1200, 40)])
+@pytest.mark.parametrize("T", [3, 64, 250])
+def test_step_equals_its_phases(dp, ctx, library_text, spec, T):  # noqa: F811
+    cells, start, depth = spec
+    text = netgen.netlist_text(netgen.NetlistSpec(cells, start // 3, start - start // 3, depth, 16, 7))
+    d = dp.dp_design_load(ctx, text, library_text)
+    try:
+        info = dp.dp_design_info(d)
+        cfg = dp.config(grad_mode=2, tr_mode=0, sim_words=T)
+        for seed in (1, 2):
+            sp, tr = (a[:, 0].copy() for a in netgen.scenario_inputs(info.n_start, seed, 1))
+            got = {}
+            for how in ("phases", "step"):
+                g = [np.zeros(n, np.float32) for n in (info.n_start, info.n_start, info.n_cells)]
+                dp.dp_set_inputs(ctx, d, sp, tr)
+                if how == "step":
+                    dp.dp_step(ctx, d, cfg, g[0], g[1], g[2])
+                else:
+                    dp.dp_propagate(ctx, d, cfg)
+                    dp.dp_simulate(ctx, d, cfg)
+                    dp.dp_backward(ctx, d, cfg, g[0], g[1], g[2])
+                got[how] = g + nets(dp, ctx, d, info)
+            for a, b in zip(got["phases"], got["step"]):
+                np.testing.assert_array_equal(a, b)
+            assert got["step"][5][info.n_start:].any()
+    finally:
+        dp.dp_design_free(d)
