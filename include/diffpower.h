@@ -308,9 +308,11 @@ dp_status dp_step(dp_design *d, const dp_config *cfg, float *grad_sp_in, float *
 
 /* Device time in milliseconds of the last dp_step / dp_propagate / dp_simulate /
  * dp_backward per phase (CUDA events on the context stream; synchronises):
- * ms5[0] forward + model power, ms5[1] simulation levels (the bitwise cells;
- * in dp_step the startpoint generator runs beside the forward pass),
- * ms5[2] beta + hybrid power, ms5[3] backward, ms5[4] gradient outputs. */
+ * ms5[0] forward + model power, ms5[1] simulation levels (the bitwise cells),
+ * ms5[2] beta + hybrid power, ms5[3] backward, ms5[4] gradient outputs.  In
+ * dp_step the startpoint generator, and a sliced simulation with it, run beside
+ * the forward pass (ms5[1] is what is left of them), and both powers beside the
+ * backward pass. */
 dp_status dp_phase_times(dp_design *d, float *ms5);
 
 /* ------------------ batched scenarios (S scenarios per launch) ------------------

@@ -253,23 +253,17 @@ void repair_tags(dp_design *D, cudaStream_t s) {
 }
 
 // each q_* returns the first launch error (a cooperative launch reports it directly)
-// The forward pass and the model power.  ready (may be null) is recorded on s just before
+// The forward pass (q_forward: and the model power).  ready (may be null) is recorded on s just before
 // the first forward kernel: a branch forked there becomes ready with that kernel.
-cudaError_t q_forward(dp_design *D, const dp_config &c, cudaStream_t s, cudaEvent_t ready = nullptr) {
+cudaError_t q_forward_pass(dp_design *D, const dp_config &c, cudaStream_t s, cudaEvent_t ready = nullptr) {
     if (small_pass(D, c)) {   // the kernel advances the pass counter itself
         if (ready) cudaEventRecord(ready, s);
-        cudaError_t e = dp::launch_fwd_block(D->d, D->ops, c.tr_mode, D->block_threads, s);
-        if (e != cudaSuccess) return e;
-        dp::launch_power(D->d, false, power_K(c), 0, s);
-        return cudaGetLastError();
+        return dp::launch_fwd_block(D->d, D->ops, c.tr_mode, D->block_threads, s);
     }
     if (cluster_pass(D, c) || dataflow(D, c, 0)) {   // these advance it too
         if (ready) cudaEventRecord(ready, s);
-        cudaError_t e = cluster_pass(D, c) ? dp::launch_fwd_cluster(D->d, D->ops, D->cl, c.tr_mode, s)
-                                           : dp::launch_fwd_flow(D->d, D->ops, c.tr_mode, D->flow_grid[0], s);
-        if (e != cudaSuccess) return e;
-        dp::launch_power(D->d, false, power_K(c), 0, s);
-        return cudaGetLastError();
+        return cluster_pass(D, c) ? dp::launch_fwd_cluster(D->d, D->ops, D->cl, c.tr_mode, s)
+                                  : dp::launch_fwd_flow(D->d, D->ops, c.tr_mode, D->flow_grid[0], s);
     }
     dp::launch_bump(D->d.epoch, s);   // new parity for the stored (P, Q) pairs
     if (persistent(D, c, 0)) {
@@ -281,6 +275,11 @@ cudaError_t q_forward(dp_design *D, const dp_config &c, cudaStream_t s, cudaEven
         for (int l = 1; l <= D->d.n_levels; l++)
             dp::launch_fwd_level(D->d, D->ops, D->lvl_ptr[l - 1], D->lvl_ptr[l], s);
     }
+    return cudaGetLastError();
+}
+cudaError_t q_forward(dp_design *D, const dp_config &c, cudaStream_t s) {
+    cudaError_t e = q_forward_pass(D, c, s);
+    if (e != cudaSuccess) return e;
     dp::launch_power(D->d, false, power_K(c), 0, s);
     return cudaGetLastError();
 }
@@ -1182,7 +1181,7 @@ dp_status dp_step(dp_design *D, const dp_config *cfg, float *gsp, float *gtr, fl
         // earlier, the generator's blocks fill the SMs first when the GPU is idle at the
         // launch, and the cooperative forward kernel waits for room.
         cudaEventRecordWithFlags(D->ev[0], cs, cudaEventRecordExternal);
-        cudaError_t le = q_forward(D, *cfg, cs, D->fork);
+        cudaError_t le = q_forward_pass(D, *cfg, cs, D->fork);
         cudaEventRecordWithFlags(D->ev[1], cs, cudaEventRecordExternal);
         q_coef(D, *cfg, cs);   // beside the rest of the generator
         cudaStreamWaitEvent(D->cap_stream2, D->fork, 0);
@@ -1193,15 +1192,17 @@ dp_status dp_step(dp_design *D, const dp_config *cfg, float *gsp, float *gtr, fl
         cudaStreamWaitEvent(cs, D->join, 0);
         if (beside == 0 && le == cudaSuccess) le = q_sim_levels(D, *cfg, cs, D->ctx->sm_count);
         cudaEventRecordWithFlags(D->ev[2], cs, cudaEventRecordExternal);
-        if (le == cudaSuccess) le = q_hybrid(D, *cfg, cs);
+        dp::launch_hybrid(D->d, cfg->sim_words, cfg->tr_mode, cfg->beta_min, cfg->beta_max, cs);
         cudaEventRecordWithFlags(D->ev[3], cs, cudaEventRecordExternal);
-        // the cap and TR gradients need only the hybrid activities: a second branch
-        // writes them to the staging buffers beside the (latency-bound) backward pass
+        // the powers, which the reverse pass does not need, and the cap and TR gradients, which need
+        // only the hybrid activities, on a second branch beside the (latency-bound) backward pass
         cudaEventRecord(D->fork, cs);
         cudaStreamWaitEvent(D->cap_stream2, D->fork, 0);
         dp::launch_cap_grads(D->d, D->ops, cfg->grad_mode != 0, cfg->tr_mode, power_K(*cfg), D->st_gcl, D->st_gpin,
                              D->st_gtr, D->cap_stream2);
         cudaEventRecordWithFlags(D->ev_grads, D->cap_stream2, cudaEventRecordExternal);
+        dp::launch_power(D->d, false, power_K(*cfg), 0, D->cap_stream2);
+        dp::launch_power(D->d, true, power_K(*cfg), 1, D->cap_stream2);
         cudaEventRecord(D->join, D->cap_stream2);
         if (le == cudaSuccess) le = q_backward(D, *cfg, nullptr, cs, true);
         cudaStreamWaitEvent(cs, D->join, 0);
