@@ -312,7 +312,8 @@ dp_status dp_step(dp_design *d, const dp_config *cfg, float *grad_sp_in, float *
  * ms5[2] beta + hybrid power, ms5[3] backward, ms5[4] gradient outputs.  In
  * dp_step the startpoint generator, and a sliced simulation with it, run beside
  * the forward pass (ms5[1] is what is left of them), and both powers beside the
- * backward pass. */
+ * backward pass; a sliced dp_simulate that directly follows its dp_propagate runs
+ * beside that in the same way. */
 dp_status dp_phase_times(dp_design *d, float *ms5);
 
 /* ------------------ batched scenarios (S scenarios per launch) ------------------

@@ -227,10 +227,11 @@ dp::SliceShape sliced(const dp_design *D, const dp_config &c, int sms) {
     if (c.schedule != 0 || D->sl.slots == 0) return dp::SliceShape{0, 0};
     return dp::slice_shape(D->sl, D->d.n_cells, D->d.n_levels, c.sim_words, sms);
 }
-// SMs that the forward pass of a step leaves to the sliced simulation, which needs the generator's words only and has
+// SMs that the forward pass of a step, or of the dp_propagate just before, leaves to the sliced simulation, which needs the generator's words only and has
 // no waits of its own: beside a forward pass in one cluster or block the simulation hides its latency-bound levels
 // (0: the simulation follows the forward pass).  13,000 cells / 70 levels, 250 words: forward 78 us, generator 22 and
-// slices 43 on the branch; whole step 226 us one after the other, 196 so.
+// slices 43 on the branch; whole step 226 us one after the other, 195 so.  117,000 / 84, 256 words: forward 99 us,
+// generator 68 and slices 133; dp_propagate, dp_simulate and the results 381 us, 307 so.
 int step_slice_sms(const dp_design *D, const dp_config &c) {
     const int left = D->ctx->sm_count - (small_pass(D, c) ? 1 : dp::kClusterBlocks);
     if (!(small_pass(D, c) || cluster_pass(D, c)) || left < 1) return 0;
@@ -466,6 +467,7 @@ dp_status dp_sync(dp_ctx *c) {
 
 dp_status dp_set_stream(dp_ctx *c, void *cuda_stream) {
     if (!c) return DP_EINVAL;
+    if (c->stream != static_cast<cudaStream_t>(cuda_stream)) c->switched = true;
     c->stream = static_cast<cudaStream_t>(cuda_stream);
     return DP_OK;
 }
@@ -1039,7 +1041,9 @@ dp_status dp_propagate(dp_design *D, const dp_config *cfg) {
     rec(D, 0, st);
     cudaError_t le = q_forward(D, *cfg, st);
     rec(D, 1, st);
+    D->sim_ahead = false;
     if ((s = cuda_err(D->ctx, le, "dp_propagate")) != DP_OK) return s;
+    D->sim_ahead = !D->ctx->switched && !D->sim_captured && !capturing(st);
     D->fwd_valid = true;
     D->fwd_tr_mode = cfg->tr_mode;
     D->sim_valid = false;
@@ -1058,9 +1062,24 @@ dp_status dp_simulate(dp_design *D, const dp_config *cfg) {
     DeviceGuard g(D->ctx->device);
     if ((s = ensure_words(D, cfg->sim_words)) != DP_OK) return s;
     cudaStream_t st = D->ctx->stream;
+    const bool ahead = D->sim_ahead && !D->ctx->switched && !capturing(st);
+    D->sim_ahead = false;
+    if (capturing(st)) D->sim_captured = true;
     rec(D, 1, st);
-    q_sim_start(D, *cfg, st);
-    cudaError_t le = q_sim_levels(D, *cfg, st, D->ctx->sm_count);
+    const int beside = ahead ? step_slice_sms(D, *cfg) : 0;
+    cudaError_t le = cudaSuccess;
+    if (beside > 0) {   // as in dp_step, on a stream that joins again here
+        if ((s = ensure_step_streams(D)) != DP_OK) return s;
+        cudaStream_t o = D->out_stream;
+        le = cudaStreamWaitEvent(o, D->ev[0], 0);
+        q_sim_start(D, *cfg, o);
+        if (le == cudaSuccess) le = q_sim_levels(D, *cfg, o, beside);
+        cudaEventRecord(D->join, o);
+        cudaStreamWaitEvent(st, D->join, 0);
+    } else {
+        q_sim_start(D, *cfg, st);
+        le = q_sim_levels(D, *cfg, st, D->ctx->sm_count);
+    }
     rec(D, 2, st);
     if (le == cudaSuccess) le = q_hybrid(D, *cfg, st);
     rec(D, 3, st);
@@ -1166,6 +1185,7 @@ dp_status dp_step(dp_design *D, const dp_config *cfg, float *gsp, float *gtr, fl
     if ((s = ensure_words(D, cfg->sim_words)) != DP_OK) return s;
     if ((s = ensure_stage(D)) != DP_OK) return s;
     if ((s = ensure_step_streams(D)) != DP_OK) return s;
+    D->sim_ahead = false;
     cudaStream_t st = D->ctx->stream;
     if (!D->graph || std::memcmp(&D->graph_cfg, cfg, sizeof *cfg) != 0) {
         if (D->graph) { cudaGraphExecDestroy(D->graph); D->graph = nullptr; }

@@ -16,6 +16,7 @@ struct dp_ctx {
     int sm_count = 0;
     int clock_khz = 0;
     int *d_err = nullptr;   // device error word: a bounded wait gave up
+    bool switched = false;  // the calls have been on more than one stream
     unsigned timeouts = 0;  // times a synchronising call found it set
     std::string err;
 };
@@ -93,6 +94,10 @@ struct dp_design {
     // the step graph is done (ev_grads, recorded by the graph), and their completion
     cudaStream_t out_stream = nullptr;
     cudaEvent_t ev_grads = nullptr, ev_copies = nullptr;
+    // a dp_simulate that directly follows a dp_propagate may start beside it, at ev[0]: nothing queued on the stream
+    // since uses what it writes
+    bool sim_ahead = false;
+    bool sim_captured = false;   // a user's graph may hold a simulation of this design
     int grid[4] = {0, 0, 0, 0};   // persistent grids: forward, simulation, backward, wide simulation
     int flow_grid[3] = {0, 0, 0};  // dataflow grids: forward, simulation, reverse
     int block_threads = 0;         // > 0: the design fits the single-block passes, with this many threads

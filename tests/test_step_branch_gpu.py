@@ -42,3 +42,59 @@ def test_step_equals_its_phases(dp, ctx, library_text, spec, T):  # noqa: F811
             assert got["step"][5][info.n_start:].any()
     finally:
         dp.dp_design_free(d)
+
+
+@pytest.mark.parametrize("spec", [(900, 60, 9), (16000, 1200, 40)])
+def test_simulation_beside_the_pass_before(dp, library_text, spec):  # noqa: F811
+    """dp_simulate right after dp_propagate, again, after other calls, under capture and after a change of stream: the
+    counts are those of the step."""
+    torch = pytest.importorskip("torch")
+    cells, start, depth = spec
+    text = netgen.netlist_text(netgen.NetlistSpec(cells, start // 3, start - start // 3, depth, 16, 7))
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    c = dp.dp_create(0, a.cuda_stream)
+    d = dp.dp_design_load(c, text, library_text)
+    try:
+        info = dp.dp_design_info(d)
+        cfg = dp.config(grad_mode=2, tr_mode=0, sim_words=64)
+        inputs = [[x[:, 0].copy() for x in netgen.scenario_inputs(info.n_start, seed, 1)] for seed in (1, 2)]
+        ref = []
+        for i in inputs:
+            dp.dp_set_inputs(c, d, *i)
+            dp.dp_step(c, d, cfg, np.zeros(info.n_start, np.float32))
+            ref.append(nets(dp, c, d, info))
+
+        def check(k, what):
+            for x, y in zip(nets(dp, c, d, info), ref[k]):
+                np.testing.assert_array_equal(x, y, err_msg=what)
+
+        for k in (0, 1, 0, 1):
+            dp.dp_set_inputs(c, d, *inputs[k])
+            dp.dp_propagate(c, d, cfg)
+            dp.dp_simulate(c, d, cfg)
+            check(k, "after propagate")
+            dp.dp_simulate(c, d, cfg)
+            check(k, "again")
+            dp.dp_propagate(c, d, cfg)
+            dp.dp_step(c, d, cfg, np.zeros(info.n_start, np.float32))
+            dp.dp_simulate(c, d, cfg)
+            check(k, "after a step")
+        g = torch.cuda.CUDAGraph()
+        dp.dp_propagate(c, d, cfg)
+        a.synchronize()
+        with torch.cuda.graph(g, stream=a):
+            dp.dp_propagate(c, d, cfg)
+            dp.dp_simulate(c, d, cfg)
+        for _ in range(3):
+            with torch.cuda.stream(a):
+                dp.dp_propagate(c, d, cfg)
+                g.replay()
+                dp.dp_simulate(c, d, cfg)
+            check(1, "after a replay")
+        dp.dp_set_stream(c, b.cuda_stream)
+        dp.dp_propagate(c, d, cfg)
+        dp.dp_simulate(c, d, cfg)
+        check(1, "another stream")
+    finally:
+        dp.dp_design_free(d)
+        dp.dp_destroy(c)
