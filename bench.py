@@ -107,9 +107,9 @@ def batched_algorithmic_bytes(nn: int, ns: int, nc: int, ne: int, S: int) -> int
 TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,lts__t_bytes.sum,... (one launch),
     # 2M-cell step, 4th step (profiles/roofline_step_k_sim_wide_traffic.md)
-    "k_sim_wide": {"bytes": 224_526_080 + 162_210_304, "l2_bytes": 7_799_694_112, "workload": "roofline",
+    "k_sim_wide": {"bytes": 224_710_000 + 162_070_000, "l2_bytes": 7_781_440_000, "workload": "roofline",
                    "files": ["kern_persist.cu", "kern_common.cuh"],
-                   "sha": "d68f35c894eb261c"},
+                   "sha": "4f736507c33e30e4"},
 }
 
 
@@ -487,7 +487,7 @@ def bench_paper_shaped(dp, torch, dev, reps: int, pk: dict) -> dict:
 
 def bench_batched(args, dp, torch, dev, pk: dict) -> dict:
     """The 120,000-cell netlist x 512 input-activity scenarios (scenario-innermost SoA, one
-    launch per level for all scenarios, launch shapes from the library's autotuner):
+    launch per pass, or per level where the library's autotuner finds that faster):
     forward + power + reverse pass timed with CUDA events, L2 flushed before each
     repetition; then 200 projected ascent steps for all 512 starts (Algorithm 4) through
     the autograd Function, captured in a CUDA graph, and P_virus (Eq. 3) of the result."""
@@ -526,8 +526,9 @@ def bench_batched(args, dp, torch, dev, pk: dict) -> dict:
         fwd_shape, bwd_shape, tune_ms = dp.dp_batch_tuning(des.d)
         ab = batched_algorithmic_bytes(nn, ns, nc, ne, S)
         ach = ab / (ms * 1e-3) / 1e9
-        # kernels per forward + reverse pass: start + L levels, 2 power, seed, L levels + start
-        launches = (1 if ns else 0) + L + 2 + 1 + L + (1 if ns else 0)
+        # kernels per forward + reverse pass, at least (the dataflow passes; the level launches have one per
+        # level): preparation + pass, 2 power, seed, preparation + pass
+        launches = 2 + 2 + 1 + 2
 
         # Algorithm 4: 200 steps for all 512 starts, the proxy of Eq. 9 (tr_mode 1)
         steps = 200
@@ -544,7 +545,7 @@ def bench_batched(args, dp, torch, dev, pk: dict) -> dict:
                         "frac": ab / (statistics.median(warm) * 1e-3) / 1e9 / pk["hbm_gbs"]},
             "roofline": {"bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s",
                          "frac": ach / pk["hbm_gbs"], "algorithmic_bytes": ab, "traffic": None,
-                         "kernels": "k_fwdb_level / k_bwdb_level per level, k_powerb_*"},
+                         "kernels": "k_fwdb_flow, k_bwdb_flow, k_powerb_*"},
             "shapes": {"forward": list(fwd_shape), "backward": list(bwd_shape), "tuner_ms": list(tune_ms)},
             "gpu_launches_per_fwd_bwd": launches,
             "ascent": {"steps": steps, "starts": S, "eta": ETA, "proxy": "Eq. 9 (tr_mode 1)",
@@ -902,7 +903,7 @@ def main() -> None:
     pk = peaks()
     ab = algorithmic_bytes(nn, ns, nc, ne, cfg.sim_words)
     names = ["forward", "simulation", "hybrid", "backward", "outputs"]
-    kernel_of = {"forward": "k_fwd_persist", "simulation": "k_sim_wide", "backward": "k_bwd_persist"}
+    kernel_of = {"forward": "k_fwd_flow", "simulation": "k_sim_wide", "backward": "k_bwd_flow"}
     per_phase = {}
     for i, n in enumerate(names):
         t = float(ph[i]) * 1e-3

@@ -1043,7 +1043,7 @@ dp_status dp_propagate(dp_design *D, const dp_config *cfg) {
     rec(D, 1, st);
     D->sim_ahead = false;
     if ((s = cuda_err(D->ctx, le, "dp_propagate")) != DP_OK) return s;
-    D->sim_ahead = !D->ctx->switched && !D->sim_captured && !capturing(st);
+    D->sim_ahead = !D->ctx->switched && !D->sim_captured;
     D->fwd_valid = true;
     D->fwd_tr_mode = cfg->tr_mode;
     D->sim_valid = false;
@@ -1062,9 +1062,15 @@ dp_status dp_simulate(dp_design *D, const dp_config *cfg) {
     DeviceGuard g(D->ctx->device);
     if ((s = ensure_words(D, cfg->sim_words)) != DP_OK) return s;
     cudaStream_t st = D->ctx->stream;
-    const bool ahead = D->sim_ahead && !D->ctx->switched && !capturing(st);
+    const bool captured = capturing(st);
+    bool ahead = D->sim_ahead && !D->ctx->switched && !captured;
     D->sim_ahead = false;
-    if (capturing(st)) D->sim_captured = true;
+    if (captured) D->sim_captured = true;
+    if (ahead) {   // an event that a capture recorded cannot be waited for here
+        const cudaError_t q = cudaEventQuery(D->ev[0]);
+        ahead = q == cudaSuccess || q == cudaErrorNotReady;
+        cudaGetLastError();
+    }
     rec(D, 1, st);
     const int beside = ahead ? step_slice_sms(D, *cfg) : 0;
     cudaError_t le = cudaSuccess;

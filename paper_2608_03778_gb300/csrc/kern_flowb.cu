@@ -11,7 +11,8 @@
 //
 // What bounds it: the level launches end a grid and start the next per level, about 3 us, with 58 instructions per
 // (cell, scenario) to do in between (30 % of the issue slots used, 38 % of the warps active).  Without them a pass
-// runs into the L2: 50,000 cells / 44 levels x 256 scenarios forward 81 us with 29 M sectors, 120,000 / 48 x 512 217 us.
+// runs into the L2: 120,000 cells / 48 levels x 512 scenarios forward 217 us at 7.7 TB/s, reverse 385 us at 8.5 (reads
+// alone reach 8.1 to 8.7 on this part); 50,000 / 44 x 256 forward 81 us, more than half of its load sectors polls.
 // Four scenarios per thread spread the item's address and record work; 24 warps per SM forward, 20 reverse, where the
 // registers end without spills to speak of (a reverse pass whose 80 registers spilled wrote three times the
 // sectors).  Fetching the next item's record ahead cost more registers than it hid.  The reverse pass computes the

@@ -200,7 +200,7 @@ bool slice_fits(int64_t slots) {
 // A block takes about 0.35 + 0.12 NV ns per cell and 0.35 us per level, and the blocks go over the
 // SMs in waves; of two equal shapes the wider slice (a startpoint word is then read by fewer blocks).
 // The wide simulation takes about 2.3 us per level and its words' way through L2 (three gathers and a
-// store of 8 T bytes per cell at 4.8 TB/s).  Measured, this against that, with the generator:
+// store of 8 T bytes per cell at 4.8 TB/s).  Measured, this against that, with the generator (a third slower then):
 // 13,000 cells / 70 levels 64 words 45 / 193 us, 250 words 70 / 355; 117,000 / 84 64 words 122 / 262, 250
 // words 213 / 568; 120,000 / 48 120 / 181 and 276 / 385; 300,000 / 54 33 words 205 / 288, but 64 words
 // (two waves) 364 / 272, where the rule takes the wide one.

@@ -79,7 +79,15 @@ def test_simulation_beside_the_pass_before(dp, library_text, spec):  # noqa: F81
             dp.dp_step(c, d, cfg, np.zeros(info.n_start, np.float32))
             dp.dp_simulate(c, d, cfg)
             check(k, "after a step")
-        g = torch.cuda.CUDAGraph()
+        e, g = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+        dp.dp_propagate(c, d, cfg)
+        a.synchronize()
+        with torch.cuda.graph(e, stream=a):
+            dp.dp_propagate(c, d, cfg)
+        with torch.cuda.stream(a):
+            e.replay()
+            dp.dp_simulate(c, d, cfg)   # the pass before was captured
+        check(1, "after a captured pass")
         dp.dp_propagate(c, d, cfg)
         a.synchronize()
         with torch.cuda.graph(g, stream=a):
