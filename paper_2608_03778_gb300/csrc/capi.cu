@@ -1150,33 +1150,26 @@ dp_status dp_get_nets(dp_design *D, float *sp, float *tr, float *beta, float *tr
     cudaStream_t st = c->stream;
     const int64_t nn = D->d.n_nets;
     if (nn == 0) return DP_OK;
-    dp_status s = DP_OK;
-    float *stage = nullptr;
-    if (!on_device) {
-        if ((s = ensure_stage(D)) != DP_OK) return s;
-        stage = D->st_gcl;  // n_nets floats
+    if (on_device) {
+        dp::launch_nets_user(D->d, dp::NetOutputs{sp, tr, beta, trh, tg, on}, st);
+        return launch_check(c, "dp_get_nets");
     }
-    struct Out { void *dst; int kind; };
-    Out outs[6] = {{sp, 0}, {tr, 1}, {beta, 2}, {trh, 3}, {tg, 4}, {on, 5}};
-    for (auto &o : outs) {
-        if (!o.dst) continue;
-        void *dst = on_device ? o.dst : (void *)stage;
-        switch (o.kind) {
-            case 0: dp::launch_sp_user(D->d, (float *)dst, st); break;
-            case 1: dp::launch_gather_f32(D->d.tr, D->d.net_of_user, (float *)dst, nn, st); break;
-            case 2: dp::launch_gather_f32(D->d.beta, D->d.net_of_user, (float *)dst, nn, st); break;
-            case 3: dp::launch_trh_user(D->d, (float *)dst, st); break;
-            case 4: dp::launch_gather_u32(D->d.toggles, D->d.net_of_user, (uint32_t *)dst, nn, st); break;
-            case 5: dp::launch_gather_u32(D->d.ones, D->d.net_of_user, (uint32_t *)dst, nn, st); break;
-        }
+    dp_status s = ensure_stage(D);
+    if (s != DP_OK) return s;
+    float *const stage = D->st_gcl;  // n_nets floats
+    uint32_t *const words = reinterpret_cast<uint32_t *>(stage);
+    void *const outs[6] = {sp, tr, beta, trh, tg, on};
+    for (int k = 0; k < 6; k++) {
+        if (!outs[k]) continue;
+        dp::launch_nets_user(D->d, dp::NetOutputs{k == 0 ? stage : nullptr, k == 1 ? stage : nullptr,
+                                                  k == 2 ? stage : nullptr, k == 3 ? stage : nullptr,
+                                                  k == 4 ? words : nullptr, k == 5 ? words : nullptr}, st);
         if ((s = launch_check(c, "dp_get_nets")) != DP_OK) return s;
-        if (!on_device) {
-            cudaError_t e = cudaMemcpyAsync(o.dst, stage, 4 * (size_t)nn, cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            if (e != cudaSuccess) return cuda_err(c, e, "dp_get_nets");
-        }
+        cudaError_t e = cudaMemcpyAsync(outs[k], stage, 4 * (size_t)nn, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return cuda_err(c, e, "dp_get_nets");
     }
-    return on_device ? DP_OK : check_device_error(c);
+    return check_device_error(c);
 }
 
 dp_status dp_step(dp_design *D, const dp_config *cfg, float *gsp, float *gtr, float *gpin, float *gcl, double *watts,

@@ -92,10 +92,12 @@ void launch_power(const DevDesign &d, bool hybrid, double K, int slot, cudaStrea
 // outputs in user order: grad_cload (K alpha), grad_pincap (K sum fanin alpha), grad_tr_in (K beta C or 0)
 void launch_cap_grads(const DevDesign &d, const OpTable &ops, bool hybrid, int tr_mode, double K, float *grad_cload,
                       float *grad_pincap, float *grad_tr_in, cudaStream_t s);
-void launch_gather_f32(const float *src, const int32_t *idx, float *dst, int64_t n, cudaStream_t s);
-void launch_gather_u32(const uint32_t *src, const int32_t *idx, uint32_t *dst, int64_t n, cudaStream_t s);
-void launch_trh_user(const DevDesign &d, float *dst, cudaStream_t s);
-void launch_sp_user(const DevDesign &d, float *dst, cudaStream_t s);
+// per-net results of the single-scenario passes in user order (NULL: not wanted)
+struct NetOutputs {
+    float *sp, *tr, *beta, *trh;
+    uint32_t *toggles, *ones;
+};
+void launch_nets_user(const DevDesign &d, const NetOutputs &o, cudaStream_t s);
 
 // backward (kern_bwd.cu)
 void launch_bwd_level(const DevDesign &d, const OpTable &ops, int32_t c0, int32_t c1, int grad_mode, float K,
