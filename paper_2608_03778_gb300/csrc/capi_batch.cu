@@ -164,12 +164,17 @@ dp::GroupShape group_in_use(const dp_design *D, int tr_mode, int pass) {
     return group_rule(D, B.S);
 }
 
+// whether a design's batch of S can take the dataflow passes
+bool flow_can(const dp_design *D, int64_t S) {
+    return D->d.n_start > 0 && D->d.n_levels > 0 && D->d.n_levels <= dp::kFlowbLevels && S <= ((int64_t)1 << 28);
+}
+
 // scenarios per thread of the staged batch's dataflow pass (0 forward, 1 reverse); 0: not used.  The tuner takes them
 // where they are fastest; the results are bitwise those of the other passes.  (A design without startpoints has no
 // launch that would tell them of a pass by level launches.)
 int flow_in_use(const dp_design *D, int tr_mode, int pass) {
     const dp_batch &B = D->batch;
-    if (D->d.n_start == 0) return 0;
+    if (!flow_can(D, B.S)) return 0;
     dp::GroupShape g;
     int v = flow_env(B.S);
     if (v == 0 && !B.shape_from_env && !parse_group_env(&g) && B.tuned_S == B.S && !B.shapes_locked)
@@ -249,7 +254,7 @@ dp_status tune(dp_design *D) {
         }
     }
     float least[2] = {best[0], best[1]};
-    if (D->d.n_levels > 0 && D->d.n_start > 0)
+    if (flow_can(D, S))
         for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
             const int v = flow_v(S, W);
             const float t = timed(   // the first run also brings the arrays to rest

@@ -215,7 +215,9 @@ cudaError_t launch_fwdb_group(const DevDesign &d, const BatchBufs &b, const OpTa
 cudaError_t launch_bwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
                               cudaStream_t s);
 // the same passes in one launch each without barriers between levels (kern_flowb.cu): v scenarios
-// per thread (S a multiple of v; in the lag-one mode at most 2); edges: the elements of gfo
+// per thread (S a multiple of v; in the lag-one mode at most 2); edges: the elements of gfo.  At most kFlowbLevels
+// levels (their bounds are in shared memory) and 2^28 scenarios (a row's bytes are counted in 32 bits).
+constexpr int kFlowbLevels = 8192;
 cudaError_t launch_fwdb_flow(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, int v, int sms,
                              cudaStream_t s);
 cudaError_t launch_bwdb_flow(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, int v,

@@ -157,3 +157,14 @@ def test_dataflow_in_a_graph(dp, library_text):  # noqa: F811
     finally:
         dp.dp_design_free(d)
         dp.dp_destroy(c)
+
+
+def test_more_levels_than_the_dataflow_passes_take(dp, ctx):  # noqa: F811
+    """a chain of inverters and buffers beyond their level bounds runs as before"""
+    n = 8200
+    lib = "cell BUF Z 0.7 A\ncell INV ZN 0.6 !A\nseq DFF D Q 0.8\n"
+    lines = [f"net n{i} 1.0" for i in range(n + 1)] + ["input n0"]
+    lines += [f"cell u{i} " + (f"INV A=n{i} ZN=n{i + 1}" if i % 3 else f"BUF A=n{i} Z=n{i + 1}") for i in range(n)]
+    text = "\n".join(lines) + "\n"
+    sp, tr = netgen.scenario_inputs(1, 3, 8)
+    same(run(dp, ctx, text, lib, 1, sp, tr, 1), run(dp, ctx, text, lib, "level", sp, tr, 1), "chain")
