@@ -193,7 +193,7 @@ int flow_v(int64_t S, int64_t W) {
 }
 
 // Autotuner: times the forward and the reverse pass of this design at this S (CUDA events) for every candidate shape
-// of the level launches, for the dataflow passes, and for a small batch for a few group shapes, and keeps the
+// of the level launches, and for the dataflow passes, or for a single scenario for a group shape, and keeps the
 // fastest of each.  The first shape of a kernel runs once before it is timed; a shape that is
 // more than a tenth slower than the best is not timed twice.  Runs on the staged inputs; the results it
 // leaves are overwritten by the next dp_propagate.
@@ -253,8 +253,12 @@ dp_status tune(dp_design *D) {
             }
         }
     }
+    // One scenario by groups (31 of 32 lanes of a dataflow item would be idle: 20,000 cells / 38 levels 70 + 94 us against
+    // 90 + 99), from two on by dataflow (S = 2: 48 + 56 against 49 + 56 at 2,000 / 24, and ahead from there)
     float least[2] = {best[0], best[1]};
-    if (flow_can(D, S))
+    const dp::GroupShape g{2, 1, 16, 512};
+    const bool groups = S == 1 && D->d.n_levels > 0 && W <= 6000;
+    if (!groups && flow_can(D, S))
         for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
             const int v = flow_v(S, W);
             const float t = timed(   // the first run also brings the arrays to rest
@@ -268,29 +272,19 @@ dp_status tune(dp_design *D) {
                 (pass == 0 ? B.fwd_flow : B.bwd_flow) = v;
             }
         }
-    // groups: from eight scenarios the dataflow passes were faster at every size
-    if (D->d.n_levels > 0 && S < 8 && W * S <= 150000 && W <= 6000) {
-        dp::GroupShape cand[4];
-        int n = 0;
-        for (int lanes : {2, 4})
-            if (W * lanes <= 16384) cand[n++] = dp::GroupShape{lanes, 1, 16, 512};
-        if (W * 8 <= 16384) cand[n++] = dp::GroupShape{8, 1, 16, 512};
-        cand[n++] = dp::GroupShape{8, 1, 8, 512};
-        for (int pass = 0; pass < 2 && e == cudaSuccess; pass++)
-            for (int i = 0; i < n; i++) {
-                const float t = timed(
-                    [&] {
-                        return pass == 0 ? dp::launch_fwdb_group(D->d, B.b, D->ops, 0, cand[i], st)
-                                         : dp::launch_bwdb_group(D->d, B.b, D->ops, 0, cand[i], st);
-                    },
-                    i == 0, least[pass]);
-                if (t < least[pass]) {
-                    least[pass] = t;
-                    (pass == 0 ? B.fwd_group : B.bwd_group) = cand[i];
-                    (pass == 0 ? B.fwd_flow : B.bwd_flow) = 0;
-                }
+    if (groups)
+        for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
+            const float t = timed(
+                [&] {
+                    return pass == 0 ? dp::launch_fwdb_group(D->d, B.b, D->ops, 0, g, st)
+                                     : dp::launch_bwdb_group(D->d, B.b, D->ops, 0, g, st);
+                },
+                true, least[pass]);
+            if (t < least[pass]) {
+                (pass == 0 ? B.fwd_group : B.bwd_group) = g;
+                (pass == 0 ? B.fwd_flow : B.bwd_flow) = 0;
             }
-    }
+        }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (e == cudaSuccess) e = cudaGetLastError();
