@@ -109,7 +109,7 @@ TRAFFIC = {
     # 2M-cell step, 4th step (profiles/roofline_step_k_sim_wide_traffic.md)
     "k_sim_wide": {"bytes": 224_710_000 + 162_070_000, "l2_bytes": 7_781_440_000, "workload": "roofline",
                    "files": ["kern_persist.cu", "kern_common.cuh"],
-                   "sha": "4f736507c33e30e4"},
+                   "sha": "d68f35c894eb261c"},
 }
 
 

@@ -700,7 +700,8 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
         uint32_t lut = 0;
         if (k <= 3)
             for (uint32_t m = 0; m < 8; m++) lut |= ((tt >> (m & ((1u << k) - 1u))) & 1u) << m;
-        D->ops.e[i] = tt | (k << 16) | (dp::cell_class(k, tt) << 19) | (lut << 24);
+        D->ops.e[i] = tt | (k << 16) | (lut << 24);
+        D->cell_ops.e[i] = D->ops.e[i] | (dp::cell_class(k, tt) << 19);
     }
     const size_t nn = (size_t)d.n_nets, nc = (size_t)d.n_cells, ns = (size_t)d.n_start;
     dp_status s = DP_OK;

@@ -234,15 +234,15 @@ dp_status tune(dp_design *D) {
     float best[2] = {1e30f, 1e30f};
     dp::BatchShape pick[2] = {B.fwd_shape, B.bwd_shape};
     for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
-        if (pass == 1) dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), 0, pick[0], st);
+        if (pass == 1) dp::launch_fwdb(D->d, B.b, D->cell_ops, D->lvl_ptr.data(), 0, pick[0], st);
         int seen = 0;
         for (const dp::BatchShape &sh : kShapes) {
             if (sh.bx > limit) continue;
             const int v = S % sh.v ? 1 : sh.v;
             const float t = timed(
                 [&] {
-                    if (pass == 0) dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), 0, sh, st);
-                    else dp::launch_bwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), 0, sh, st);
+                    if (pass == 0) dp::launch_fwdb(D->d, B.b, D->cell_ops, D->lvl_ptr.data(), 0, sh, st);
+                    else dp::launch_bwdb(D->d, B.b, D->cell_ops, D->lvl_ptr.data(), 0, sh, st);
                     return cudaSuccess;
                 },
                 (seen & v) == 0, best[pass]);
@@ -263,8 +263,8 @@ dp_status tune(dp_design *D) {
             const int v = flow_v(S, W);
             const float t = timed(   // the first run also brings the arrays to rest
                 [&] {
-                    return pass == 0 ? dp::launch_fwdb_flow(D->d, B.b, D->ops, 0, v, c->sm_count, st)
-                                     : dp::launch_bwdb_flow(D->d, B.b, D->ops, 0, v, D->n_edges * B.cap, c->sm_count, st);
+                    return pass == 0 ? dp::launch_fwdb_flow(D->d, B.b, D->cell_ops, 0, v, c->sm_count, st)
+                                     : dp::launch_bwdb_flow(D->d, B.b, D->cell_ops, 0, v, D->n_edges * B.cap, c->sm_count, st);
                 },
                 true, least[pass]);
             if (t < least[pass]) {
@@ -276,8 +276,8 @@ dp_status tune(dp_design *D) {
         for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
             const float t = timed(
                 [&] {
-                    return pass == 0 ? dp::launch_fwdb_group(D->d, B.b, D->ops, 0, g, st)
-                                     : dp::launch_bwdb_group(D->d, B.b, D->ops, 0, g, st);
+                    return pass == 0 ? dp::launch_fwdb_group(D->d, B.b, D->cell_ops, 0, g, st)
+                                     : dp::launch_bwdb_group(D->d, B.b, D->cell_ops, 0, g, st);
                 },
                 true, least[pass]);
             if (t < least[pass]) {
@@ -304,20 +304,20 @@ namespace dpi {
 cudaError_t batch_forward(dp_design *D, int tr_mode, cudaStream_t s) {
     dp_batch &B = D->batch;
     const int v = flow_in_use(D, tr_mode, 0);
-    if (v > 0) return dp::launch_fwdb_flow(D->d, B.b, D->ops, tr_mode, v, D->ctx->sm_count, s);
+    if (v > 0) return dp::launch_fwdb_flow(D->d, B.b, D->cell_ops, tr_mode, v, D->ctx->sm_count, s);
     const dp::GroupShape g = group_in_use(D, tr_mode, 0);
-    if (g.v > 0) return dp::launch_fwdb_group(D->d, B.b, D->ops, tr_mode, g, s);
-    dp::launch_fwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), tr_mode, B.fwd_shape, s);
+    if (g.v > 0) return dp::launch_fwdb_group(D->d, B.b, D->cell_ops, tr_mode, g, s);
+    dp::launch_fwdb(D->d, B.b, D->cell_ops, D->lvl_ptr.data(), tr_mode, B.fwd_shape, s);
     return cudaGetLastError();
 }
 
 cudaError_t batch_reverse(dp_design *D, int tr_mode, cudaStream_t s) {
     dp_batch &B = D->batch;
     const int v = flow_in_use(D, tr_mode, 1);
-    if (v > 0) return dp::launch_bwdb_flow(D->d, B.b, D->ops, tr_mode, v, D->n_edges * B.cap, D->ctx->sm_count, s);
+    if (v > 0) return dp::launch_bwdb_flow(D->d, B.b, D->cell_ops, tr_mode, v, D->n_edges * B.cap, D->ctx->sm_count, s);
     const dp::GroupShape g = group_in_use(D, tr_mode, 1);
-    if (g.v > 0) return dp::launch_bwdb_group(D->d, B.b, D->ops, tr_mode, g, s);
-    dp::launch_bwdb(D->d, B.b, D->ops, D->lvl_ptr.data(), tr_mode, B.bwd_shape, s);
+    if (g.v > 0) return dp::launch_bwdb_group(D->d, B.b, D->cell_ops, tr_mode, g, s);
+    dp::launch_bwdb(D->d, B.b, D->cell_ops, D->lvl_ptr.data(), tr_mode, B.bwd_shape, s);
     return cudaGetLastError();
 }
 

@@ -53,7 +53,7 @@ struct dp_batch {
 struct dp_design {
     dp_ctx *ctx = nullptr;
     dp::DevDesign d{};
-    dp::OpTable ops{};
+    dp::OpTable ops{}, cell_ops{};   // the function table; the same with the functions' classes, for the batched passes
     std::vector<int32_t> lvl_ptr;
     int64_t n_edges = 0;
     int32_t n_ops = 0;

@@ -9,7 +9,7 @@ namespace dp {
 
 constexpr uint32_t kMask24 = 0xFFFFFFu;
 
-__device__ __forceinline__ int op_arity(const OpTable &t, uint32_t op) { return (int)((t.e[op] >> 16) & 7u); }
+__device__ __forceinline__ int op_arity(const OpTable &t, uint32_t op) { return (int)((t.e[op] >> 16) & 0xFFu); }
 __device__ __forceinline__ uint32_t op_lut(const OpTable &t, uint32_t op) { return t.e[op] >> 24; }
 __device__ __forceinline__ uint32_t op_tt(const OpTable &t, uint32_t op) { return t.e[op] & 0xFFFFu; }
 

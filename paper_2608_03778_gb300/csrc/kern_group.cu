@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kGroupThreads) k_fwdb_group(const uint4 *__res
             if (c < c1) r = fanin[c];
             const uint32_t op = cur.x >> 24;
             const uint32_t n[4] = {cur.x & kMask24, cur.y, cur.z, cur.w};
-            const int k = op_arity(ops, op);
+            const int k = (int)((ops.e[op] >> 16) & 7u);
             Row2<V> x[4], o;
             Row1<V> t[4], ot;
 #pragma unroll
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kGroupThreads) k_bwdb_group(
             const uint32_t op = cur.x >> 24;
             const uint32_t nid[4] = {cur.x & kMask24, cur.y, cur.z, cur.w};
             const int pos[4] = {pos4.x, pos4.y, pos4.z, pos4.w};
-            const int k = op_arity(ops, op);
+            const int k = (int)((ops.e[op] >> 16) & 7u);
             Row2<V> x[4], self;
             Row1<V> t[4], a, b;
 #pragma unroll

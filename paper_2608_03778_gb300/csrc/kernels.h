@@ -21,7 +21,7 @@ inline uint32_t cell_class(uint32_t k, uint32_t tt) {
 }
 
 // Per-design function table passed by value to kernels (lives in the
-// constant bank): entry = truth table (bits 0..15) | arity << 16 | class << 19 |
+// constant bank): entry = truth table (bits 0..15) | arity << 16 | (batched passes only) class << 19 |
 // (for arity <= 3) the 8-bit LOP3 table of the function << 24, whose entry
 // 4 x2 + 2 x1 + x0 is f(x0, x1, x2) (inputs beyond the arity ignored).
 struct OpTable {
