@@ -122,9 +122,7 @@ bool parse_shape_env(dp::BatchShape *f, dp::BatchShape *b) {
 bool parse_group_env(dp::GroupShape *g) {
     const char *v = std::getenv("DP_BATCH_GROUP");
     if (!v || std::sscanf(v, "%d,%d,%d,%d", &g->lanes, &g->v, &g->blocks, &g->threads) != 4) return false;
-    return (g->v == 1 || g->v == 2 || g->v == 4) && g->blocks >= 1 && g->blocks <= 16 &&
-           (g->blocks & (g->blocks - 1)) == 0 && g->threads >= 32 && g->threads <= 512 && (g->threads & 31) == 0 &&
-           g->lanes >= 1 && g->lanes <= 32 && g->threads % g->lanes == 0;
+    return dp::group_ok(*g) && g->lanes <= 32;
 }
 
 // DP_BATCH_FLOW = "v": the dataflow passes wherever v divides S

@@ -194,6 +194,7 @@ __global__ void __launch_bounds__(kGroupThreads) k_bwdb_group(
 
 template <class... KArgs, class... Args>
 cudaError_t launch_group(void (*kern)(KArgs...), GroupShape sh, int64_t S, cudaStream_t s, Args... args) {
+    if (!group_ok(sh) || S % sh.v != 0) return cudaErrorInvalidConfiguration;
     cudaError_t e = cudaSuccess;
     if (sh.blocks > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
@@ -216,7 +217,7 @@ cudaError_t launch_group(void (*kern)(KArgs...), GroupShape sh, int64_t S, cudaS
 
 cudaError_t launch_fwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
                               cudaStream_t s) {
-    if (tr_mode == 2 && sh.v == 4) sh.v = 2, sh.lanes *= 2;   // the lag-one state takes two scenarios' registers
+    sh = group_for(sh, tr_mode);
     auto go = [&](auto kern) {
         return launch_group(kern, sh, b.S, s, d.fanin, b.pq, b.tq, b.sp_in, b.tr_in, d.lvl, d.n_levels, d.n_start, b.S,
                             sh.lanes, ops, b.state);
@@ -227,7 +228,7 @@ cudaError_t launch_fwdb_group(const DevDesign &d, const BatchBufs &b, const OpTa
 
 cudaError_t launch_bwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
                               cudaStream_t s) {
-    if (tr_mode == 2 && sh.v == 4) sh.v = 2, sh.lanes *= 2;
+    sh = group_for(sh, tr_mode);
     auto go = [&](auto kern) {
         return launch_group(kern, sh, b.S, s, d.fanin, d.fout_ptr, (const int4 *)d.edge_fpos, b.pq, b.tq, d.cload, b.dcl,
                             b.ks, b.gfo, b.gfo2, b.gsp, b.gtr, d.lvl, d.n_levels, d.n_start, b.S, sh.lanes, tr_mode,

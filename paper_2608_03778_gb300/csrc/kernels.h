@@ -210,6 +210,21 @@ void launch_bwdl(const DevDesign &d, const BatchBufs &b, const OpTable &ops, con
 struct GroupShape {
     int lanes = 0, v = 0, blocks = 0, threads = 0;
 };
+// a block is whole rows of lanes threads, at least one (a stride of no rows would never end), in whole warps
+inline bool group_ok(const GroupShape &g) {
+    return (g.v == 1 || g.v == 2 || g.v == 4) && g.blocks >= 1 && g.blocks <= 16 && (g.blocks & (g.blocks - 1)) == 0 &&
+           g.threads >= 32 && g.threads <= 512 && (g.threads & 31) == 0 && g.lanes >= 1 && g.lanes <= g.threads &&
+           g.threads % g.lanes == 0;
+}
+// the shape as a pass runs it: the lag-one state takes two scenarios' registers, in twice the lanes where they still
+// make whole rows
+inline GroupShape group_for(GroupShape g, int tr_mode) {
+    if (tr_mode == 2 && g.v == 4) {
+        g.v = 2;
+        if (g.threads % (2 * g.lanes) == 0) g.lanes *= 2;
+    }
+    return g;
+}
 cudaError_t launch_fwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
                               cudaStream_t s);
 cudaError_t launch_bwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
