@@ -3,8 +3,8 @@
 // item waits only for its own inputs.  The data is its own ready flag.
 //
 // Forward: the low part of a stored P never has bit 30 set (|lo| < 2 for |P| < 2^25), so the bit carries the
-// parity of the pass that wrote it, in the same single-copy atomic word; everything that reads a
-// stored P drops it (pair_get).  Reverse: an edge's contribution is written once and read once, and its
+// parity of the pass that wrote it; a stored P (hi, lo) is written and read as one 64-bit element, so the bit speaks
+// for both halves.  Everything that reads a stored P drops it (pair_get).  Reverse: an edge's contribution is written once and read once, and its
 // reader leaves kNotYet behind for the next pass.  k_flowb_prep brings both to rest where another pass wrote
 // the arrays in between.  Lag-one mode: a net's T has no bit to spare; it starts as kNotYet in every pass (27 MB, 6 us
 // at 50,000 x 128).
@@ -41,23 +41,30 @@ __device__ __forceinline__ uint32_t ld_word(const void *p) {
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-// rows of single-copy atomic elements, read through L2 at the point of the call
+// Rows between warps of the grid, through L2, by relaxed accesses whose elements are single-copy atomic: a (hi, lo) or
+// (P, T) pair is one 64-bit element, so a reader that sees the tag in one half has the other half of the same store.
+// (The elements of a vector access are accesses of their own: four-byte elements would let a new lo come with an old hi.)
+__device__ __forceinline__ uint64_t pair_bits(const float2 &v) {
+    return (uint64_t)__float_as_uint(v.x) | (uint64_t)__float_as_uint(v.y) << 32;
+}
+__device__ __forceinline__ float2 bits_pair(uint64_t b) {
+    return make_float2(__uint_as_float((uint32_t)b), __uint_as_float((uint32_t)(b >> 32)));
+}
 template <int V>
 __device__ __forceinline__ Row2<V> ld_row(const float2 *p) {
-    Row2<V> r;
+    uint64_t b[V];
     if constexpr (V == 1)
-        asm volatile("ld.relaxed.gpu.global.v2.f32 {%0,%1}, [%2];" : "=f"(r.v[0].x), "=f"(r.v[0].y) : "l"(p) : "memory");
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(b[0]) : "l"(p) : "memory");
     else if constexpr (V == 2)
-        asm volatile("ld.relaxed.gpu.global.v4.f32 {%0,%1,%2,%3}, [%4];"
-                     : "=f"(r.v[0].x), "=f"(r.v[0].y), "=f"(r.v[1].x), "=f"(r.v[1].y)
-                     : "l"(p)
-                     : "memory");
+        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0,%1}, [%2];" : "=l"(b[0]), "=l"(b[1]) : "l"(p) : "memory");
     else
-        asm volatile("ld.relaxed.gpu.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=f"(r.v[0].x), "=f"(r.v[0].y), "=f"(r.v[1].x), "=f"(r.v[1].y), "=f"(r.v[2].x), "=f"(r.v[2].y),
-                       "=f"(r.v[3].x), "=f"(r.v[3].y)
+        asm volatile("ld.relaxed.gpu.global.v4.u64 {%0,%1,%2,%3}, [%4];"
+                     : "=l"(b[0]), "=l"(b[1]), "=l"(b[2]), "=l"(b[3])
                      : "l"(p)
                      : "memory");
+    Row2<V> r;
+#pragma unroll
+    for (int i = 0; i < V; i++) r.v[i] = bits_pair(b[i]);
     return r;
 }
 template <int V>
@@ -73,6 +80,29 @@ __device__ __forceinline__ Row1<V> ld_row(const float *p) {
                      : "l"(p)
                      : "memory");
     return r;
+}
+template <int V>
+__device__ __forceinline__ void put_row(float2 *p, const Row2<V> &r) {
+    if constexpr (V == 1)
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(pair_bits(r.v[0])) : "memory");
+    else if constexpr (V == 2)
+        asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1,%2};" ::"l"(p), "l"(pair_bits(r.v[0])), "l"(pair_bits(r.v[1]))
+                     : "memory");
+    else
+        asm volatile("st.relaxed.gpu.global.v4.u64 [%0], {%1,%2,%3,%4};" ::"l"(p), "l"(pair_bits(r.v[0])),
+                     "l"(pair_bits(r.v[1])), "l"(pair_bits(r.v[2])), "l"(pair_bits(r.v[3]))
+                     : "memory");
+}
+template <int V>
+__device__ __forceinline__ void put_row(float *p, const Row1<V> &r) {
+    if constexpr (V == 1)
+        asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(p), "f"(r.v[0]) : "memory");
+    else if constexpr (V == 2)
+        asm volatile("st.relaxed.gpu.global.v2.f32 [%0], {%1,%2};" ::"l"(p), "f"(r.v[0]), "f"(r.v[1]) : "memory");
+    else
+        asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(p), "f"(r.v[0]), "f"(r.v[1]), "f"(r.v[2]),
+                     "f"(r.v[3])
+                     : "memory");
 }
 
 // true (in every lane) when a wait that began at t0 has to give up
@@ -105,10 +135,6 @@ struct Edge<true> {
 };
 __device__ __forceinline__ bool waits(float v) { return __float_as_uint(v) == kNotYet; }
 __device__ __forceinline__ bool waits(const float2 &v) { return waits(v.x) || waits(v.y); }
-template <int V>
-__device__ __forceinline__ void put(float *p, const Row1<V> &r) { st1<V>(p, r); }
-template <int V>
-__device__ __forceinline__ void put(float2 *p, const Row2<V> &r) { st2<V>(p, r); }
 
 // A warp's walk through the items: a net of the level and one of m chunks of 32 V scenarios.
 struct Walk {
@@ -258,8 +284,8 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
 #pragma unroll
             for (int i = 0; i < V; i++)
                 o.v[i].y = __uint_as_float((__float_as_uint(o.v[i].y) & ~kTagBit) | tag);
-            st2<V>(row_at(pqs, c, S), o);
-            if (LAG) st1<V>(row_at(tqs, c, S), ot);
+            put_row<V>(row_at(pqs, c, S), o);
+            if (LAG) put_row<V>(row_at(tqs, c, S), ot);
         }
     }
     if (last_block(state + 3)) {
@@ -383,7 +409,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
                         if constexpr (LAG) a.v[i] += u[j].v[i].x, b.v[i] += u[j].v[i].y;
                         else a.v[i] += u[j].v[i];
                     }
-                    if (on) put(row_at(gs, (uint32_t)(p + j), S), rest);
+                    if (on) put_row(row_at(gs, (uint32_t)(p + j), S), rest);
                 }
         }
         if (!on) continue;
@@ -410,7 +436,7 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
                                              __fmul_rn(b.v[i], dt[j].v[i]));
                     else g.v[i] = __fmul_rn(a.v[i], d[j].v[i]);
                 }
-                put(row_at(gs, pos[j], S), g);
+                put_row(row_at(gs, pos[j], S), g);
             }
     }
     if (last_block(state + 4)) state[LAG ? 5 : 2] = ld_word(err) ? 0u : 1u;
