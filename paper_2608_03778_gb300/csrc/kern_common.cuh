@@ -67,19 +67,27 @@ __device__ __forceinline__ ff ff_div(ff a, ff b) {
 struct pair_ff {
     ff p, q;
 };
-// Storage tag: P.hi and Q.hi are never negative, so their sign bits carry the
-// parity of the forward pass that wrote them (a counter in device memory,
+// Storage tag: probabilities have no sign, so the sign bits of P.hi and Q.hi carry
+// the parity of the forward pass that wrote them (a counter in device memory,
 // advanced once per pass).  A reader of the dataflow schedule knows a pair is
-// from the current pass when both tags match; every reader masks the tags.
+// from the current pass when both tags match; every reader masks the tags.  A
+// sign that is there all the same (an input of -0.0, or one outside [0, 1] that
+// a device caller brought) is dropped where the tag is written, or a reader
+// would wait for a parity that never comes.  The instruction is spelled out:
+// of an OR with a sign bit known at compile time the compiler makes -|v|, which
+// loses the sign of a NaN.
 __device__ __forceinline__ float untag(float v) { return __int_as_float(__float_as_int(v) & 0x7FFFFFFF); }
 __device__ __forceinline__ float4 pq_decode(float4 v) { return make_float4(untag(v.x), v.y, untag(v.z), v.w); }
 __device__ __forceinline__ pair_ff pair_load(const float4 &v) {
     return pair_ff{ff{untag(v.x), v.y}, ff{untag(v.z), v.w}};
 }
 __device__ __forceinline__ float4 pair_store(const pair_ff &a, uint32_t parity) {
-    const int t = (int)(parity << 31);
-    return make_float4(__int_as_float(__float_as_int(a.p.hi) | t), a.p.lo, __int_as_float(__float_as_int(a.q.hi) | t),
-                       a.q.lo);
+    auto tagged = [parity](float v) {
+        uint32_t o;   // (v & 0x7FFFFFFF) | parity << 31
+        asm("lop3.b32 %0, %1, 0x7FFFFFFF, %2, 0xEA;" : "=r"(o) : "r"(__float_as_uint(v)), "r"(parity << 31));
+        return __uint_as_float(o);
+    };
+    return make_float4(tagged(a.p.hi), a.p.lo, tagged(a.q.hi), a.q.lo);
 }
 // writes a tagged pair as two 8-byte halves (P.hi, P.lo) and (Q.hi, Q.lo), each
 // single-copy atomic, so a concurrent reader never sees a half torn
