@@ -974,6 +974,7 @@ dp_status dp_set_inputs(dp_design *D, const float *sp, const float *tr, int32_t 
                                    "input SP and TR must lie in [0,1] (startpoint " + std::to_string(k) + ")");
     }
     DeviceGuard g(c->device);
+    note_capture(D);
     cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     cudaError_t e = cudaSuccess;
     if (ns) e = cudaMemcpyAsync(D->d.sp_in, sp, sizeof(float) * (size_t)ns, kind, c->stream);
@@ -995,6 +996,7 @@ dp_status dp_set_pincap(dp_design *D, const int32_t *cells, const float *caps, i
     if (!cells && n != D->d.n_cells) return set_err(c, DP_EINVAL, "a NULL cell list needs one cap per cell");
     if (n == 0) return DP_OK;
     DeviceGuard g(c->device);
+    note_capture(D);
     int32_t *dc = nullptr;
     float *dv = nullptr;
     cudaError_t e = cudaSuccess;
@@ -1037,6 +1039,7 @@ dp_status dp_propagate(dp_design *D, const dp_config *cfg) {
     if (D->batched) return batch_propagate(D, *cfg);
     if (cfg->tr_mode == 2) return set_err(D->ctx, DP_EUNSUPPORTED, "the lag-one mode runs on batched inputs");
     DeviceGuard g(D->ctx->device);
+    note_capture(D);
     cudaStream_t st = D->ctx->stream;
     repair_tags(D, st);
     rec(D, 0, st);
@@ -1044,7 +1047,7 @@ dp_status dp_propagate(dp_design *D, const dp_config *cfg) {
     rec(D, 1, st);
     D->sim_ahead = false;
     if ((s = cuda_err(D->ctx, le, "dp_propagate")) != DP_OK) return s;
-    D->sim_ahead = !D->ctx->switched && !D->sim_captured;
+    D->sim_ahead = !D->ctx->switched && !D->captured;
     D->fwd_valid = true;
     D->fwd_tr_mode = cfg->tr_mode;
     D->sim_valid = false;
@@ -1063,10 +1066,9 @@ dp_status dp_simulate(dp_design *D, const dp_config *cfg) {
     DeviceGuard g(D->ctx->device);
     if ((s = ensure_words(D, cfg->sim_words)) != DP_OK) return s;
     cudaStream_t st = D->ctx->stream;
-    const bool captured = capturing(st);
-    bool ahead = D->sim_ahead && !D->ctx->switched && !captured;
+    note_capture(D);
+    bool ahead = D->sim_ahead && !D->ctx->switched && !D->captured;
     D->sim_ahead = false;
-    if (captured) D->sim_captured = true;
     if (ahead) {   // an event that a capture recorded cannot be waited for here
         const cudaError_t q = cudaEventQuery(D->ev[0]);
         ahead = q == cudaSuccess || q == cudaErrorNotReady;
@@ -1103,6 +1105,7 @@ dp_status dp_get_power(dp_design *D, int hybrid, double *watts, int on_device) {
     if (!D->fwd_valid || (hybrid && !D->sim_valid))
         return set_err(D->ctx, DP_ESTATE, hybrid ? "hybrid power needs dp_simulate" : "power needs dp_propagate");
     DeviceGuard g(D->ctx->device);
+    note_capture(D);
     cudaError_t e = cudaMemcpyAsync(watts, D->d.power + (hybrid ? 1 : 0), sizeof(double),
                                     on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, D->ctx->stream);
     if (e != cudaSuccess) return cuda_err(D->ctx, e, "dp_get_power");
@@ -1123,6 +1126,7 @@ dp_status dp_backward(dp_design *D, const dp_config *cfg, float *gsp, float *gtr
     if (cfg->grad_mode != 0 && !D->sim_valid)
         return set_err(D->ctx, DP_ESTATE, "hybrid gradients need dp_simulate");
     DeviceGuard g(D->ctx->device);
+    note_capture(D);
     cudaStream_t st = D->ctx->stream;
     rec(D, 3, st);
     q_coef(D, *cfg, st);
@@ -1148,6 +1152,7 @@ dp_status dp_get_nets(dp_design *D, float *sp, float *tr, float *beta, float *tr
     if ((sp || tr) && !D->fwd_valid) return set_err(c, DP_ESTATE, "SP/TR need dp_propagate");
     if ((beta || trh || tg || on) && !D->sim_valid) return set_err(c, DP_ESTATE, "simulation outputs need dp_simulate");
     DeviceGuard g(c->device);
+    note_capture(D);
     cudaStream_t st = c->stream;
     const int64_t nn = D->d.n_nets;
     if (nn == 0) return DP_OK;
@@ -1182,6 +1187,7 @@ dp_status dp_step(dp_design *D, const dp_config *cfg, float *gsp, float *gtr, fl
     if (D->batched) return set_err(D->ctx, DP_EUNSUPPORTED, "dp_step runs on single-scenario inputs");
     if (cfg->tr_mode == 2) return set_err(D->ctx, DP_EUNSUPPORTED, "the lag-one mode runs on batched inputs");
     DeviceGuard g(D->ctx->device);
+    note_capture(D);
     if ((s = ensure_words(D, cfg->sim_words)) != DP_OK) return s;
     if ((s = ensure_stage(D)) != DP_OK) return s;
     if ((s = ensure_step_streams(D)) != DP_OK) return s;
@@ -1272,6 +1278,7 @@ dp_status dp_sizing_scores(dp_design *D, const dp_config *cfg, int32_t mode, flo
     if (!D->bwd_valid || D->bwd_grad_mode != cfg->grad_mode || D->fwd_tr_mode != cfg->tr_mode)
         return set_err(c, DP_ESTATE, "sizing scores need dp_backward (or dp_step) with the same config");
     DeviceGuard g(c->device);
+    note_capture(D);
     cudaStream_t st = c->stream;
     const int64_t kk = k < nc ? k : nc;
     if (!D->sc_tops) {   // the last one

@@ -95,9 +95,10 @@ struct dp_design {
     cudaStream_t out_stream = nullptr;
     cudaEvent_t ev_grads = nullptr, ev_copies = nullptr;
     // a dp_simulate that directly follows a dp_propagate may start beside it, at ev[0]: nothing queued on the stream
-    // since uses what it writes
+    // since writes what it reads or uses what it writes.  Not once any call on the design has been captured: a replay
+    // of the user's graph queues that call's work without the library knowing
     bool sim_ahead = false;
-    bool sim_captured = false;   // a user's graph may hold a simulation of this design
+    bool captured = false;
     int grid[4] = {0, 0, 0, 0};   // persistent grids: forward, simulation, backward, wide simulation
     int flow_grid[3] = {0, 0, 0};  // dataflow grids: forward, simulation, reverse
     int block_threads = 0;         // > 0: the design fits the single-block passes, with this many threads
@@ -137,6 +138,8 @@ double power_K(const dp_config &c);
 dp_status check_cfg(dp_ctx *ctx, const dp_config *c);
 // true when the stream is being captured into a CUDA graph
 bool capturing(cudaStream_t s);
+// notes a call on the design that is being captured (every entry point that queues work on its single-scenario state)
+inline void note_capture(dp_design *D) { D->captured = D->captured || capturing(D->ctx->stream); }
 // frees the batched buffers (the caller has synchronised)
 void free_batch(dp_design *D);
 // batched halves of dp_propagate, dp_get_power and dp_get_nets (capi_batch.cu)
