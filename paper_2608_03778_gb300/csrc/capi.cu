@@ -1067,13 +1067,9 @@ dp_status dp_simulate(dp_design *D, const dp_config *cfg) {
     if ((s = ensure_words(D, cfg->sim_words)) != DP_OK) return s;
     cudaStream_t st = D->ctx->stream;
     note_capture(D);
-    bool ahead = D->sim_ahead && !D->ctx->switched && !D->captured;
+    // (no query of the event here: while another stream captures in global mode a query is an error, and ends that capture)
+    const bool ahead = D->sim_ahead && !D->ctx->switched && !D->captured;
     D->sim_ahead = false;
-    if (ahead) {   // an event that a capture recorded cannot be waited for here
-        const cudaError_t q = cudaEventQuery(D->ev[0]);
-        ahead = q == cudaSuccess || q == cudaErrorNotReady;
-        cudaGetLastError();
-    }
     rec(D, 1, st);
     const int beside = ahead ? step_slice_sms(D, *cfg) : 0;
     cudaError_t le = cudaSuccess;

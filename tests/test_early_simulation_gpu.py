@@ -95,3 +95,28 @@ def test_replayed_reads_come_before_the_simulation(dp, library_text, spec):  # n
             t.check(now, "after the replay")
     finally:
         t.close()
+
+
+@pytest.mark.parametrize("spec", SPECS)
+def test_another_streams_capture_goes_on(dp, library_text, spec):  # noqa: F811
+    """while another stream captures (torch's mode: global), the phases run on their own stream as before, and the
+    capture stays whole"""
+    t = Case(dp, spec, library_text)
+    try:
+        dp.dp_set_inputs(t.c, t.d, *t.inputs[0])
+        dp.dp_propagate(t.c, t.d, t.cfg)
+        dp.dp_simulate(t.c, t.d, t.cfg)   # whatever is made on first use
+        x = torch.zeros(8, device="cuda")
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            x.add_(1.0)
+            dp.dp_propagate(t.c, t.d, t.cfg)
+            dp.dp_simulate(t.c, t.d, t.cfg)
+            x.add_(1.0)
+        t.check(0, "beside a capture")
+        g.replay()
+        torch.cuda.synchronize()
+        assert x.eq(2.0).all()
+    finally:
+        t.close()
