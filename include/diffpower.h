@@ -339,7 +339,7 @@ dp_status dp_phase_times(dp_design *d, float *ms5);
  * variable DP_BATCH_SHAPE="bx,by[,bx2,by2]" fixes the shapes instead.  It
  * also times the passes without level barriers, one cooperative launch each
  * (DP_BATCH_FLOW="v" takes them with v scenarios per thread wherever v divides
- * n_scen), or for one scenario those by scenario groups
+ * n_scen; not in a server), or for one scenario those by scenario groups
  * (DP_BATCH_GROUP="lanes,v,blocks,threads" fixes them); a wait in the former
  * that gives up is reported as DP_ETIMEOUT by the next synchronising call.
  * Every shape gives bitwise identical results. */

@@ -169,13 +169,14 @@ bool flow_can(const dp_design *D, int64_t S) {
 
 // scenarios per thread of the staged batch's dataflow pass (0 forward, 1 reverse); 0: not used.  The tuner takes them
 // where they are fastest; the results are bitwise those of the other passes.  (A design without startpoints has no
-// launch that would tell them of a pass by level launches.)
+// launch that would tell them of a pass by level launches.)  Never in a server's slot (shapes_locked): the slots'
+// cooperative grids would keep each other out, and nobody there would see that a wait gave up.
 int flow_in_use(const dp_design *D, int tr_mode, int pass) {
     const dp_batch &B = D->batch;
-    if (!flow_can(D, B.S)) return 0;
+    if (B.shapes_locked || !flow_can(D, B.S)) return 0;
     dp::GroupShape g;
     int v = flow_env(B.S);
-    if (v == 0 && !B.shape_from_env && !parse_group_env(&g) && B.tuned_S == B.S && !B.shapes_locked)
+    if (v == 0 && !B.shape_from_env && !parse_group_env(&g) && B.tuned_S == B.S)
         v = pass == 0 ? B.fwd_flow : B.bwd_flow;
     return tr_mode == 2 && v > 2 ? 2 : v;
 }
@@ -194,7 +195,8 @@ int flow_v(int64_t S, int64_t W) {
 // of the level launches, and for the dataflow passes, or for a single scenario for a group shape, and keeps the
 // fastest of each.  The first shape of a kernel runs once before it is timed; a shape that is
 // more than a tenth slower than the best is not timed twice.  Runs on the staged inputs; the results it
-// leaves are overwritten by the next dp_propagate.
+// leaves are overwritten by the next dp_propagate.  Locked shapes (a server's) take level launches and the group rule
+// only, so only the former are timed.
 dp_status tune(dp_design *D) {
     dp_batch &B = D->batch;
     dp_ctx *c = D->ctx;
@@ -255,8 +257,8 @@ dp_status tune(dp_design *D) {
     // 90 + 99), from two on by dataflow (S = 2: 48 + 56 against 49 + 56 at 2,000 / 24, and ahead from there)
     float least[2] = {best[0], best[1]};
     const dp::GroupShape g{2, 1, 16, 512};
-    const bool groups = S == 1 && D->d.n_levels > 0 && W <= 6000;
-    if (!groups && flow_can(D, S))
+    const bool groups = !B.shapes_locked && S == 1 && D->d.n_levels > 0 && W <= 6000;
+    if (!groups && !B.shapes_locked && flow_can(D, S))
         for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
             const int v = flow_v(S, W);
             const float t = timed(   // the first run also brings the arrays to rest
@@ -331,9 +333,8 @@ dp_status batch_reserve(dp_design *D, int64_t S) {
 }
 
 dp_status batch_tune_and_lock(dp_design *D) {
-    dp_status s = tune(D);
-    if (s == DP_OK) D->batch.shapes_locked = true;
-    return s;
+    D->batch.shapes_locked = true;
+    return tune(D);
 }
 
 // the lag-one state (every net's TR, two adjoints per edge, the startpoints' TR adjoint),

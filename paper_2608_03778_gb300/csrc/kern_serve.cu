@@ -112,8 +112,9 @@ __global__ void k_delta_clear_cells(const int32_t *__restrict__ cell, const int3
 // every scenario column of a batch gets the reference inputs' forward state:
 // the float-float P of every net and the input TR of every startpoint
 __global__ void k_bcast_ref(const float2 *__restrict__ ref_pq, const float *__restrict__ ref_tr, float2 *pq,
-                            float *tr_in, int64_t nn, int64_t ns, int64_t S) {
+                            float *tr_in, int64_t nn, int64_t ns, int64_t S, uint32_t *state) {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s == 0 && blockIdx.y == 0) state[0] = 0u;   // no dataflow pass wrote these
     if (s >= S) return;
     for (int64_t n = blockIdx.y; n < nn; n += gridDim.y) {
         pq[n * S + s] = ref_pq[n];
@@ -196,11 +197,11 @@ void launch_sizing_clear(const DevDesign &d, const SizingDeltas &z, int64_t ne, 
 }
 
 void launch_bcast_ref(const float2 *ref_pq, const float *ref_tr, float2 *pq, float *tr_in, int64_t nn, int64_t ns,
-                      int64_t S, cudaStream_t s) {
+                      int64_t S, uint32_t *state, cudaStream_t s) {
     if (nn <= 0 || S <= 0) return;
     const unsigned bx = S >= 128 ? 128u : 32u;
     k_bcast_ref<<<dim3((unsigned)cdiv(S, bx), (unsigned)(nn < 8192 ? nn : 8192)), bx, 0, s>>>(ref_pq, ref_tr, pq,
-                                                                                              tr_in, nn, ns, S);
+                                                                                              tr_in, nn, ns, S, state);
 }
 
 }  // namespace dp

@@ -280,9 +280,9 @@ void launch_serve_in(const ServeIo *io, int64_t S, int64_t ns, int64_t most_nd, 
 void launch_serve_out(const ServeIo *io, int64_t S, int64_t ns, int64_t nc, const float *sp, const float *tr,
                       const float *pin, cudaStream_t s);
 // the reference inputs' forward state (P of every net, TR of every startpoint) into every
-// scenario column of a batch: a batch of requests on the reference inputs skips the forward pass
+// scenario column of a batch: a batch of requests on the reference inputs skips the forward pass (state: BatchBufs')
 void launch_bcast_ref(const float2 *ref_pq, const float *ref_tr, float2 *pq, float *tr_in, int64_t nn, int64_t ns,
-                      int64_t S, cudaStream_t s);
+                      int64_t S, uint32_t *state, cudaStream_t s);
 void launch_sizing_clear(const DevDesign &d, const SizingDeltas &z, int64_t ne, int64_t S, float *dcl,
                          cudaStream_t s);
 // out[c][r] = in[r][c] (row-major R x C in, C x R out)

@@ -264,7 +264,7 @@ cudaError_t capture_batch_graph(dp_server *srv, Slot *sl, int64_t Sg, bool grad,
     cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
     if (ref) {
-        dp::launch_bcast_ref(sl->d_ref_pq, sl->d_ref_tr, B.b.pq, B.b.tr_in, sl->nn, ns, Sg, st);
+        dp::launch_bcast_ref(sl->d_ref_pq, sl->d_ref_tr, B.b.pq, B.b.tr_in, sl->nn, ns, Sg, B.b.state, st);
     } else {
         dp::launch_transpose(sl->d_in_sp, B.b.sp_in, Sg, ns, st);
         dp::launch_transpose(sl->d_in_tr, B.b.tr_in, Sg, ns, st);
