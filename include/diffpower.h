@@ -214,6 +214,12 @@ dp_status dp_sync(dp_ctx *ctx);
  * No GPU fault is involved. */
 dp_status dp_selftest_wait(dp_ctx *ctx, double seconds);
 
+/* Test hook: sets the context's error word, in stream order, as a wait that
+ * gave up does.  Waits of the passes queued behind it that are not over after
+ * some polls then give up as well, and the next synchronising call returns
+ * DP_ETIMEOUT and clears the word.  Not under stream capture. */
+dp_status dp_selftest_give_up(dp_ctx *ctx);
+
 /* Test hook on the calling thread's CUDA runtime error state (the library's
  * own runtime, linked statically).  action 1 plants a launch-configuration
  * error: a kernel launch with zero threads per block, which the runtime

@@ -48,7 +48,6 @@ dp_status check_device_error(dp_ctx *c) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_err(c, e, "device error word");
     if (v != 0) {
-        c->timeouts++;
         cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
         cudaStreamSynchronize(c->stream);
         return set_err(c, DP_ETIMEOUT, "a bounded device wait gave up (grid barrier timeout)");
@@ -241,16 +240,6 @@ int step_slice_sms(const dp_design *D, const dp_config &c) {
 // above (schedule 0), and on request (schedule 3, which has a dataflow simulation too)
 bool dataflow(const dp_design *D, const dp_config &c, int which) {
     return (c.schedule == 3 || (c.schedule == 0 && which != 1)) && D->flow_grid[which] > 0 && D->d.n_levels > 0;
-}
-
-// A pass that timed out may have left nets of two parities behind, which a later dataflow pass
-// could take for its own: back to the state after the upload.
-void repair_tags(dp_design *D, cudaStream_t s) {
-    if (D->timeouts_seen == D->ctx->timeouts) return;
-    D->timeouts_seen = D->ctx->timeouts;
-    cudaMemsetAsync(D->d.pq, 0, sizeof(float4) * (size_t)D->d.n_nets, s);
-    cudaMemsetAsync(D->d.epoch, 0, sizeof(uint32_t), s);
-    cudaMemsetAsync(D->d.epoch + 4, 0, 2 * sizeof(uint32_t), s);
 }
 
 // each q_* returns the first launch error (a cooperative launch reports it directly)
@@ -484,6 +473,13 @@ dp_status dp_selftest_wait(dp_ctx *c, double seconds) {
     cudaFree(gs);
     if (e != cudaSuccess) return cuda_err(c, e, "dp_selftest_wait");
     return check_device_error(c);
+}
+
+dp_status dp_selftest_give_up(dp_ctx *c) {
+    if (!c) return DP_EINVAL;
+    DeviceGuard g(c->device);
+    if (capturing(c->stream)) return set_err(c, DP_ESTATE, "dp_selftest_give_up under capture");
+    return cuda_err(c, cudaMemsetAsync(c->d_err, 1, sizeof(int), c->stream), "dp_selftest_give_up");
 }
 
 namespace {
@@ -899,7 +895,6 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
         D->sl = dp::SlicePlan{slice.slots, slice.threads, drec, dround, dfourth, dstart};
     }
     for (int w = 0; w < 3; w++) D->flow_grid[w] = dp::flow_grid(w, ctx->sm_count);
-    D->timeouts_seen = ctx->timeouts;
     if (e != cudaSuccess) { s = cuda_err(ctx, e, "upload"); free_design(D); return s; }
     dp::launch_cload(d, st);
     for (auto &ev : D->ev)
@@ -1041,7 +1036,6 @@ dp_status dp_propagate(dp_design *D, const dp_config *cfg) {
     DeviceGuard g(D->ctx->device);
     note_capture(D);
     cudaStream_t st = D->ctx->stream;
-    repair_tags(D, st);
     rec(D, 0, st);
     cudaError_t le = q_forward(D, *cfg, st);
     rec(D, 1, st);
@@ -1248,7 +1242,6 @@ dp_status dp_step(dp_design *D, const dp_config *cfg, float *gsp, float *gtr, fl
         if (e != cudaSuccess) { D->graph = nullptr; return cuda_err(D->ctx, e, "graph instantiate"); }
         D->graph_cfg = *cfg;
     }
-    repair_tags(D, st);
     cudaError_t e = cudaGraphLaunch(D->graph, st);
     if (e != cudaSuccess) return cuda_err(D->ctx, e, "graph launch");
     for (int i = 0; i < 5; i++) D->ev_valid[i] = true;

@@ -17,7 +17,6 @@ struct dp_ctx {
     int clock_khz = 0;
     int *d_err = nullptr;   // device error word: a bounded wait gave up
     bool switched = false;  // the calls have been on more than one stream
-    unsigned timeouts = 0;  // times a synchronising call found it set
     std::string err;
 };
 
@@ -104,7 +103,6 @@ struct dp_design {
     int block_threads = 0;         // > 0: the design fits the single-block passes, with this many threads
     dp::SlicePlan sl;              // the sliced simulation (sl.slots > 0: the design uses it)
     dp::ClusterMap cl;             // the single-cluster passes (cl.threads > 0: the design uses them)
-    unsigned timeouts_seen = 0;    // the context's count of timed-out waits when the pair tags were last sound
     int64_t graph_kernels = 0;
     int64_t step_kernels = 0;
     // phase boundaries: start, forward, simulation levels, hybrid + power, backward, outputs

@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(kClusterMaxThreads) k_fwd_cluster(
         tr[n] = tr_mode ? pair_tr(a) : tr_in[n];
     }
     __syncwarp();
+    bool ok = true;
     for (int l = 1; l <= L; l++) {
         if (__any_sync(0xFFFFFFFFu, on)) {
             const uint32_t op = r.x >> 24;
@@ -166,7 +167,6 @@ __global__ void __launch_bounds__(kClusterMaxThreads) k_fwd_cluster(
                 if (j < k) dsm_ld_pair(at[j], h0[j], h1[j]);
             }
             auto late = [&](int j) { return (~(uint32_t)h0[j] | ~(uint32_t)h1[j]) & 0x80000000u; };
-            bool ok = true;
             if (__any_sync(0xFFFFFFFFu, (late(0) | late(1) | late(2) | late(3)) != 0)) {
                 const long long t0 = clock64();
                 unsigned spins = 0;
@@ -177,7 +177,8 @@ __global__ void __launch_bounds__(kClusterMaxThreads) k_fwd_cluster(
                     if (gives_up(spins, t0, err, limit)) ok = false;
                 } while (__any_sync(0xFFFFFFFFu, (late(0) | late(1) | late(2) | late(3)) != 0) &&
                          __all_sync(0xFFFFFFFFu, ok));
-                if (!__all_sync(0xFFFFFFFFu, ok)) break;
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok) break;
             }
             if (on) {
                 pair_ff x[4];
@@ -197,6 +198,7 @@ __global__ void __launch_bounds__(kClusterMaxThreads) k_fwd_cluster(
         on1 = cell_at(s, l + 2, L, rk, t, c1, slot1);
         if (on1) r1 = fanin[c1], f1 = floc[c1];
     }
+    if (!ok) epoch[3] = 1u;   // pairs of two parities: the power pass puts the tags right
     cluster_arrive();
     cluster_wait();   // nothing remote after this
     if (rk == 0 && t == 0) epoch[0] = pass;

@@ -146,7 +146,10 @@ __global__ void __launch_bounds__(kFlowThreads) k_fwd_flow(const uint4 *__restri
             issue_pairs(w, pq, r0, k, par);
             pair_ff x[4];
             ok = wait_pairs(w, pq, par, err, limit, x);
-            if (!ok) break;
+            if (!ok) {
+                epoch[3] = 1u;   // pairs of two parities: the power pass puts the tags right
+                break;
+            }
             if (c < c1) {
                 const pair_ff o = cell_pair(k, op_tt(ops, r0.x >> 24), x);
                 pair_put(pq + ns + c, o, par);

@@ -183,12 +183,14 @@ __device__ __forceinline__ void level_bounds(int *bounds, const int32_t *lvl, in
     __syncthreads();
 }
 
-// true in one thread of the last block to get here (a block that gave up has recorded it before); done is 0 again
+// true in one thread of the last block to get here (a block that gave up has recorded it before, in a word of the pass's
+// own: the context's error word may be read and cleared by a call on another stream); done is 0 again
 __device__ __forceinline__ bool last_block(uint32_t *done) {
     __syncthreads();
     if (threadIdx.x != 0) return false;
     __threadfence();
     if (atomicAdd(done, 1u) != gridDim.x - 1) return false;
+    __threadfence();
     *done = 0u;
     return true;
 }
@@ -288,9 +290,11 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
             if (LAG) put_row<V>(row_at(tqs, c, S), ot);
         }
     }
+    if (!ok) state[6] = 1u;   // before the block's arrival
     if (last_block(state + 3)) {
-        state[0] = ld_word(err) ? 0u : S;
+        state[0] = ld_word(state + 6) ? 0u : S;
         state[1] = pass;
+        state[6] = 0u;
     }
 }
 
@@ -439,7 +443,11 @@ __global__ void __launch_bounds__(THREADS, BLOCKS)
                 put_row(row_at(gs, pos[j], S), g);
             }
     }
-    if (last_block(state + 4)) state[LAG ? 5 : 2] = ld_word(err) ? 0u : 1u;
+    if (!ok) state[7] = 1u;
+    if (last_block(state + 4)) {
+        state[LAG ? 5 : 2] = ld_word(state + 7) ? 0u : 1u;
+        state[7] = 0u;
+    }
 }
 
 // The arrays of a pass as it expects them: which 0, the forward pass's pairs, where the last to write them was not a

@@ -54,11 +54,19 @@ __global__ void k_set_pincap(const int32_t *__restrict__ cells, const float *__r
 __device__ __forceinline__ double warp_sum(double v) { return warp_sum_f64(v); }
 
 // power partials: a fixed grid and a fixed per-thread stride make the FP64
-// summation order independent of timing, so the result is reproducible
+// summation order independent of timing, so the result is reproducible.
+//
+// Every forward pass is followed by its power, so this is also where the pairs' tags are put
+// right after a pass in which a wait gave up (epoch[3]): it leaves pairs of two parities, and
+// the pass after next would take the older ones for its own.  All get the parity of the pass
+// that has just ended.  It happens on the device, so a replayed graph is as safe as a call.
 __global__ void __launch_bounds__(kPowerThreads) k_power_partials(const float *__restrict__ tr,
                                                                   const float *__restrict__ beta,
                                                                   const float *__restrict__ cload, double *partials,
-                                                                  int64_t nn) {
+                                                                  int64_t nn, float4 *pq, const uint32_t *epoch) {
+    if (epoch[3])
+        for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < nn; n += (int64_t)gridDim.x * blockDim.x)
+            pq[n] = pair_store(pair_load(pq[n]), epoch[0] & 1u);
     // each term alpha C rounded once to binary32 (rel. 6e-8), the sum in FP64: one
     // conversion and one FP64 add per net, on a part whose FP64 pipe is narrow
     double s = 0.0;
@@ -78,7 +86,8 @@ __global__ void __launch_bounds__(kPowerThreads) k_power_partials(const float *_
 }
 
 __global__ void __launch_bounds__(kPowerThreads) k_power_final(const double *__restrict__ partials, int nb, double K,
-                                                               double *out) {
+                                                               double *out, uint32_t *epoch) {
+    if (threadIdx.x == 0) epoch[3] = 0u;
     double s = 0.0;
     for (int i = threadIdx.x; i < nb; i += blockDim.x) s += partials[i];
     __shared__ double sh[kPowerThreads / 32];
@@ -166,8 +175,8 @@ void launch_set_pincap(const DevDesign &d, const int32_t *cells, const float *ca
 
 void launch_power(const DevDesign &d, bool hybrid, double K, int slot, cudaStream_t s) {
     k_power_partials<<<kPowerBlocks, kPowerThreads, 0, s>>>(d.tr, hybrid ? d.beta : nullptr, d.cload, d.partials,
-                                                            d.n_nets);
-    k_power_final<<<1, kPowerThreads, 0, s>>>(d.partials, kPowerBlocks, K, d.power + slot);
+                                                            d.n_nets, d.pq, d.epoch);
+    k_power_final<<<1, kPowerThreads, 0, s>>>(d.partials, kPowerBlocks, K, d.power + slot, d.epoch);
 }
 
 void launch_cap_grads(const DevDesign &d, const OpTable &ops, bool hybrid, int tr_mode, double K,

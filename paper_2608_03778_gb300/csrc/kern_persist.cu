@@ -94,7 +94,7 @@ __device__ __forceinline__ void fwd_cell(const uint4 &r, int64_t c, float4 *pq, 
 __global__ void __launch_bounds__(kFwdThreads) k_fwd_persist(
     const uint4 *__restrict__ fanin, float4 *pq, float *tr, const float *__restrict__ sp_in,
     const float *__restrict__ tr_in, const int32_t *__restrict__ lvl, int L, int64_t ns, int tr_mode, OpTable ops,
-    unsigned *bar, int *err, long long limit, const uint32_t *epoch) {
+    unsigned *bar, int *err, long long limit, uint32_t *epoch) {
     const int64_t tid = spread_tid();
     const int64_t T = (int64_t)gridDim.x * blockDim.x;
     const uint32_t par = epoch[0] & 1u;
@@ -113,7 +113,10 @@ __global__ void __launch_bounds__(kFwdThreads) k_fwd_persist(
             const int64_t cp = lvl[l + 1] + tid;
             if (cp < lvl[l + 2]) prefetch_l2(fanin + cp);
         }
-        if (!barrier_wait(bar + 32 * (l - 1), err, gridDim.x, limit)) return;
+        if (!barrier_wait(bar + 32 * (l - 1), err, gridDim.x, limit)) {
+            if (threadIdx.x == 0) epoch[3] = 1u;   // pairs of two parities: the power pass puts the tags right
+            return;
+        }
         if (c < c1) fwd_cell(r, c, pq, tr, ns, ops, par);
         for (int64_t cc = c + T; cc < c1; cc += T) fwd_cell(fanin[cc], cc, pq, tr, ns, ops, par);
     }
@@ -743,7 +746,7 @@ cudaError_t launch_fwd_persist(const DevDesign &d, const OpTable &ops, int tr_mo
     if (ready) cudaEventRecord(ready, s);   // work forked here becomes ready together with the kernel
     return launch_coop(k_fwd_persist, grid, kFwdThreads, s, d.fanin, d.pq, d.tr, (const float *)d.sp_in,
                        (const float *)d.tr_in, d.lvl, d.n_levels, d.n_start, tr_mode, ops, bar, d.err,
-                       kWaitLimitCycles, (const uint32_t *)d.epoch);
+                       kWaitLimitCycles, d.epoch);
 }
 
 cudaError_t launch_sim_persist(const DevDesign &d, const OpTable &ops, int T, int grid, cudaStream_t s) {

@@ -71,7 +71,8 @@ struct DevDesign {
     unsigned *bar;             // level-barrier arrival counters of the persistent passes (128-byte lines)
     unsigned long long *gcell; // [n_cells] the dataflow reverse pass's cell adjoints: value, pass number << 32
     uint32_t *epoch;           // [8] pass counters: [0] forward (its parity tags the stored pairs), [1] dataflow
-                               // simulation, [2] dataflow reverse; [4], [5] blocks done of [0], [2] (0 at rest)
+                               // simulation, [2] dataflow reverse; [4], [5] blocks done of [0], [2] and [3] a wait
+                               // of [0] gave up (0 at rest)
     const int32_t *pair_ptr;   // [n_levels+1] level-aligned cell pairs: pairs of level l are [pair_ptr[l-1], pair_ptr[l])
     unsigned *simdone;         // [n_cells] pass number of the simulation pass that last wrote the cell's words
     const int32_t *dead_ptr;   // [n_levels+2] nets by death level d (the highest level reading the net, else
@@ -88,6 +89,7 @@ void launch_fwd_level(const DevDesign &d, const OpTable &ops, int32_t c0, int32_
 void launch_cload(const DevDesign &d, cudaStream_t s);
 void launch_set_pincap(const DevDesign &d, const int32_t *cells, const float *caps, int32_t n, cudaStream_t s);
 // power: sum_n alpha_n C_n (alpha = tr, or beta*tr when hybrid), times K, into d.power[slot]
+// (and, after a forward pass in which a wait gave up, the pairs' tags)
 void launch_power(const DevDesign &d, bool hybrid, double K, int slot, cudaStream_t s);
 // outputs in user order: grad_cload (K alpha), grad_pincap (K sum fanin alpha), grad_tr_in (K beta C or 0)
 void launch_cap_grads(const DevDesign &d, const OpTable &ops, bool hybrid, int tr_mode, double K, float *grad_cload,
@@ -185,7 +187,8 @@ struct BatchBufs {
     float *ks;              // [S] per-scenario seed of the backward (K * weight), binary32
     const float *dcl;       // [n_nets * S] per-scenario change of C_load (sizing deltas), or NULL
     uint32_t *state;        // [8] the dataflow passes' (0 at rest): [0] columns of pq if such a pass wrote it, else 0;
-                            // [1] forward passes; [2] 1: every word of gfo is at rest; [3], [4] blocks done; [5] as [2], of gfo2
+                            // [1] forward passes; [2] 1: every word of gfo is at rest; [3], [4] blocks done; [5] as [2], of gfo2;
+                            // [6], [7] a wait of the pass that runs gave up (forward, reverse)
     // lag-one mode (tr_mode 2) only, else NULL:
     float *tq;              // [n_nets * S] TR of every net
     float2 *gfo2;           // [n_edges * S] edge adjoints of (P, TR)
