@@ -526,9 +526,10 @@ def bench_batched(args, dp, torch, dev, pk: dict) -> dict:
         fwd_shape, bwd_shape, tune_ms = dp.dp_batch_tuning(des.d)
         ab = batched_algorithmic_bytes(nn, ns, nc, ne, S)
         ach = ab / (ms * 1e-3) / 1e9
-        # kernels per forward + reverse pass, at least (the dataflow passes; the level launches have one per
-        # level): preparation + pass, 2 power, seed, preparation + pass
-        launches = 2 + 2 + 1 + 2
+        # kernels per forward + reverse pass: the passes that the tuner took, 2 power, seed
+        passes = dp.dp_batch_passes(des.d, 0)
+        launches = passes[0][2] + 2 + 1 + passes[1][2]
+        names = {"level": "level", "group": "group", "dataflow": "flow"}
 
         # Algorithm 4: 200 steps for all 512 starts, the proxy of Eq. 9 (tr_mode 1)
         steps = 200
@@ -545,8 +546,10 @@ def bench_batched(args, dp, torch, dev, pk: dict) -> dict:
                         "frac": ab / (statistics.median(warm) * 1e-3) / 1e9 / pk["hbm_gbs"]},
             "roofline": {"bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s",
                          "frac": ach / pk["hbm_gbs"], "algorithmic_bytes": ab, "traffic": None,
-                         "kernels": "k_fwdb_flow, k_bwdb_flow, k_powerb_*"},
-            "shapes": {"forward": list(fwd_shape), "backward": list(bwd_shape), "tuner_ms": list(tune_ms)},
+                         "kernels": f"k_fwdb_{names[passes[0][0]]}, k_bwdb_{names[passes[1][0]]}, k_powerb_*"},
+            "passes": {w: {"kind": p[0], "scenarios_per_thread": p[1], "launches": p[2], "tuner_ms": p[3]}
+                       for w, p in zip(("forward", "backward"), passes)},
+            "level_shapes": {"forward": list(fwd_shape), "backward": list(bwd_shape), "tuner_ms": list(tune_ms)},
             "gpu_launches_per_fwd_bwd": launches,
             "ascent": {"steps": steps, "starts": S, "eta": ETA, "proxy": "Eq. 9 (tr_mode 1)",
                        "graph": res.graph, "ms_total": res.ms_ascent, "ms_per_step": res.ms_ascent / steps,

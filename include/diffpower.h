@@ -352,11 +352,19 @@ dp_status dp_phase_times(dp_design *d, float *ms5);
 dp_status dp_set_inputs_batch(dp_design *d, const float *sp, const float *tr, int32_t n_scen, int on_device);
 
 /* Shapes of the level launches (bx threads over scenarios x by cells per block x v scenarios
- * per thread, v = 1 or 2; v = 2 applies to even n_scen) for the forward
+ * per thread, v = 1, 2 or 4; 2 and 4 apply where they divide n_scen) for the forward
  * (shape6[0..2]) and the reverse pass (shape6[3..5]), and the tuner's best
  * times in ms (ms2, may be NULL; 0 when fixed by the environment).  Every
  * shape gives bitwise the same results. */
 dp_status dp_batch_tuning(const dp_design *d, int32_t *shape6, float *ms2);
+
+/* The passes that the staged batch takes in tr_mode: for the forward
+ * (pass6[0..2]) and the reverse pass (pass6[3..5]) their kind (0 level
+ * launches, 1 scenario groups, 2 dataflow), scenarios per thread and number of
+ * kernel launches (the model power's two and the reverse pass's seed not
+ * counted); ms2 (may be NULL) the tuner's times of both in ms, in tr_mode 0
+ * (0: not timed, as where the environment or a rule decides). */
+dp_status dp_batch_passes(const dp_design *d, int32_t tr_mode, int32_t *pass6, float *ms2);
 
 /* Reverse pass of the model power (Sec. III-E, Eq. 7) for every scenario,
  * scaled by weights[n_scen] (NULL: all 1): the gradient of

@@ -202,6 +202,7 @@ dp_status tune(dp_design *D) {
     dp_ctx *c = D->ctx;
     B.fwd_group = B.bwd_group = dp::GroupShape{};
     B.fwd_flow = B.bwd_flow = 0;
+    B.tune_ms[0] = B.tune_ms[1] = B.pass_ms[0] = B.pass_ms[1] = 0.f;
     B.shape_from_env = parse_shape_env(&B.fwd_shape, &B.bwd_shape);
     if (B.shape_from_env) {
         B.tuned_S = B.S;
@@ -281,6 +282,7 @@ dp_status tune(dp_design *D) {
                 },
                 true, least[pass]);
             if (t < least[pass]) {
+                least[pass] = t;
                 (pass == 0 ? B.fwd_group : B.bwd_group) = g;
                 (pass == 0 ? B.fwd_flow : B.bwd_flow) = 0;
             }
@@ -291,8 +293,10 @@ dp_status tune(dp_design *D) {
     if (e != cudaSuccess) return cuda_err(c, e, "batch autotuner");
     B.fwd_shape = pick[0];
     B.bwd_shape = pick[1];
-    B.tune_ms[0] = best[0];
-    B.tune_ms[1] = best[1];
+    for (int pass = 0; pass < 2; pass++) {
+        B.tune_ms[pass] = best[pass];
+        B.pass_ms[pass] = least[pass];
+    }
     B.tuned_S = S;
     return check_device_error(c);
 }
@@ -455,6 +459,27 @@ dp_status dp_batch_tuning(const dp_design *D, int32_t *shape6, float *ms2) {
     if (ms2) {
         ms2[0] = B.tune_ms[0];
         ms2[1] = B.tune_ms[1];
+    }
+    return DP_OK;
+}
+
+dp_status dp_batch_passes(const dp_design *D, int32_t tr_mode, int32_t *pass6, float *ms2) {
+    if (!D || !pass6 || tr_mode < 0 || tr_mode > 2) return DP_EINVAL;
+    const dp_batch &B = D->batch;
+    if (B.cap == 0) return set_err(D->ctx, DP_ESTATE, "dp_batch_passes before dp_set_inputs_batch");
+    for (int pass = 0; pass < 2; pass++) {
+        int32_t *o = pass6 + 3 * pass;
+        const int v = flow_in_use(D, tr_mode, pass);
+        const dp::GroupShape g = dp::group_for(group_in_use(D, tr_mode, pass), tr_mode);
+        const dp::BatchShape &sh = pass == 0 ? B.fwd_shape : B.bwd_shape;
+        o[0] = v > 0 ? 2 : g.v > 0 ? 1 : 0;
+        o[1] = v > 0 ? v : g.v > 0 ? g.v : tr_mode == 2 || B.S % sh.v ? 1 : sh.v;
+        o[2] = v > 0 ? 2 : g.v > 0 ? 1 : D->d.n_levels + (D->d.n_start > 0 ? 1 : 0);
+        // what was timed is what is taken, unless the environment has its way or the lag-one mode's rule
+        dp::GroupShape env;
+        const bool timed = B.tuned_S == B.S && !B.shapes_locked && flow_env(B.S) == 0 && !parse_group_env(&env) &&
+                           (tr_mode != 2 || o[0] == 2);
+        if (ms2) ms2[pass] = timed ? B.pass_ms[pass] : 0.f;
     }
     return DP_OK;
 }

@@ -38,7 +38,8 @@ struct dp_batch {
     bool shape_from_env = false;   // DP_BATCH_SHAPE fixed the level launches
     int64_t tuned_S = 0;           // S the shapes were tuned for (0: not tuned)
     bool shapes_locked = false;    // keep the shapes whatever S comes (a server fixes them once)
-    float tune_ms[2] = {0.f, 0.f}; // best forward / backward time seen by the tuner
+    float tune_ms[2] = {0.f, 0.f}; // best forward / backward time of the level launches seen by the tuner
+    float pass_ms[2] = {0.f, 0.f}; // ... of all passes: the ones in use (0: not timed)
     // power-virus evaluation (Eq. 3): words [n_nets * 2 ceil(S/64)], partials, sums, staging
     int64_t vcap = 0;
     uint64_t *vwords = nullptr;
