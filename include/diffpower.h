@@ -348,6 +348,7 @@ dp_status dp_phase_times(dp_design *d, float *ms5);
  * n_scen; not in a server), or for one scenario those by scenario groups
  * (DP_BATCH_GROUP="lanes,v,blocks,threads" fixes them); a wait in the former
  * that gives up is reported as DP_ETIMEOUT by the next synchronising call.
+ * Where such a launch is refused the other passes run.
  * Every shape gives bitwise identical results. */
 dp_status dp_set_inputs_batch(dp_design *d, const float *sp, const float *tr, int32_t n_scen, int on_device);
 
@@ -357,6 +358,13 @@ dp_status dp_set_inputs_batch(dp_design *d, const float *sp, const float *tr, in
  * times in ms (ms2, may be NULL; 0 when fixed by the environment).  Every
  * shape gives bitwise the same results. */
 dp_status dp_batch_tuning(const dp_design *d, int32_t *shape6, float *ms2);
+
+/* Test hook: the batched passes without level barriers ask for the grid of
+ * `sms` SMs (0: the device's own).  With more than the device has, the runtime
+ * refuses their cooperative launches on the host, and the library takes the
+ * other passes, as on a GPU that has no room for such a grid.  The next
+ * dp_set_inputs_batch tunes again. */
+dp_status dp_selftest_flow_grid(dp_design *d, int32_t sms);
 
 /* The passes that the staged batch takes in tr_mode: for the forward
  * (pass6[0..2]) and the reverse pass (pass6[3..5]) their kind (0 level

@@ -173,12 +173,29 @@ bool flow_can(const dp_design *D, int64_t S) {
 // cooperative grids would keep each other out, and nobody there would see that a wait gave up.
 int flow_in_use(const dp_design *D, int tr_mode, int pass) {
     const dp_batch &B = D->batch;
-    if (B.shapes_locked || !flow_can(D, B.S)) return 0;
+    if (B.shapes_locked || B.flow_refused || !flow_can(D, B.S)) return 0;
     dp::GroupShape g;
     int v = flow_env(B.S);
     if (v == 0 && !B.shape_from_env && !parse_group_env(&g) && B.tuned_S == B.S)
         v = pass == 0 ? B.fwd_flow : B.bwd_flow;
     return tr_mode == 2 && v > 2 ? 2 : v;
+}
+
+// The dataflow pass (0 forward, 1 reverse) of the staged batch.  Its grid has to be resident as a whole, which a
+// partitioned GPU may not have room for: the runtime then refuses the launch.
+cudaError_t launch_flow(dp_design *D, int tr_mode, int pass, int v, cudaStream_t s) {
+    dp_batch &B = D->batch;
+    const int sms = B.flow_sms > 0 ? B.flow_sms : D->ctx->sm_count;
+    return pass == 0 ? dp::launch_fwdb_flow(D->d, B.b, D->cell_ops, tr_mode, v, sms, s)
+                     : dp::launch_bwdb_flow(D->d, B.b, D->cell_ops, tr_mode, v, D->n_edges * B.cap, sms, s);
+}
+
+// true when e is such a refusal: the design's batches take the other passes from then on
+bool refused(dp_batch &B, cudaError_t e) {
+    if (e != cudaErrorCooperativeLaunchTooLarge) return false;
+    cudaGetLastError();
+    B.flow_refused = true;
+    return true;
 }
 
 // Scenarios per thread of the dataflow passes of a design with W cells per level: as many as leave whole warps and
@@ -259,15 +276,15 @@ dp_status tune(dp_design *D) {
     float least[2] = {best[0], best[1]};
     const dp::GroupShape g{2, 1, 16, 512};
     const bool groups = !B.shapes_locked && S == 1 && D->d.n_levels > 0 && W <= 6000;
-    if (!groups && !B.shapes_locked && flow_can(D, S))
+    if (!groups && !B.shapes_locked && !B.flow_refused && flow_can(D, S))
         for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
             const int v = flow_v(S, W);
-            const float t = timed(   // the first run also brings the arrays to rest
-                [&] {
-                    return pass == 0 ? dp::launch_fwdb_flow(D->d, B.b, D->cell_ops, 0, v, c->sm_count, st)
-                                     : dp::launch_bwdb_flow(D->d, B.b, D->cell_ops, 0, v, D->n_edges * B.cap, c->sm_count, st);
-                },
-                true, least[pass]);
+            // the first run also brings the arrays to rest
+            const float t = timed([&] { return launch_flow(D, 0, pass, v, st); }, true, least[pass]);
+            if (refused(B, e)) {
+                e = cudaSuccess;
+                break;
+            }
             if (t < least[pass]) {
                 least[pass] = t;
                 (pass == 0 ? B.fwd_flow : B.bwd_flow) = v;
@@ -307,8 +324,10 @@ namespace dpi {
 
 cudaError_t batch_forward(dp_design *D, int tr_mode, cudaStream_t s) {
     dp_batch &B = D->batch;
-    const int v = flow_in_use(D, tr_mode, 0);
-    if (v > 0) return dp::launch_fwdb_flow(D->d, B.b, D->cell_ops, tr_mode, v, D->ctx->sm_count, s);
+    if (const int v = flow_in_use(D, tr_mode, 0); v > 0) {
+        const cudaError_t e = launch_flow(D, tr_mode, 0, v, s);
+        if (!refused(B, e)) return e;
+    }
     const dp::GroupShape g = group_in_use(D, tr_mode, 0);
     if (g.v > 0) return dp::launch_fwdb_group(D->d, B.b, D->cell_ops, tr_mode, g, s);
     dp::launch_fwdb(D->d, B.b, D->cell_ops, D->lvl_ptr.data(), tr_mode, B.fwd_shape, s);
@@ -317,8 +336,10 @@ cudaError_t batch_forward(dp_design *D, int tr_mode, cudaStream_t s) {
 
 cudaError_t batch_reverse(dp_design *D, int tr_mode, cudaStream_t s) {
     dp_batch &B = D->batch;
-    const int v = flow_in_use(D, tr_mode, 1);
-    if (v > 0) return dp::launch_bwdb_flow(D->d, B.b, D->cell_ops, tr_mode, v, D->n_edges * B.cap, D->ctx->sm_count, s);
+    if (const int v = flow_in_use(D, tr_mode, 1); v > 0) {
+        const cudaError_t e = launch_flow(D, tr_mode, 1, v, s);
+        if (!refused(B, e)) return e;
+    }
     const dp::GroupShape g = group_in_use(D, tr_mode, 1);
     if (g.v > 0) return dp::launch_bwdb_group(D->d, B.b, D->cell_ops, tr_mode, g, s);
     dp::launch_bwdb(D->d, B.b, D->cell_ops, D->lvl_ptr.data(), tr_mode, B.bwd_shape, s);
@@ -463,6 +484,14 @@ dp_status dp_batch_tuning(const dp_design *D, int32_t *shape6, float *ms2) {
     return DP_OK;
 }
 
+dp_status dp_selftest_flow_grid(dp_design *D, int32_t sms) {
+    if (!D || sms < 0) return DP_EINVAL;
+    D->batch.flow_sms = sms;
+    D->batch.flow_refused = false;
+    D->batch.tuned_S = 0;
+    return DP_OK;
+}
+
 dp_status dp_batch_passes(const dp_design *D, int32_t tr_mode, int32_t *pass6, float *ms2) {
     if (!D || !pass6 || tr_mode < 0 || tr_mode > 2) return DP_EINVAL;
     const dp_batch &B = D->batch;
@@ -479,7 +508,7 @@ dp_status dp_batch_passes(const dp_design *D, int32_t tr_mode, int32_t *pass6, f
         dp::GroupShape env;
         const bool timed = B.tuned_S == B.S && !B.shapes_locked && flow_env(B.S) == 0 && !parse_group_env(&env) &&
                            (tr_mode != 2 || o[0] == 2);
-        if (ms2) ms2[pass] = timed ? B.pass_ms[pass] : 0.f;
+        if (ms2) ms2[pass] = timed ? (o[0] == 0 ? B.tune_ms : B.pass_ms)[pass] : 0.f;
     }
     return DP_OK;
 }

@@ -132,6 +132,7 @@ _sig("dp_server_get_stats", [_P, ctypes.POINTER(dp_server_stats)])
 _sig("dp_get_power", [_P, _S, _P, _S])
 _sig("dp_set_inputs_batch", [_P, _P, _P, ctypes.c_int32, _S])
 _sig("dp_batch_tuning", [_P, _P, _P])
+_sig("dp_selftest_flow_grid", [_P, ctypes.c_int32])
 _sig("dp_batch_passes", [_P, ctypes.c_int32, _P, _P])
 _sig("dp_backward_weighted", [_P, ctypes.POINTER(dp_config), _P, ctypes.c_int32, _P, _P, _P, _P, _S])
 _sig("dp_ascent_step", [_P, _P, _P, ctypes.c_int64, ctypes.c_float])
@@ -148,7 +149,7 @@ EXPORTED = ["dp_config_default", "dp_last_error", "dp_compile", "dp_compiled_fre
             "dp_propagate", "dp_simulate", "dp_total_power", "dp_backward", "dp_get_nets", "dp_step",
             "dp_phase_times", "dp_step_kernels", "dp_power_noalloc", "dp_selftest_wait", "dp_selftest_give_up",
             "dp_selftest_pending_error", "dp_probe_latency", "dp_set_stream",
-            "dp_get_power", "dp_set_inputs_batch", "dp_batch_tuning", "dp_batch_passes", "dp_backward_weighted",
+            "dp_get_power", "dp_set_inputs_batch", "dp_batch_tuning", "dp_batch_passes", "dp_selftest_flow_grid", "dp_backward_weighted",
             "dp_ascent_step", "dp_virus_eval", "dp_sizing_scores", "dp_server_config_default", "dp_server_create", "dp_server_destroy",
             "dp_server_last_error", "dp_server_add_design", "dp_server_design_info", "dp_server_submit",
             "dp_server_submit_many",
@@ -420,6 +421,11 @@ def dp_batch_tuning(d):
     ms = np.zeros(2, np.float32)
     _check(_lib.dp_batch_tuning(d, sh.ctypes.data, ms.ctypes.data))
     return (int(sh[0]), int(sh[1]), int(sh[2])), (int(sh[3]), int(sh[4]), int(sh[5])), (float(ms[0]), float(ms[1]))
+
+
+def dp_selftest_flow_grid(d, sms: int) -> None:
+    """The batched dataflow passes ask for the grid of ``sms`` SMs (0: the device's own)."""
+    _check(_lib.dp_selftest_flow_grid(d, sms))
 
 
 def dp_batch_passes(d, tr_mode: int = 0):

@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from paper_2608_03778_gb300 import netgen
-from tests.test_batch_gpu import ctx, dp  # noqa: F401
+from tests.test_batch_gpu import ctx, dp, run_batch  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -35,5 +35,34 @@ def test_passes_in_use(dp, ctx, library_text, monkeypatch, tr_mode):  # noqa: F8
             assert kind in ("level", "group", "dataflow") and 64 % v == 0
             assert launches == {"level": levels + 1, "group": 1, "dataflow": 2}[kind]
             assert 0 < ms <= best or (lag and kind != "dataflow" and ms == 0)
+    finally:
+        dp.dp_design_free(d)
+
+
+@pytest.mark.parametrize("tr_mode", [0, 1, 2])
+def test_refused_cooperative_launch(dp, ctx, library_text, monkeypatch, tr_mode):  # noqa: F811
+    """A grid the device has no room for, which the runtime refuses before anything runs: the tuner leaves the dataflow
+    passes out, a call that was to take them takes the others, and the results are the same bits."""
+    d = dp.dp_design_load(ctx, netgen.netlist_text(SPEC), library_text)
+    cfg = dp.config(grad_mode=0, tr_mode=tr_mode)
+    sp, tr = netgen.scenario_inputs(60, 78, 64)
+    try:
+        want = run_batch(dp, ctx, d, sp, tr, cfg)
+        for forced in (False, True):
+            dp.dp_selftest_flow_grid(d, 100_000)
+            with monkeypatch.context() as m:
+                if forced:   # (set after the tuner has run: the launch itself is what is refused)
+                    m.setenv("DP_BATCH_SHAPE", "32,4")
+                    stage(dp, ctx, d, 64)
+                    m.delenv("DP_BATCH_SHAPE")
+                    m.setenv("DP_BATCH_FLOW", "1")
+                got = run_batch(dp, ctx, d, sp, tr, cfg)
+                assert all(p[0] != "dataflow" for p in dp.dp_batch_passes(d, tr_mode))
+            for k in want:
+                np.testing.assert_array_equal(got[k], want[k], err_msg=k)
+            dp.dp_selftest_flow_grid(d, 0)
+            got = run_batch(dp, ctx, d, sp, tr, cfg)
+            for k in want:
+                np.testing.assert_array_equal(got[k], want[k], err_msg=k)
     finally:
         dp.dp_design_free(d)
