@@ -580,9 +580,8 @@ namespace {
 // The tables of the sliced simulation (kern_slice.cu), built on a thread of their own beside the
 // rest of an upload.  slots = 0: the design does not use it.
 struct SliceTables {
-    std::vector<int32_t> start_slot, round_ptr;
-    std::vector<uint32_t> rec;
-    std::vector<uint16_t> fourth;
+    std::vector<uint32_t> all;   // the records, then the levels' first rounds, the startpoints' slots, the fourth inputs
+    size_t at_round = 0, at_start = 0, at_fourth = 0;
     int64_t slots = 0;
     int threads = 0;
     struct Worker {
@@ -632,15 +631,19 @@ struct SliceTables {
                 cost += 60.0 + (double)((lvl[l] - lvl[l - 1] + p - 1) / p) * std::max(200.0, 14.0 * p / 32);
             if (threads == 0 || cost < best) threads = p, best = cost;
         }
-        round_ptr.assign((size_t)L + 1, 0);
+        std::vector<int32_t> round_ptr((size_t)L + 1, 0);
         for (int l = 1; l <= L; l++)
             round_ptr[(size_t)l] = round_ptr[(size_t)l - 1] + (lvl[l] - lvl[l - 1] + threads - 1) / threads;
-        rec.resize(4 * (size_t)threads * (size_t)round_ptr[(size_t)L]);
-        fourth.assign((size_t)nc, 0);
-        start_slot.assign(slot.begin(), slot.begin() + ns);
+        at_round = 4 * (size_t)threads * (size_t)round_ptr[(size_t)L];
+        at_start = at_round + round_ptr.size();
+        at_fourth = at_start + (size_t)ns;
+        all.resize(at_fourth + ((size_t)nc + 1) / 2);
+        std::copy(round_ptr.begin(), round_ptr.end(), all.begin() + (std::ptrdiff_t)at_round);
+        std::copy(slot.begin(), slot.begin() + ns, all.begin() + (std::ptrdiff_t)at_start);
+        uint16_t *const fourth = reinterpret_cast<uint16_t *>(all.data() + at_fourth);
         for (int l = 1; l <= L; l++) {
-            uint32_t *o = &rec[4 * (size_t)threads * (size_t)round_ptr[(size_t)l - 1]];
-            uint32_t *const end = &rec[0] + 4 * (size_t)threads * (size_t)round_ptr[(size_t)l];
+            uint32_t *o = all.data() + 4 * (size_t)threads * (size_t)round_ptr[(size_t)l - 1];
+            uint32_t *const end = all.data() + 4 * (size_t)threads * (size_t)round_ptr[(size_t)l];
             for (int64_t c = lvl[l - 1]; c < lvl[l]; c++, o += 4) {
                 const uint32_t *r = &cp->fanin[4 * (size_t)c];
                 const uint32_t op = r[0] >> 24, k = cp->op_arity[op], tt = cp->op_tt[op];
@@ -650,7 +653,7 @@ struct SliceTables {
                 o[1] = in[2] | ((uint32_t)slot[(size_t)(ns + c)] & 0xFFFFu) << 16;
                 o[2] = k <= 3 ? ops.e[op] >> 24 : (tt & 0xFFu) | 0x100u | (tt >> 8) << 16;
                 o[3] = (uint32_t)c;
-                if (k > 3) fourth[(size_t)c] = (uint16_t)in[3];
+                if (k > 3) fourth[c] = (uint16_t)in[3];
             }
             for (; o < end; o += 4) o[0] = 0u, o[1] = 0xFFFF0000u, o[2] = 0u, o[3] = 0xFFFFFFFFu;   // padding
         }
@@ -881,18 +884,15 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
     }
     slice.worker.join();
     if (slice.slots > 0 && e == cudaSuccess && dp::slice_fits(slice.slots)) {
-        uint32_t *drec = nullptr;
-        uint16_t *dfourth = nullptr;
-        int32_t *dround = nullptr, *dstart = nullptr;
-        TRY(dalloc(D, &drec, slice.rec.size()));
-        TRY(dalloc(D, &dround, slice.round_ptr.size()));
-        TRY(dalloc(D, &dfourth, slice.fourth.size()));
-        TRY(dalloc(D, &dstart, slice.start_slot.size()));
-        up(drec, slice.rec.data(), sizeof(uint32_t) * slice.rec.size());
-        up(dround, slice.round_ptr.data(), sizeof(int32_t) * slice.round_ptr.size());
-        up(dfourth, slice.fourth.data(), sizeof(uint16_t) * slice.fourth.size());
-        up(dstart, slice.start_slot.data(), sizeof(int32_t) * slice.start_slot.size());
-        D->sl = dp::SlicePlan{slice.slots, slice.threads, drec, dround, dfourth, dstart};
+        uint32_t *t = nullptr;
+        if (dalloc(D, &t, slice.all.size()) == DP_OK) {
+            up(t, slice.all.data(), sizeof(uint32_t) * slice.all.size());
+            D->sl = dp::SlicePlan{slice.slots, slice.threads, t, reinterpret_cast<const int32_t *>(t + slice.at_round),
+                                  reinterpret_cast<const uint16_t *>(t + slice.at_fourth),
+                                  reinterpret_cast<const int32_t *>(t + slice.at_start)};
+        } else {
+            ctx->err.clear();   // without memory for them the other simulations run
+        }
     }
     for (int w = 0; w < 3; w++) D->flow_grid[w] = dp::flow_grid(w, ctx->sm_count);
     if (e != cudaSuccess) { s = cuda_err(ctx, e, "upload"); free_design(D); return s; }
