@@ -623,14 +623,23 @@ struct SliceTables {
                 if (v >= 0) open[(size_t)(v & 31)].push_back(v), n_open++;
             }
         }
-        // threads per block: a round costs about 14 cycles per warp, or its latency, and a level a barrier
+        // threads per block: a round costs about 14 cycles per warp, or its latency, and a level a barrier.  Levels are
+        // padded to whole rounds: a long chain takes fewer threads, or no table, so that the padding stays bounded
+        // (64 MiB and 64 bytes a cell: 100,000 levels of one cell 51 MB with 32 threads, 205 with 128)
+        const int64_t most = ((int64_t)64 << 20) / 16 + 4 * nc;   // records
         double best = 0;
-        for (int p = 128; p <= 1024; p += 32) {
+        for (int p = 128; p > 0; p = p == 1024 ? 96 : p < 128 ? p - 32 : p + 32) {
+            if (p == 96 && threads) break;
             double cost = 0;
-            for (int l = 1; l <= L; l++)
-                cost += 60.0 + (double)((lvl[l] - lvl[l - 1] + p - 1) / p) * std::max(200.0, 14.0 * p / 32);
-            if (threads == 0 || cost < best) threads = p, best = cost;
+            int64_t rounds = 0;
+            for (int l = 1; l <= L; l++) {
+                const int64_t n = (lvl[l] - lvl[l - 1] + p - 1) / p;
+                cost += 60.0 + (double)n * std::max(200.0, 14.0 * p / 32);
+                rounds += n;
+            }
+            if (rounds * p <= most && (threads == 0 || cost < best)) threads = p, best = cost;
         }
+        if (threads == 0) return;
         std::vector<int32_t> round_ptr((size_t)L + 1, 0);
         for (int l = 1; l <= L; l++)
             round_ptr[(size_t)l] = round_ptr[(size_t)l - 1] + (lvl[l] - lvl[l - 1] + threads - 1) / threads;

@@ -1,4 +1,5 @@
-"""The tables of the sliced simulation, which a design can do without: an upload that has no memory for them goes on."""
+"""The tables of the sliced simulation, which a design can do without: an upload that has no memory for them goes on, and
+what a long narrow netlist pads them to is bounded."""
 import os
 import subprocess
 import sys
@@ -51,3 +52,27 @@ def test_no_memory_for_the_slices():
     assert len(last) == 4 and last[1:] == full[1:]
     assert int(last[0]) < int(full[0])
 
+
+@pytest.mark.parametrize("n", [40_000, 100_000])
+def test_padding_of_a_chain_is_bounded(dp, ctx, n):  # noqa: F811
+    lib = "cell BUF Z 0.7 A\ncell INV ZN 0.6 !A\nseq DFF D Q 0.8\n"
+    lines = [f"net n{i} 1.0" for i in range(n + 1)] + ["input n0"]
+    lines += [f"cell u{i} " + (f"INV A=n{i} ZN=n{i + 1}" if i % 3 else f"BUF A=n{i} Z=n{i + 1}") for i in range(n)]
+    d = dp.dp_design_load(ctx, "\n".join(lines) + "\n", lib)
+    try:
+        info = dp.dp_design_info(d)
+        assert info.n_levels == n
+        # 64 MiB and 64 bytes a cell for the tables, 384 a level for the barriers, 200 for the rest
+        assert info.device_bytes < (64 << 20) + n * (64 + 384 + 200)
+        dp.dp_set_inputs(ctx, d, *(a[:, 0].copy() for a in netgen.scenario_inputs(1, 6, 1)))
+        got = []
+        for schedule in (0, 2):
+            cfg = dp.config(schedule=schedule, sim_words=5)
+            dp.dp_propagate(ctx, d, cfg)
+            dp.dp_simulate(ctx, d, cfg)
+            got.append([np.zeros(info.n_nets, np.uint32) for _ in range(2)])
+            dp.dp_get_nets(ctx, d, toggles=got[-1][0], ones=got[-1][1])
+        for a, b in zip(*got):
+            np.testing.assert_array_equal(a, b)
+    finally:
+        dp.dp_design_free(d)
