@@ -678,6 +678,7 @@ struct SliceTables {
                 slots = 0;   // without memory for them the other simulations run
             }
         };
+        if (cp->n_cells < 4096) return run();   // sooner than a thread starts
         try {
             worker.t = std::thread(run);
         } catch (const std::system_error &) {
@@ -689,6 +690,12 @@ struct SliceTables {
 }  // namespace
 
 dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) {
+    return dpi::upload_design(ctx, cp, true, out);
+}
+
+}  // extern "C"
+
+dp_status dpi::upload_design(dp_ctx *ctx, const dp_compiled *cp, bool simulates, dp_design **out) {
     if (!ctx || !cp || !out) return set_err(ctx, DP_EINVAL, "NULL argument");
     *out = nullptr;
     DeviceGuard g(ctx->device);
@@ -726,7 +733,7 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
                 const int k = cp->op_arity[r[0] >> 24];
                 for (int j = 0; j < k; j++) {
                     const uint32_t n = j == 0 ? (r[0] & dp::kNetMask) : r[j];
-                    death[n] = std::max(death[n], l);
+                    death[n] = l;   // (levels ascend)
                 }
             }
         for (int32_t d : death) dead_ptr[(size_t)d + 1]++;
@@ -735,7 +742,7 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
         for (size_t n = 0; n < death.size(); n++) dead_net[(size_t)at[(size_t)death[n]]++] = (int32_t)n;
     }
     SliceTables slice;
-    slice.start(cp, D->ops, dead_ptr, dead_net);
+    if (simulates) slice.start(cp, D->ops, dead_ptr, dead_net);
     int32_t *dptr = nullptr, *dnet = nullptr;
     // level-aligned cell pairs (the dataflow simulation's unit of work)
     std::vector<int32_t> pair_ptr((size_t)cp->n_levels + 1, 0);
@@ -919,6 +926,8 @@ dp_status dp_design_upload(dp_ctx *ctx, const dp_compiled *cp, dp_design **out) 
     *out = D;
     return DP_OK;
 }
+
+extern "C" {
 
 dp_status dp_design_load(dp_ctx *ctx, const char *netlist, size_t netlist_len, const char *library,
                          size_t library_len, dp_design **out) {

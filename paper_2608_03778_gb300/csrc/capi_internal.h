@@ -139,6 +139,8 @@ double power_K(const dp_config &c);
 dp_status check_cfg(dp_ctx *ctx, const dp_config *c);
 // true when the stream is being captured into a CUDA graph
 bool capturing(cudaStream_t s);
+// dp_design_upload; simulates: with the tables of the sliced simulation (a server's designs do without)
+dp_status upload_design(dp_ctx *ctx, const dp_compiled *cp, bool simulates, dp_design **out);
 // notes a call on the design that is being captured (every entry point that queues work on its single-scenario state)
 inline void note_capture(dp_design *D) { D->captured = D->captured || capturing(D->ctx->stream); }
 // frees the batched buffers (the caller has synchronised)

@@ -670,7 +670,7 @@ dp_status make_slot(dp_server *srv, const dp_compiled *cp, const float *ref_sp, 
         return srv_err(srv, DP_ECUDA, std::string("stream: ") + cudaGetErrorString(e));
     }
     st = dp_create(srv->cfg.device, sl->stream, &sl->ctx);
-    if (st == DP_OK) st = dp_design_upload(sl->ctx, cp, &sl->D);
+    if (st == DP_OK) st = upload_design(sl->ctx, cp, false, &sl->D);
     if (st != DP_OK) {
         srv_err(srv, st, sl->ctx ? dp_last_error(sl->ctx) : "context");
         free_slot(sl);
