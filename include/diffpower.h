@@ -100,7 +100,9 @@ typedef struct {
                                0) in one cluster of 16 blocks, with the pairs and edge adjoints
                                spread over the blocks' shared memory; otherwise over the whole
                                grid.  The last two have no barrier between levels: each cell
-                               waits for its own inputs.  The simulation as 2;
+                               waits for its own inputs.  The simulation by slices of lanes and
+                               cycles in shared memory where the live nets fit and that is the
+                               faster one, else as 2;
                             2: one cooperative launch per pass with grid-wide level barriers;
                             1: one launch per level;
                             3: the whole grid without barriers for the forward and the reverse

@@ -123,11 +123,9 @@ int persist_grid(int which, int sm_count);   // which: 0 forward, 1 simulation, 
 bool wide_ok(int T);                         // the wide simulation handles this word count
 cudaError_t launch_sim_wide(const DevDesign &d, const OpTable &ops, int T, int grid, cudaStream_t s);
 size_t persist_bar_words(int n_levels);      // counters needed by the three passes
-// ready (may be null) is recorded on s just before the kernel: a branch forked there becomes
-// ready with it rather than ahead of it
 // the forward and the reverse pass of a mid-size design in one cluster of kClusterBlocks blocks
 // (kern_cluster.cu): every level cut into one contiguous chunk per block, each net kept in the
-// shared memory of the block that computes it, the hardware cluster barrier between levels.
+// shared memory of the block that computes it; no barrier between levels, a cell waits for its own inputs.
 constexpr int kClusterBlocks = 16;
 constexpr int kClusterMaxThreads = 512;
 struct ClusterMap {
@@ -161,6 +159,8 @@ bool block_smem_init();
 cudaError_t launch_fwd_block(const DevDesign &d, const OpTable &ops, int tr_mode, int threads, cudaStream_t s);
 cudaError_t launch_bwd_block(const DevDesign &d, const OpTable &ops, int grad_mode, int tr_mode, float K,
                              float *out_gsp, int64_t n_edges, int threads, cudaStream_t s);
+// ready (may be null) is recorded on s just before the kernel: a branch forked there becomes
+// ready with it rather than ahead of it
 cudaError_t launch_fwd_persist(const DevDesign &d, const OpTable &ops, int tr_mode, int grid, cudaStream_t s,
                                cudaEvent_t ready = nullptr);
 cudaError_t launch_sim_persist(const DevDesign &d, const OpTable &ops, int T, int grid, cudaStream_t s);
@@ -266,7 +266,6 @@ struct SizingDeltas {
 // fills dcl[n * S + s] for every net loaded by a changed cell
 void launch_sizing_deltas(const DevDesign &d, const OpTable &ops, const SizingDeltas &z, int64_t ne, int64_t S,
                           float *dcl, cudaStream_t s);
-// returns win, dpin, flag and dcl to rest after the batch
 // A request's host buffers, as the device reads and writes them (sp, tr NULL: the reference inputs; nd resized cells
 // from entry off of the batch's on; a gradient NULL: not wanted)
 struct ServeIo {
@@ -286,6 +285,7 @@ void launch_serve_out(const ServeIo *io, int64_t S, int64_t ns, int64_t nc, cons
 // scenario column of a batch: a batch of requests on the reference inputs skips the forward pass (state: BatchBufs')
 void launch_bcast_ref(const float2 *ref_pq, const float *ref_tr, float2 *pq, float *tr_in, int64_t nn, int64_t ns,
                       int64_t S, uint32_t *state, cudaStream_t s);
+// returns win, dpin, flag and dcl to rest after the batch
 void launch_sizing_clear(const DevDesign &d, const SizingDeltas &z, int64_t ne, int64_t S, float *dcl,
                          cudaStream_t s);
 // out[c][r] = in[r][c] (row-major R x C in, C x R out)
