@@ -350,7 +350,7 @@ dp_status dp_phase_times(dp_design *d, float *ms5);
  * n_scen; not in a server), or for one scenario those by scenario groups
  * (DP_BATCH_GROUP="lanes,v,blocks,threads" fixes them); a wait in the former
  * that gives up is reported as DP_ETIMEOUT by the next synchronising call.
- * Where such a launch is refused the other passes run.
+ * Where the device has no room for the grid or the clusters the other passes run.
  * Every shape gives bitwise identical results. */
 dp_status dp_set_inputs_batch(dp_design *d, const float *sp, const float *tr, int32_t n_scen, int on_device);
 
@@ -364,8 +364,9 @@ dp_status dp_batch_tuning(const dp_design *d, int32_t *shape6, float *ms2);
 /* Test hook: the batched passes without level barriers ask for the grid of
  * `sms` SMs (0: the device's own).  With more than the device has, the runtime
  * refuses their cooperative launches on the host, and the library takes the
- * other passes, as on a GPU that has no room for such a grid.  The next
- * dp_set_inputs_batch tunes again. */
+ * other passes, as on a GPU that has no room for such a grid.  Any value but 0
+ * also makes the passes by groups ask for clusters that no device has.  The
+ * next dp_set_inputs_batch tunes again. */
 dp_status dp_selftest_flow_grid(dp_design *d, int32_t sms);
 
 /* The passes that the staged batch takes in tr_mode: for the forward
@@ -374,7 +375,7 @@ dp_status dp_selftest_flow_grid(dp_design *d, int32_t sms);
  * kernel launches (the model power's two and the reverse pass's seed not
  * counted); ms2 (may be NULL) the tuner's times of both in ms, in tr_mode 0
  * (0: not timed, as where the environment or a rule decides). */
-dp_status dp_batch_passes(const dp_design *d, int32_t tr_mode, int32_t *pass6, float *ms2);
+dp_status dp_batch_passes(dp_design *d, int32_t tr_mode, int32_t *pass6, float *ms2);
 
 /* Reverse pass of the model power (Sec. III-E, Eq. 7) for every scenario,
  * scaled by weights[n_scen] (NULL: all 1): the gradient of

@@ -152,14 +152,22 @@ dp::GroupShape group_rule(const dp_design *D, int64_t S) {
     return g;
 }
 
+// whether the device has room for the clusters of 16 blocks (a partitioned GPU may not); the self-test asks for a
+// size that no device has
+bool groups_fit(dp_batch &B) {
+    if (B.groups_fit < 0) B.groups_fit = dp::group_fits(B.flow_sms > 0 ? 64 : 16) ? 1 : 0;
+    return B.groups_fit == 1;
+}
+
 // the group shape of the staged batch's pass (0 forward, 1 reverse); v = 0: level launches
-dp::GroupShape group_in_use(const dp_design *D, int tr_mode, int pass) {
-    const dp_batch &B = D->batch;
+dp::GroupShape group_in_use(dp_design *D, int tr_mode, int pass) {
+    dp_batch &B = D->batch;
     dp::GroupShape g;
     if (parse_group_env(&g) && B.S % g.v == 0) return g;
     if (B.shape_from_env) return dp::GroupShape{};
     if (B.tuned_S == B.S && !B.shapes_locked && tr_mode != 2) return pass == 0 ? B.fwd_group : B.bwd_group;
-    return group_rule(D, B.S);
+    const dp::GroupShape r = group_rule(D, B.S);
+    return r.v > 0 && groups_fit(B) ? r : dp::GroupShape{};
 }
 
 // whether a design's batch of S can take the dataflow passes
@@ -275,7 +283,7 @@ dp_status tune(dp_design *D) {
     // 90 + 99), from two on by dataflow (S = 2: 48 + 56 against 49 + 56 at 2,000 / 24, and ahead from there)
     float least[2] = {best[0], best[1]};
     const dp::GroupShape g{2, 1, 16, 512};
-    const bool groups = !B.shapes_locked && S == 1 && D->d.n_levels > 0 && W <= 6000;
+    const bool groups = !B.shapes_locked && S == 1 && D->d.n_levels > 0 && W <= 6000 && groups_fit(B);
     if (!groups && !B.shapes_locked && !B.flow_refused && flow_can(D, S))
         for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
             const int v = flow_v(S, W);
@@ -488,11 +496,12 @@ dp_status dp_selftest_flow_grid(dp_design *D, int32_t sms) {
     if (!D || sms < 0) return DP_EINVAL;
     D->batch.flow_sms = sms;
     D->batch.flow_refused = false;
+    D->batch.groups_fit = -1;
     D->batch.tuned_S = 0;
     return DP_OK;
 }
 
-dp_status dp_batch_passes(const dp_design *D, int32_t tr_mode, int32_t *pass6, float *ms2) {
+dp_status dp_batch_passes(dp_design *D, int32_t tr_mode, int32_t *pass6, float *ms2) {
     if (!D || !pass6 || tr_mode < 0 || tr_mode > 2) return DP_EINVAL;
     const dp_batch &B = D->batch;
     if (B.cap == 0) return set_err(D->ctx, DP_ESTATE, "dp_batch_passes before dp_set_inputs_batch");

@@ -37,6 +37,7 @@ struct dp_batch {
     int fwd_flow = 0, bwd_flow = 0;        // scenarios per thread of the dataflow passes, where faster than both (0: not)
     bool flow_refused = false;     // the runtime refused a dataflow pass's cooperative launch: the others run
     int flow_sms = 0;              // > 0: a self-test's SM count for its grid
+    int groups_fit = -1;           // the device has room for the groups' clusters of 16 blocks (-1: not asked yet)
     bool shape_from_env = false;   // DP_BATCH_SHAPE fixed the level launches
     int64_t tuned_S = 0;           // S the shapes were tuned for (0: not tuned)
     bool shapes_locked = false;    // keep the shapes whatever S comes (a server fixes them once)

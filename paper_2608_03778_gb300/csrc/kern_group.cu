@@ -213,7 +213,33 @@ cudaError_t launch_group(void (*kern)(KArgs...), GroupShape sh, int64_t S, cudaS
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+template <class K>
+bool fits(K kern, int blocks) {
+    if (blocks > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)kGroupThreads);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)blocks;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    return cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0;
+}
+
 }  // namespace
+
+bool group_fits(int blocks) {
+    const bool ok = fits(k_fwdb_group<1, false>, blocks) && fits(k_fwdb_group<2, false>, blocks) &&
+                    fits(k_fwdb_group<1, true>, blocks) && fits(k_fwdb_group<2, true>, blocks) &&
+                    fits(k_bwdb_group<1, false>, blocks) && fits(k_bwdb_group<2, false>, blocks) &&
+                    fits(k_bwdb_group<1, true>, blocks) && fits(k_bwdb_group<2, true>, blocks);
+    cudaGetLastError();
+    return ok;
+}
 
 cudaError_t launch_fwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
                               cudaStream_t s) {

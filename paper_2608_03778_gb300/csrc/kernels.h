@@ -228,6 +228,8 @@ inline GroupShape group_for(GroupShape g, int tr_mode) {
     }
     return g;
 }
+// whether clusters of `blocks` full blocks can run on this device, in every mode with one or two scenarios per thread
+bool group_fits(int blocks);
 cudaError_t launch_fwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,
                               cudaStream_t s);
 cudaError_t launch_bwdb_group(const DevDesign &d, const BatchBufs &b, const OpTable &ops, int tr_mode, GroupShape sh,

@@ -66,3 +66,22 @@ def test_refused_cooperative_launch(dp, ctx, library_text, monkeypatch, tr_mode)
                 np.testing.assert_array_equal(got[k], want[k], err_msg=k)
     finally:
         dp.dp_design_free(d)
+
+
+@pytest.mark.parametrize("tr_mode", [0, 2])
+@pytest.mark.parametrize("S", [1, 6])
+def test_no_room_for_the_clusters(dp, ctx, library_text, tr_mode, S):  # noqa: F811
+    """A device without room for the groups' clusters (asked for a size that none has): level launches, in the tuner for
+    one scenario, and where the lag-one mode goes by the rule; the same bits."""
+    d = dp.dp_design_load(ctx, netgen.netlist_text(SPEC), library_text)
+    cfg = dp.config(grad_mode=0, tr_mode=tr_mode)
+    sp, tr = netgen.scenario_inputs(60, 79, S)
+    try:
+        want = run_batch(dp, ctx, d, sp, tr, cfg)
+        dp.dp_selftest_flow_grid(d, 100_000)
+        got = run_batch(dp, ctx, d, sp, tr, cfg)
+        assert all(p[0] == "level" for p in dp.dp_batch_passes(d, tr_mode))
+        for k in want:
+            np.testing.assert_array_equal(got[k], want[k], err_msg=k)
+    finally:
+        dp.dp_design_free(d)
