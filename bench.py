@@ -107,9 +107,9 @@ def batched_algorithmic_bytes(nn: int, ns: int, nc: int, ne: int, S: int) -> int
 TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,lts__t_bytes.sum,... (one launch),
     # 2M-cell step, 4th step (profiles/roofline_step_k_sim_wide_traffic.md)
-    "k_sim_wide": {"bytes": 224_710_000 + 162_070_000, "l2_bytes": 7_781_440_000, "workload": "roofline",
+    "k_sim_wide": {"bytes": 224_391_680 + 162_347_776, "l2_bytes": 7_804_059_808, "workload": "roofline",
                    "files": ["kern_persist.cu", "kern_common.cuh"],
-                   "sha": "d68f35c894eb261c"},
+                   "sha": "5417b4d114f391bc"},
 }
 
 
